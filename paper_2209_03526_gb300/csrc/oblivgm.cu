@@ -20,6 +20,7 @@
 #include "ptx_async.cuh"
 #include "oblivgm.h"
 #include "runtime.h"
+#include "staged.h"
 
 namespace ogm {
 
@@ -58,27 +59,6 @@ oblivgm_status ws_alloc(oblivgm_ctx* ctx, void** p, size_t bytes, cudaStream_t s
 // (mbarriers, bulk copies and the bounded wait are in ptx_async.cuh)
 
 // ------------------------------------------------------------------ fused secEval
-
-struct GroupDesc {
-    const uint32_t* share[3];   // share set j of the group's table: [attr][stride]
-    uint32_t* out[3];           // RSS share sets of the result, n_elems each
-    uint64_t stride;
-    uint64_t n_elems;
-    uint32_t query_id, table_id, pred_begin, n_preds;
-    uint32_t vec_out;           // out pointers are 16-byte aligned
-    uint32_t tile;              // elements per work item of this group (k_filter_wp; k_filter uses the launch's)
-    uint32_t slots;             // k_filter_wp: walk threads per element, 6 (equality predicates only) or 12
-    uint32_t pad;
-};
-
-struct PredDesc {
-    uint32_t kind, n_bits, attr, step;
-    uint32_t r[3];
-    uint32_t cbeta;
-    uint32_t key_begin, n_keys;
-    // fold into the group's result: w_i = lin (a_i + b_i) + prod (a_i b_i + a_i b_{i+1} + a_{i+1} b_i)
-    uint32_t lin, prod;
-};
 
 struct FilterParams {
     AesParams aes;
@@ -623,6 +603,8 @@ struct Plan {
     std::vector<PredDesc> preds;
     std::vector<DevKey> keys;
     std::vector<uint64_t> item_start;
+    bool staged = false;   // the staged evaluation (staged.cu) instead of a fused kernel
+    Staged sg;
 };
 
 // Element tile per work item.  The items (group, tile) are taken by one persistent CTA
@@ -843,11 +825,13 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
 
 // Plan a batch for the fused kernel in the context's launch shape; a batch whose groups
 // hold at most ctx->wp_max_elems elements in all goes to the walk-parallel kernel instead,
-// in tiles of kWpElems elements.
+// in tiles of kWpElems elements, and a larger one to the staged evaluation (staged_ok) where
+// its estimate is below the fused kernel's.
 oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& tables, uint32_t n_queries,
                            const uint32_t* query_ids, const ParsedQuery* parsed, const uint32_t* n_groups,
-                           uint32_t* const* const* outs, Plan* plan) {
+                           uint32_t* const* const* outs, bool staged_ok, Plan* plan) {
     const uint32_t threads = ctx->threads, E = ctx->elems_per_thread;
+    plan->staged = false;
     plan->elems_per_thread = E;
     plan->threads = threads;
     plan->wp = false;
@@ -856,7 +840,14 @@ oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& ta
     if (s != OBLIVGM_OK) return s;
     uint64_t total = 0;
     for (const GroupDesc& g : plan->groups) total += g.n_elems;
-    if (total == 0 || total > ctx->wp_max_elems) return OBLIVGM_OK;
+    if (total == 0) return OBLIVGM_OK;
+    if (total > ctx->wp_max_elems) {
+        // large launches share tree nodes between elements where that pays; the key-staging
+        // expiry hook is about the fused kernels' waits
+        if (staged_ok && !ctx->test_expire_next)
+            plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->scratch_cap, &plan->sg);
+        return OBLIVGM_OK;
+    }
     // a forced tile (oblivgm_set_walk_parallel_tile) skips the search: step 0
     s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, ctx->wp_tile ? ctx->wp_tile : kWpElems,
                      ctx->wp_tile ? 0 : 1, true, ctx->sm_count, plan);
@@ -939,8 +930,43 @@ void apply_test_expiry(oblivgm_ctx* ctx, FilterParams* P) {
     ctx->test_expire_next = false;
 }
 
-oblivgm_status launch_plan(oblivgm_ctx* ctx, const Plan& plan, cudaStream_t st, uint32_t* error_flag) {
+// The staged evaluation of a plan: a small descriptor image and a scratch block, both stream
+// ordered.  *ran is false when the device has no room for the scratch: the fused kernel, which
+// needs next to none, runs then.
+oblivgm_status launch_staged(oblivgm_ctx* ctx, Plan& plan, cudaStream_t st, bool* ran) {
+    *ran = false;
+    unsigned char *image = nullptr, *scratch = nullptr;
+    const oblivgm_status as =
+        ws_alloc(ctx, reinterpret_cast<void**>(&image), plan.sg.image_bytes, st, "workspace allocation");
+    if (as != OBLIVGM_OK) return as;
+    ScratchGuard guard(image, st);
+    const cudaError_t ae = cudaMallocAsync(reinterpret_cast<void**>(&scratch), plan.sg.scratch_bytes, st);
+    if (ae == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        return OBLIVGM_OK;
+    }
+    if (ae != cudaSuccess) return cuda_fail(ae, "scratch allocation");
+    ScratchGuard scratch_guard(scratch, st);
+    std::vector<unsigned char> bytes;
+    staged_image(&plan.sg, plan.keys.data(), scratch, &bytes);
+    OGM_CUDA(cudaMemcpyAsync(image, bytes.data(), bytes.size(), cudaMemcpyHostToDevice, st), "descriptor upload");
+    const oblivgm_status ls = staged_launch(ctx, plan.sg, image, st);
+    if (ls != OBLIVGM_OK) return ls;
+    *ran = true;
+    scratch_guard.done();
+    OGM_CUDA(cudaFreeAsync(scratch, st), "scratch release");
+    guard.done();
+    OGM_CUDA(cudaFreeAsync(image, st), "workspace release");
+    return OBLIVGM_OK;
+}
+
+oblivgm_status launch_plan(oblivgm_ctx* ctx, Plan& plan, cudaStream_t st, uint32_t* error_flag) {
     if (plan.item_start.back() == 0) return OBLIVGM_OK;   // nothing to evaluate
+    if (plan.staged) {
+        bool ran = false;
+        const oblivgm_status s = launch_staged(ctx, plan, st, &ran);
+        if (s != OBLIVGM_OK || ran) return s;
+    }
     const WsImage im = build_ws_image(plan);
     unsigned char* ws = nullptr;
     oblivgm_status as = ws_alloc(ctx, reinterpret_cast<void**>(&ws), im.total, st, "workspace allocation");
@@ -960,9 +986,9 @@ oblivgm_status launch_plan(oblivgm_ctx* ctx, const Plan& plan, cudaStream_t st, 
 
 oblivgm_status launch_parsed(oblivgm_ctx* ctx, uint32_t n_queries, const uint32_t* query_ids,
                              const ParsedQuery* parsed, const uint32_t* n_groups, uint32_t* const* const* outs,
-                             const std::map<uint32_t, Table>& tables, cudaStream_t st) {
+                             const std::map<uint32_t, Table>& tables, cudaStream_t st, bool staged_ok) {
     Plan plan;
-    oblivgm_status s = plan_filter(ctx, tables, n_queries, query_ids, parsed, n_groups, outs, &plan);
+    oblivgm_status s = plan_filter(ctx, tables, n_queries, query_ids, parsed, n_groups, outs, staged_ok, &plan);
     if (s != OBLIVGM_OK) return s;
     return launch_plan(ctx, plan, st, ctx->d_error);
 }
@@ -1006,6 +1032,7 @@ oblivgm_status oblivgm_create(oblivgm_ctx** out, int32_t device, const oblivgm_c
     if (!ctx) return fail(OBLIVGM_ENOMEM, "host allocation");
     ctx->device = device;
     ctx->sm_count = prop.multiProcessorCount;
+    ctx->scratch_cap = prop.totalGlobalMem / 8;
     ctx->wp_max_elems = (uint64_t)ctx->sm_count * kWpDefaultElemsPerSm;
     build_aes_params(&ctx->aes);
     for (int i = 0; i < 3; i++) {
@@ -1014,6 +1041,7 @@ oblivgm_status oblivgm_create(oblivgm_ctx** out, int32_t device, const oblivgm_c
     }
     ctx->cfg = *cfg;
     oblivgm_status st = set_filter_attrs();
+    if (st == OBLIVGM_OK) st = set_staged_attrs();
     if (st == OBLIVGM_OK) st = set_onehot_attrs();
     if (st == OBLIVGM_OK) st = set_keygen_attrs();
     if (st == OBLIVGM_OK) st = set_fresh_attrs();
@@ -1297,7 +1325,7 @@ oblivgm_status oblivgm_autotune(oblivgm_ctx* ctx, uint32_t* threads, uint32_t* e
         float ms_best = 1e30f;
         for (int rep = 0; rep < 3; rep++) {
             cudaEventRecord(a, 0);
-            st = launch_parsed(ctx, 1, &qid, &pq, &ng, outs, tabs, 0);
+            st = launch_parsed(ctx, 1, &qid, &pq, &ng, outs, tabs, 0, /*staged_ok=*/false);
             cudaEventRecord(b, 0);
             if (st != OBLIVGM_OK) break;
             cudaEventSynchronize(b);
@@ -1436,7 +1464,7 @@ extern "C" oblivgm_status oblivgm_filter_and_combine_noalloc(oblivgm_ctx* ctx, u
     if (st != OBLIVGM_OK) return fail(st, err);
     uint32_t* const* outs[1] = {out};
     Plan plan;
-    st = plan_filter(ctx, ctx->tables, 1, &query_id, &parsed, &n_groups, outs, &plan);
+    st = plan_filter(ctx, ctx->tables, 1, &query_id, &parsed, &n_groups, outs, /*staged_ok=*/false, &plan);
     if (st != OBLIVGM_OK) return st;
     if (plan.item_start.back() == 0) return OBLIVGM_OK;
     const WsImage im = build_ws_image(plan);
@@ -1459,18 +1487,21 @@ extern "C" oblivgm_status oblivgm_filter_and_combine_noalloc(oblivgm_ctx* ctx, u
 
 // ====================================================================== prepared plans (CUDA-graph capture)
 //
-// A plan holds a batch's descriptors and device keys in its own device buffer, so
-// launching it is only a counter reset and one kernel launch: no host work, no
-// allocation and no pageable copies, which is what stream capture into a CUDA graph
-// needs.  Replaying the plan recomputes the same shares into the same outputs.
+// A plan holds a batch's descriptors and device keys in its own device buffer (and, for the
+// staged evaluation, its scratch), so launching it is only a counter reset and one kernel
+// launch, or the staged kernels: no host work, no allocation and no pageable copies, which
+// is what stream capture into a CUDA graph needs.  Replaying the plan recomputes the same shares into the same outputs.
 
 struct oblivgm_plan {
     oblivgm_ctx* ctx = nullptr;
     unsigned char* ws = nullptr;
     FilterParams params{};
-    uint32_t threads = 0, E = 1;
+    uint32_t threads = 0, E = 1, tile = 0;
     bool wp = false;
     uint64_t n_items = 0;
+    bool staged = false;              // the staged evaluation: ws holds its image
+    unsigned char* scratch = nullptr;
+    Staged sg;
 };
 
 extern "C" oblivgm_status oblivgm_plan_create(oblivgm_ctx* ctx, uint32_t n_queries, const uint32_t* query_ids,
@@ -1490,20 +1521,34 @@ extern "C" oblivgm_status oblivgm_plan_create(oblivgm_ctx* ctx, uint32_t n_queri
         if (st != OBLIVGM_OK) return fail(st, err);
     }
     Plan plan;
-    st = plan_filter(ctx, ctx->tables, n_queries, query_ids, parsed.data(), n_groups, outs, &plan);
+    st = plan_filter(ctx, ctx->tables, n_queries, query_ids, parsed.data(), n_groups, outs, /*staged_ok=*/true, &plan);
     if (st != OBLIVGM_OK) return st;
-    const WsImage im = build_ws_image(plan);
     auto* p = new (std::nothrow) oblivgm_plan();
     if (!p) return fail(OBLIVGM_ENOMEM, "host allocation");
+    if (plan.staged && cudaMalloc(&p->scratch, plan.sg.scratch_bytes) != cudaSuccess) {
+        cudaGetLastError();            // no room for the scratch: the fused kernel's plan instead
+        plan.staged = false;
+    }
+    WsImage im;
+    if (plan.staged) {
+        staged_image(&plan.sg, plan.keys.data(), p->scratch, &im.bytes);
+        im.total = im.bytes.size();
+    } else {
+        im = build_ws_image(plan);
+    }
     cudaError_t e = cudaMalloc(&p->ws, im.total);
     if (e == cudaSuccess) e = cudaMemcpy(p->ws, im.bytes.data(), im.total, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         if (p->ws) cudaFree(p->ws);
+        if (p->scratch) cudaFree(p->scratch);
         delete p;
         return cuda_fail(e, "plan buffer");
     }
     p->ctx = ctx;
-    p->params = filter_params(ctx, plan, im, p->ws, ctx->d_error);
+    p->staged = plan.staged;
+    if (plan.staged) p->sg = std::move(plan.sg);
+    else p->params = filter_params(ctx, plan, im, p->ws, ctx->d_error);
+    p->tile = plan.tile;
     p->n_items = plan.item_start.back();
     p->threads = plan.threads;
     p->E = plan.elems_per_thread;
@@ -1517,6 +1562,7 @@ extern "C" oblivgm_status oblivgm_plan_launch(oblivgm_plan* p, void* stream) {
     if (!p) return fail(OBLIVGM_EINVAL, "NULL plan");
     if (p->n_items == 0) return OBLIVGM_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    if (p->staged) return staged_launch(p->ctx, p->sg, p->ws, s);
     // the walk-parallel kernel leaves its counters at zero when it ends; the per-element
     // kernel's counter is cleared before each launch
     if (!p->wp) OGM_CUDA(cudaMemsetAsync(p->ws, 0, sizeof(unsigned long long), s), "plan counter reset");
@@ -1531,7 +1577,7 @@ extern "C" oblivgm_status oblivgm_plan_describe(const oblivgm_plan* p, uint32_t*
     if (!p) return fail(OBLIVGM_EINVAL, "NULL plan");
     if (walk_parallel) *walk_parallel = p->wp ? 1u : 0u;
     if (threads) *threads = p->threads;
-    if (tile) *tile = p->params.tile;
+    if (tile) *tile = p->tile;
     if (n_items) *n_items = p->n_items;
     if (grid) *grid = (uint32_t)std::min<uint64_t>(p->n_items, (uint64_t)p->ctx->sm_count);
     return OBLIVGM_OK;
@@ -1542,6 +1588,7 @@ extern "C" oblivgm_status oblivgm_plan_destroy(oblivgm_plan* p) {
     cudaSetDevice(p->ctx->device);
     cudaDeviceSynchronize();
     cudaFree(p->ws);
+    if (p->scratch) cudaFree(p->scratch);
     delete p;
     return OBLIVGM_OK;
 }

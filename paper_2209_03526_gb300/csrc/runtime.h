@@ -117,6 +117,7 @@ struct oblivgm_ctx {
     uint32_t threads = 768;          // the autotuner's pick on GB300 (256 x 4 spills)
     uint32_t elems_per_thread = 1;
     uint64_t wp_max_elems = 0;       // batches with at most this many elements in all run walk-parallel
+    size_t scratch_cap = 0;          // most scratch a staged evaluation may take
     uint32_t wp_tile = 0;            // walk-parallel elements per tile; 0 = chosen per launch
     std::atomic<uint64_t> launches{0};
     bool test_expire_next = false;      // failure-path test hook, one-shot
@@ -138,10 +139,11 @@ oblivgm_status serve_init(oblivgm_ctx* ctx);
 void serve_shutdown(oblivgm_ctx* ctx);
 bool table_in_use(oblivgm_ctx* ctx, uint32_t table_id);
 
-// plan + launch of the fused kernel over already-parsed queries (used by the serving loop)
+// plan + launch over already-parsed queries (used by the serving loop); staged_ok lets large
+// launches take the staged evaluation
 oblivgm_status launch_parsed(oblivgm_ctx* ctx, uint32_t n_queries, const uint32_t* query_ids,
                              const ParsedQuery* parsed, const uint32_t* n_groups, uint32_t* const* const* outs,
-                             const std::map<uint32_t, Table>& tables, cudaStream_t st);
+                             const std::map<uint32_t, Table>& tables, cudaStream_t st, bool staged_ok = true);
 
 double now_ms();
 oblivgm_status set_onehot_attrs();

@@ -1,0 +1,920 @@
+// staged.cu -- masked-mode secEval of a launch whose elements share tree nodes.
+//
+// In the masked mode one predicate's keys are evaluated at x^ = x + r of every element of a
+// column, so the walks of all elements run in the same few trees: elements whose x^ agree in
+// the first l bits pass through the same node of level l, and equal values are one walk.  A
+// server that has opened the column (every server learns x^ of each element, Sec. V-C) can
+// therefore visit each node once instead of once per element.  The kernels here do that:
+//
+//   1. each column the launch reads is opened once (for its first predicate; another
+//      predicate's x^ differs by a constant) and sorted, and its distinct values and every
+//      element's rank among them are written (k_sort_*, k_uniq_*).  A column whose domain is
+//      hardly larger than its table is dense instead: the distinct values are 0 .. 2^n - 1;
+//   2. per predicate, the levels are cut into stages (choose_stages).  A run is a maximal set
+//      of distinct values that agree in the bits up to a stage's last level; k_run_* list the
+//      runs and each one's parent run;
+//   3. k_stage evaluates a stage: one walk per (key, run) from the parent's seed, control bit
+//      and value sum, which a table in memory holds; k_stage_last walks the remaining levels
+//      for every distinct value and sums the halves per server (Eq. predEval);
+//   4. k_combine looks up each element's three sums, re-shares and folds them (Sec. III-B,
+//      V-D), exactly as the fused kernel does.
+//
+// For 2^20 uniform 32-bit values a key takes about 13.5 x 2^20 level steps instead of
+// 32 x 2^20; skewed columns take far fewer.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <map>
+#include <vector>
+
+#include "device_fss.cuh"
+#include "runtime.h"
+#include "staged.h"
+
+namespace ogm {
+
+namespace {
+
+constexpr int kSortThreads = 256;
+constexpr int kSortItems = 16;                               // keys per thread
+constexpr uint32_t kSortTile = kSortThreads * kSortItems;    // 4,096 keys per CTA
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr uint32_t kRunBlock = 1024;                         // distinct values per CTA of the run kernels
+constexpr int kStageThreads = 768;                           // one CTA per SM (the tables take 128 KiB)
+constexpr uint32_t kMaxRoundPreds = 64;
+
+__device__ __forceinline__ uint32_t lanemask_lt() {
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+
+// ------------------------------------------------------------------ opened columns, sorted
+//
+// Least-significant-digit radix sort, 8 bits a pass, of all the launch's sparse columns side
+// by side (grid y).  A pass is three launches: digit counts per 4,096-key tile, their sums
+// along the tiles, and the stable scatter.  It moves 24 bytes a key and pass.
+
+__global__ void __launch_bounds__(kSortThreads) k_sort_hist(const SgCol* cols, uint32_t pass) {
+    __shared__ uint32_t h[256];
+    const SgCol& C = cols[blockIdx.y];
+    if (blockIdx.x >= C.tiles || pass >= C.passes) return;
+    h[threadIdx.x] = 0;
+    __syncthreads();
+    const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
+#pragma unroll
+    for (int i = 0; i < kSortItems; i++) {
+        const uint64_t e = base + (uint32_t)i * kSortThreads + threadIdx.x;
+        if (e < C.n) {
+            uint32_t k;
+            if (pass == 0) {
+                // open x^ = <x>_1 + <x>_2 + <x>_3 + r mod 2^n
+                k = (__ldg(C.share[0] + e) + __ldg(C.share[1] + e) + __ldg(C.share[2] + e) + C.radd) & C.mask;
+                C.key[0][e] = k;
+            } else {
+                k = C.key[pass & 1][e];
+            }
+            atomicAdd(&h[(k >> (8 * pass)) & 255u], 1u);
+        }
+    }
+    __syncthreads();
+    C.hist[(uint64_t)threadIdx.x * C.tiles + blockIdx.x] = h[threadIdx.x];
+}
+
+// exclusive sum of a CTA's 256 values; *total the sum of all
+__device__ __forceinline__ uint32_t block_exclusive_256(uint32_t v, uint32_t* warp_sums, uint32_t* total) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t s = v;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, s, off);
+        if (lane >= (uint32_t)off) s += o;
+    }
+    __syncthreads();
+    if (lane == 31) warp_sums[warp] = s;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < 8; w++) {
+        const uint32_t x = warp_sums[w];
+        before += (uint32_t)w < warp ? x : 0u;
+        all += x;
+    }
+    *total = all;
+    return before + s - v;
+}
+
+// in-place exclusive sum of row[0 .. n) by one CTA of 256 threads; the sum of all goes to *total
+__device__ __forceinline__ void row_scan(uint32_t* row, uint32_t n, uint32_t* total) {
+    __shared__ uint32_t ws[8];
+    uint32_t carry = 0;
+    for (uint32_t b = 0; b < n; b += 256) {
+        const uint32_t i = b + threadIdx.x;
+        const uint32_t v = i < n ? row[i] : 0u;
+        uint32_t all;
+        const uint32_t x = block_exclusive_256(v, ws, &all);
+        if (i < n) row[i] = carry + x;
+        carry += all;
+    }
+    if (threadIdx.x == 0) *total = carry;
+}
+
+__global__ void __launch_bounds__(256) k_sort_scan(const SgCol* cols, uint32_t pass) {
+    const SgCol& C = cols[blockIdx.y];
+    if (pass >= C.passes) return;
+    row_scan(C.hist + (uint64_t)blockIdx.x * C.tiles, C.tiles, C.tot + blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const SgCol* cols, uint32_t pass) {
+    __shared__ uint32_t cnt[kSortWarps][256];
+    __shared__ uint32_t ws[8];
+    const SgCol& C = cols[blockIdx.y];
+    if (blockIdx.x >= C.tiles || pass >= C.passes) return;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int w = 0; w < kSortWarps; w++) cnt[w][threadIdx.x] = 0;
+    __syncthreads();
+    // each warp owns 512 consecutive keys; a key's rank among its warp's keys of the same digit
+    const uint32_t* src = C.key[pass & 1];
+    const uint32_t* sidx = C.idx[pass & 1];
+    const uint64_t base = (uint64_t)blockIdx.x * kSortTile + (uint64_t)warp * (32 * kSortItems) + lane;
+    uint32_t k[kSortItems], rk[kSortItems];
+#pragma unroll
+    for (int i = 0; i < kSortItems; i++) {
+        const uint64_t e = base + 32u * i;
+        const bool ok = e < C.n;
+        k[i] = ok ? src[e] : 0u;
+        const uint32_t d = ok ? (k[i] >> (8 * pass)) & 255u : 256u;
+        const uint32_t same = __match_any_sync(0xFFFFFFFFu, d);
+        const uint32_t old = ok ? cnt[warp][d] : 0u;
+        __syncwarp();
+        const uint32_t below = same & lanemask_lt();
+        rk[i] = old + __popc(below);
+        if (ok && below == 0) cnt[warp][d] = old + __popc(same);
+        __syncwarp();
+    }
+    __syncthreads();
+    // cnt[w][d] <- first output position of warp w's keys with digit d
+    uint32_t total;
+    uint32_t at = block_exclusive_256(C.tot[threadIdx.x], ws, &total) +
+                  C.hist[(uint64_t)threadIdx.x * C.tiles + blockIdx.x];
+#pragma unroll
+    for (int w = 0; w < kSortWarps; w++) {
+        const uint32_t c = cnt[w][threadIdx.x];
+        cnt[w][threadIdx.x] = at;
+        at += c;
+    }
+    __syncthreads();
+    uint32_t* dst = C.key[(pass + 1) & 1];
+    uint32_t* didx = C.idx[(pass + 1) & 1];
+#pragma unroll
+    for (int i = 0; i < kSortItems; i++) {
+        const uint64_t e = base + 32u * i;
+        if (e < C.n) {
+            const uint32_t o = cnt[warp][(k[i] >> (8 * pass)) & 255u] + rk[i];
+            dst[o] = k[i];
+            didx[o] = pass == 0 ? (uint32_t)e : sidx[e];
+        }
+    }
+}
+
+// The sorted keys' distinct values: counts per tile, their sums, then the values and every
+// element's rank.  A warp owns 512 consecutive keys of its tile.
+__device__ __forceinline__ bool starts_value(const uint32_t* key, uint64_t e, uint64_t n) {
+    return e < n && (e == 0 || key[e] != key[e - 1]);
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_uniq_count(const SgCol* cols) {
+    __shared__ uint32_t ws[kSortWarps];
+    const SgCol& C = cols[blockIdx.y];
+    if (blockIdx.x >= C.tiles || C.passes == 0) return;
+    const uint32_t* key = C.key[C.passes & 1];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t base = (uint64_t)blockIdx.x * kSortTile + (uint64_t)warp * (32 * kSortItems) + lane;
+    uint32_t c = 0;
+#pragma unroll 4
+    for (int i = 0; i < kSortItems; i++)
+        c += __popc(__ballot_sync(0xFFFFFFFFu, starts_value(key, base + 32u * i, C.n)));
+    if (lane == 0) ws[warp] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint32_t s = 0;
+        for (int w = 0; w < kSortWarps; w++) s += ws[w];
+        C.hist[blockIdx.x] = s;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_uniq_scan(const SgCol* cols) {
+    const SgCol& C = cols[blockIdx.x];
+    if (C.passes == 0) return;
+    row_scan(C.hist, C.tiles, C.m);
+}
+
+__global__ void __launch_bounds__(kSortThreads) k_uniq_emit(const SgCol* cols) {
+    __shared__ uint32_t ws[kSortWarps];
+    const SgCol& C = cols[blockIdx.y];
+    if (blockIdx.x >= C.tiles || C.passes == 0) return;
+    const uint32_t* key = C.key[C.passes & 1];
+    const uint32_t* idx = C.idx[C.passes & 1];
+    uint32_t* u = C.key[(C.passes + 1) & 1];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t base = (uint64_t)blockIdx.x * kSortTile + (uint64_t)warp * (32 * kSortItems) + lane;
+    uint32_t flags = 0, c = 0;     // bit i: this lane's key of step i starts a value
+#pragma unroll 4
+    for (int i = 0; i < kSortItems; i++) {
+        const bool f = starts_value(key, base + 32u * i, C.n);
+        flags |= (f ? 1u : 0u) << i;
+        c += __popc(__ballot_sync(0xFFFFFFFFu, f));
+    }
+    if (lane == 0) ws[warp] = c;
+    __syncthreads();
+    uint32_t at = C.hist[blockIdx.x];
+    for (uint32_t w = 0; w < warp; w++) at += ws[w];
+#pragma unroll 4
+    for (int i = 0; i < kSortItems; i++) {
+        const uint64_t e = base + 32u * i;
+        const bool f = (flags >> i) & 1u;
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, f);
+        const uint32_t r = at + __popc(b & lanemask_lt()) + (f ? 1u : 0u) - 1u;   // values started up to e, less one
+        if (e < C.n) {
+            if (f) u[r] = key[e];
+            C.rank[idx[e]] = r;
+        }
+        at += __popc(b);
+    }
+}
+
+// ------------------------------------------------------------------ runs of a predicate
+
+// values of chunk `c` (a dense column has 2^n of them)
+__device__ __forceinline__ uint32_t chunk_values(const SgPred& P, uint32_t c) {
+    const uint64_t all = P.dense ? (uint64_t)P.mask + 1u : (uint64_t)*P.m, first = (uint64_t)c * P.chunk;
+    return all <= first ? 0u : (uint32_t)min((unsigned long long)(all - first), (unsigned long long)P.chunk);
+}
+
+// Bits in which value i of the chunk agrees with the one before, from the top; -1 for the first.
+// A run of stage s starts at i where that is below lev[s].
+__device__ __forceinline__ int common_bits(const SgPred& P, const uint32_t* u, uint32_t i, uint32_t* x) {
+    *x = (u[i] + P.delta) & P.mask;
+    if (i == 0) return -1;
+    const uint32_t d = *x ^ ((u[i - 1] + P.delta) & P.mask);     // nonzero: the values are distinct
+    return __clz((int)d) - (32 - (int)P.n);
+}
+
+__global__ void __launch_bounds__(kRunBlock) k_run_count(const SgPred* preds, uint32_t chunk) {
+    __shared__ uint32_t ws[32][kSgMaxStages];
+    const SgPred& P = preds[blockIdx.y];
+    if (P.dense) return;
+    const uint32_t n = chunk_values(P, chunk);
+    if ((uint64_t)blockIdx.x * kRunBlock >= n) return;
+    const uint32_t i = blockIdx.x * kRunBlock + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x;
+    const int cb = i < n ? common_bits(P, P.u + (uint64_t)chunk * P.chunk, i, &x) : 32;
+    const uint32_t S = P.stages - 1;
+    for (uint32_t s = 0; s < S; s++) {
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, cb < (int)P.lev[s]);
+        if (lane == 0) ws[warp][s] = __popc(b);
+    }
+    __syncthreads();
+    if (threadIdx.x < S) {
+        uint32_t c = 0;
+        for (int w = 0; w < 32; w++) c += ws[w][threadIdx.x];
+        P.blk[(uint64_t)threadIdx.x * P.blocks + blockIdx.x] = c;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_run_scan(const SgPred* preds, uint32_t chunk) {
+    const SgPred& P = preds[blockIdx.y];
+    if (P.dense || blockIdx.x + 1 >= P.stages) return;
+    const uint32_t n = chunk_values(P, chunk);
+    row_scan(P.blk + (uint64_t)blockIdx.x * P.blocks, (n + kRunBlock - 1) / kRunBlock, P.cnt + blockIdx.x);
+}
+
+__global__ void __launch_bounds__(kRunBlock) k_run_emit(const SgPred* preds, uint32_t chunk) {
+    __shared__ uint32_t ws[32][kSgMaxStages];
+    const SgPred& P = preds[blockIdx.y];
+    if (P.dense) return;
+    const uint32_t n = chunk_values(P, chunk);
+    if ((uint64_t)blockIdx.x * kRunBlock >= n) return;
+    const uint32_t i = blockIdx.x * kRunBlock + threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = 0;
+    const int cb = i < n ? common_bits(P, P.u + (uint64_t)chunk * P.chunk, i, &x) : 32;
+    const uint32_t S = P.stages - 1;
+    for (uint32_t s = 0; s < S; s++) {
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, cb < (int)P.lev[s]);
+        if (lane == 0) ws[warp][s] = __popc(b);
+    }
+    __syncthreads();
+    if (threadIdx.x < S) {
+        uint32_t at = P.blk[(uint64_t)threadIdx.x * P.blocks + blockIdx.x];
+        for (int w = 0; w < 32; w++) {
+            const uint32_t c = ws[w][threadIdx.x];
+            ws[w][threadIdx.x] = at;
+            at += c;
+        }
+    }
+    __syncthreads();
+    uint32_t parent = 0;          // the run of the stage before that value i lies in
+    for (uint32_t s = 0; s < S; s++) {
+        const bool f = cb < (int)P.lev[s];
+        const uint32_t b = __ballot_sync(0xFFFFFFFFu, f);
+        const uint32_t r = ws[warp][s] + __popc(b & lanemask_lt()) + (f ? 1u : 0u) - 1u;
+        if (f) {
+            P.pre[P.pre_off[s] + r] = x >> (P.n - P.lev[s]);
+            P.par[P.pre_off[s] + r] = parent;
+        }
+        parent = r;
+    }
+    if (i < n) P.par_last[i] = parent;
+}
+
+// ------------------------------------------------------------------ the walks
+
+struct StageParams {
+    AesParams aes;
+    const uint32_t* te0;
+    const SgPred* preds;
+    const DevKey* keys;
+    uint32_t n_preds;
+    uint32_t stage;
+    uint32_t chunk;
+};
+
+// Levels a .. b - 1 of one key's walk at x (n bits), from the node's seed s, control bit t
+// and, for a DCF, value sum V; the steps are those of dpf_walk / dcf_walk.
+template <bool DCF, class Tab>
+__device__ __forceinline__ void walk_levels(const Tab& T, const AesParams& A, const DevKey* K, uint32_t x, int n, int a,
+                                            int b, uint32_t s[4], uint32_t& t, uint32_t& V) {
+    const uint32_t tl = __ldg(&K->tl), tr = __ldg(&K->tr), party = __ldg(&K->party);
+#pragma unroll 1
+    for (int i = a; i < b; i++) {
+        const uint4 cw = __ldg(reinterpret_cast<const uint4*>(K->scw[i]));
+        const uint32_t dir = (x >> (n - 1 - i)) & 1u, m = 0u - dir;
+        uint32_t o[4];
+        aes_sel(T, A.rk_st, A.d_st, m, s, o);
+        if (DCF) {
+            const uint32_t v0 = aes_sel_w0(T, A.rk_v, A.d_v, m, s);
+            const uint32_t term = (v0 ^ s[0]) + (t ? __ldg(&K->vcw[i]) : 0u);
+            V += party ? 0u - term : term;
+        }
+#pragma unroll
+        for (int w = 0; w < 4; w++) o[w] ^= s[w];
+        uint32_t tn = o[0] & 1u;
+        o[0] &= ~1u;
+        const uint32_t tm = 0u - t;
+        s[0] = o[0] ^ (cw.x & tm);
+        s[1] = o[1] ^ (cw.y & tm);
+        s[2] = o[2] ^ (cw.z & tm);
+        s[3] = o[3] ^ (cw.w & tm);
+        tn ^= t & (((dir ? tr : tl) >> i) & 1u);
+        t = tn;
+    }
+}
+
+// first run of a dense stage: the prefix of the chunk's first value
+__device__ __forceinline__ uint32_t dense_base(const SgPred& P, uint32_t chunk, uint32_t level) {
+    return level == 0 ? 0u : (uint32_t)(((uint64_t)chunk * P.chunk) >> (P.n - level));
+}
+
+__device__ __forceinline__ uint32_t stage_runs(const SgPred& P, uint32_t chunk, uint32_t s) {
+    const uint32_t n = chunk_values(P, chunk);
+    if (n == 0) return 0u;
+    if (!P.dense) return P.cnt[s];
+    return (uint32_t)(((uint64_t)chunk * P.chunk + n - 1) >> (P.n - P.lev[s])) - dense_base(P, chunk, P.lev[s]) + 1u;
+}
+
+__device__ __forceinline__ void load_state(const SgPred& P, uint32_t buf, uint32_t key, uint32_t r, bool dcf,
+                                           uint32_t s[4], uint32_t& t, uint32_t& V) {
+    const uint64_t at = (uint64_t)key * P.cap[buf] + r;
+    const uint4 q = P.st[buf][at];
+    t = q.x & 1u;
+    s[0] = q.x & ~1u; s[1] = q.y; s[2] = q.z; s[3] = q.w;
+    V = dcf ? P.v[buf][at] : 0u;
+}
+
+// work units of the launch's predicates, 32 lanes each: first[p] .. first[p + 1] - 1 belong to p
+__device__ __forceinline__ void unit_table(unsigned long long* first, uint32_t n_preds, unsigned long long mine) {
+    if (threadIdx.x < n_preds) first[threadIdx.x + 1] = mine;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        first[0] = 0;
+        for (uint32_t p = 0; p < n_preds; p++) first[p + 1] += first[p];
+    }
+    __syncthreads();
+}
+
+// One stage but the last: a warp takes 32 runs of one key.
+__global__ void __launch_bounds__(kStageThreads, 1) k_stage(const __grid_constant__ StageParams P) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ unsigned long long first[kMaxRoundPreds + 1];
+    unsigned long long units = 0;
+    if (threadIdx.x < P.n_preds) {
+        const SgPred& D = P.preds[threadIdx.x];
+        if (P.stage + 1 < D.stages)
+            units = (unsigned long long)D.n_keys * ((stage_runs(D, P.chunk, P.stage) + 31) / 32);
+    }
+    unit_table(first, P.n_preds, units);
+    const unsigned long long total = first[P.n_preds];
+    if (total == 0) return;
+    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    __syncthreads();
+    const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
+    const uint32_t lane = threadIdx.x & 31, st = P.stage;
+    const unsigned long long step = (unsigned long long)gridDim.x * (kStageThreads / 32);
+    // consecutive units go to different SMs, so a short last wave is spread evenly
+    for (unsigned long long w = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < total; w += step) {
+        uint32_t p = 0;
+        while (first[p + 1] <= w) p++;
+        const SgPred& D = P.preds[p];
+        const uint32_t runs = stage_runs(D, P.chunk, st), per_key = (runs + 31) / 32;
+        const uint32_t local = (uint32_t)(w - first[p]), key = local / per_key;
+        const uint32_t r = (local - key * per_key) * 32 + lane;
+        if (r >= runs) continue;
+        const bool dcf = D.kind == OBLIVGM_PRED_RANGE;
+        const int a = st ? D.lev[st - 1] : 0, b = D.lev[st], n = (int)D.n;
+        const DevKey* K = P.keys + D.key_begin + key;
+        uint32_t pre, par;
+        if (D.dense) {
+            pre = dense_base(D, P.chunk, (uint32_t)b) + r;
+            par = st ? (pre >> (b - a)) - dense_base(D, P.chunk, (uint32_t)a) : 0u;
+        } else {
+            pre = D.pre[D.pre_off[st] + r];
+            par = D.par[D.pre_off[st] + r];
+        }
+        uint32_t s[4], t, V = 0;
+        if (st == 0) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) s[j] = __ldg(&K->seed[j]);
+            t = __ldg(&K->party);
+        } else {
+            load_state(D, (st - 1) & 1, key, par, dcf, s, t, V);
+        }
+        const uint32_t x = pre << (n - b);      // b >= 1
+        if (dcf) walk_levels<true>(T, P.aes, K, x, n, a, b, s, t, V);
+        else walk_levels<false>(T, P.aes, K, x, n, a, b, s, t, V);
+        const uint64_t at = (uint64_t)key * D.cap[st & 1] + r;
+        D.st[st & 1][at] = make_uint4(s[0] | t, s[1], s[2], s[3]);
+        if (dcf) D.v[st & 1][at] = V;
+    }
+}
+
+// The last stage: a warp takes 32 distinct values of one output slot (a server's two key
+// halves, or one key of a raw evaluation) and walks the slot's keys one after another.
+__global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_constant__ StageParams P) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ unsigned long long first[kMaxRoundPreds + 1];
+    unsigned long long units = 0;
+    if (threadIdx.x < P.n_preds) {
+        const SgPred& D = P.preds[threadIdx.x];
+        units = (unsigned long long)D.slots * ((chunk_values(D, P.chunk) + 31) / 32);
+    }
+    unit_table(first, P.n_preds, units);
+    const unsigned long long total = first[P.n_preds];
+    if (total == 0) return;
+    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    __syncthreads();
+    const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
+    const uint32_t lane = threadIdx.x & 31;
+    const unsigned long long step = (unsigned long long)gridDim.x * (kStageThreads / 32);
+    for (unsigned long long w = (unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < total; w += step) {
+        uint32_t p = 0;
+        while (first[p + 1] <= w) p++;
+        const SgPred& D = P.preds[p];
+        const uint32_t vals = chunk_values(D, P.chunk), per_slot = (vals + 31) / 32;
+        const uint32_t local = (uint32_t)(w - first[p]), slot = local / per_slot;
+        const uint32_t i = (local - slot * per_slot) * 32 + lane;
+        if (i >= vals) continue;
+        const bool dcf = D.kind == OBLIVGM_PRED_RANGE;
+        const uint32_t S = D.stages, nk = D.n_keys / D.slots;
+        const int n = (int)D.n, a = S > 1 ? D.lev[S - 2] : 0;
+        const uint64_t gi = (uint64_t)P.chunk * D.chunk + i;
+        uint32_t x, par = 0;
+        if (D.dense) {
+            x = (uint32_t)gi;
+            if (S > 1) par = (x >> (n - a)) - dense_base(D, P.chunk, (uint32_t)a);
+        } else {
+            x = (D.u[gi] + D.delta) & D.mask;
+            if (S > 1) par = D.par_last[i];
+        }
+        uint32_t z = 0;
+#pragma unroll 1
+        for (uint32_t kk = 0; kk < nk; kk++) {
+            const uint32_t key = slot * nk + kk;
+            const DevKey* K = P.keys + D.key_begin + key;
+            const uint32_t party = __ldg(&K->party);
+            uint32_t s[4], t, V = 0;
+            if (S == 1) {
+#pragma unroll
+                for (int j = 0; j < 4; j++) s[j] = __ldg(&K->seed[j]);
+                t = party;
+            } else {
+                load_state(D, (S - 2) & 1, key, par, dcf, s, t, V);
+            }
+            if (dcf) walk_levels<true>(T, P.aes, K, x, n, a, n, s, t, V);
+            else walk_levels<false>(T, P.aes, K, x, n, a, n, s, t, V);
+            const uint32_t term = s[1] + (t ? __ldg(&K->cw_final) : 0u);   // Convert(s_n): bytes 4..7
+            z += V + (party ? 0u - term : term);
+            // RANGE: the public constant c * beta' joins party 0's half once (sub 0 of the half)
+            if (dcf && (kk & 1u) == 0 && party == 0) z += D.cbeta;
+        }
+        D.z[gi * D.z_elem + slot * D.z_slot] = z;
+    }
+}
+
+// ------------------------------------------------------------------ re-share and fold
+
+struct CombineParams {
+    uint32_t rk_prf[3][44];
+    const uint32_t* te0;
+    const SgGroup* groups;
+    const SgFold* folds;
+    uint64_t items;             // warp items of 32 elements
+    uint32_t n_groups;
+};
+
+// One thread per element of a group: for each of the round's predicates the three servers'
+// sums at the element's value (z_i), r_i = z_i + F(k_i) - F(k_{i-1}) (Sec. III-B), and the fold
+// into the group's result with its re-share (Sec. V-D).
+__global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_constant__ CombineParams P) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    __syncthreads();
+    const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
+    const uint32_t lane = threadIdx.x & 31;
+    const uint64_t step = (uint64_t)gridDim.x * (kStageThreads / 32);
+    uint32_t g = 0;
+    for (uint64_t w = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < P.items; w += step) {
+        while (g + 1 < P.n_groups && P.groups[g + 1].item_begin <= w) g++;
+        const SgGroup& G = P.groups[g];
+        const uint64_t e = (w - G.item_begin) * 32 + lane;
+        if (e >= G.n_elems) continue;
+        uint32_t acc[3] = {0, 0, 0};
+        if (!G.first) {
+#pragma unroll
+            for (int i = 0; i < 3; i++) acc[i] = G.out[i][e];
+        }
+        for (uint32_t k = 0; k < G.n_preds; k++) {
+            const SgFold& D = P.folds[G.pred_begin + k];
+            uint32_t at;
+            if (D.dense) {
+                const uint64_t row = (uint64_t)D.attr * G.stride + e;
+                at = (__ldg(G.share[0] + row) + __ldg(G.share[1] + row) + __ldg(G.share[2] + row) + D.radd) & D.mask;
+            } else {
+                at = __ldg(D.rank + e);
+            }
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(D.z) + at);
+            uint32_t z[3] = {q.x, q.y, q.z};
+            const bool fold = !(G.first && k == 0);
+            uint32_t step_ctr = D.step;
+#pragma unroll 1
+            for (int pass = 0; pass < (fold ? 2 : 1); pass++) {
+                const uint32_t ctr[4] = {(uint32_t)e, (uint32_t)(e >> 32), step_ctr | (G.table_id << 16), G.query_id};
+                uint32_t r[3] = {z[0], z[1], z[2]};
+#pragma unroll 1
+                for (int i = 0; i < 3; i++) {
+                    const uint32_t f = aes_one_w0(T, P.rk_prf[i], ctr);   // F keeps bytes 0..3
+                    r[0] += i == 0 ? f : (i == 2 ? 0u - f : 0u);
+                    r[1] += i == 1 ? f : (i == 0 ? 0u - f : 0u);
+                    r[2] += i == 2 ? f : (i == 1 ? 0u - f : 0u);
+                }
+                if (fold && pass == 0) {
+#pragma unroll
+                    for (int i = 0; i < 3; i++) {
+                        const int i1 = (i + 1) % 3;
+                        const uint32_t pr = acc[i] * r[i] + acc[i] * r[i1] + acc[i1] * r[i];
+                        z[i] = D.lin * (acc[i] + r[i]) + D.prod * pr;
+                    }
+                    step_ctr = 64u + D.step;
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 3; i++) acc[i] = r[i];
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) G.out[i][e] = acc[i];
+    }
+}
+
+// ------------------------------------------------------------------ planning
+
+// GB300 figures the plan weighs: a DPF / DCF level step of one key at the T-table lookup rate,
+// a PRF word, a launch (with its table fill) and a key of a sort pass.
+constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, kLaunch = 4.0e-6;
+constexpr double kSortKeyPass = 12e-12;
+constexpr uint64_t kMaxElems = 1ull << 28;
+constexpr uint32_t kMaxChunk = 1u << 21;      // distinct values evaluated together
+constexpr size_t kRoundBytes = 1ull << 30;    // states of the predicates evaluated together
+constexpr int kMaxDenseBits = 24;
+
+// distinct l-bit prefixes of n_vals uniform values, the most that a column can be expected to have
+double expected_nodes(double n_vals, int l) {
+    const double cells = std::ldexp(1.0, l);
+    return -cells * std::expm1(-n_vals / cells);
+}
+
+// The level boundaries: shortest path over the levels, where a stage a -> b costs one step per
+// level and node of level b, plus a state's round trip (about 15 % of a DCF step) and a launch.
+// Real columns repeat values and prefixes, and the more so the nearer the root, so deep
+// boundaries are worth a little more than uniform values would say.
+double choose_stages(double n_vals, bool dense, int n, double step_s, std::vector<uint8_t>* lev) {
+    std::vector<double> nodes(n + 1), best(n + 1, 1e300);
+    std::vector<int> from(n + 1, 0);
+    for (int l = 0; l <= n; l++)
+        nodes[l] = dense ? std::ldexp(1.0, l) : expected_nodes(n_vals, l) * (0.75 + 0.25 * l / n);
+    best[0] = 0;
+    for (int b = 1; b <= n; b++)
+        for (int a = 0; a < b; a++) {
+            const double c = best[a] + nodes[b] * step_s * ((b - a) + (b < n ? 0.15 : 0.05)) + kLaunch;
+            if (c < best[b]) { best[b] = c; from[b] = a; }
+        }
+    lev->clear();
+    for (int b = n; b > 0; b = from[b]) lev->push_back((uint8_t)b);
+    std::reverse(lev->begin(), lev->end());
+    return best[n];
+}
+
+size_t up256(size_t b) { return (b + 255) / 256 * 256; }
+
+// distinct values a predicate's column can have, and those of one chunk
+uint64_t max_values(const SgPred& p, const SgCol& c) {
+    const uint64_t domain = (uint64_t)p.mask + 1;
+    return p.dense ? domain : std::min<uint64_t>(c.n, domain);
+}
+
+// Runs a chunk can have after stage s.  A sparse chunk's values ascend in u, so in x^ = u + delta
+// they wrap once past 2^n: the prefix that holds the first value can come up again at the end.
+uint64_t max_runs(const SgPred& p, const SgCol& c, uint32_t s) {
+    return std::min<uint64_t>(std::min<uint64_t>(p.chunk, max_values(p, c)), (1ull << p.lev[s]) + (p.dense ? 0 : 1));
+}
+
+// Lays out a sparse column / a predicate from byte `at` on and returns the end; sets the
+// pointers when there is a base.
+size_t layout_col(SgCol* c, unsigned char* base, size_t at) {
+    const auto take = [&](size_t b) { unsigned char* p = base + at; at += up256(b); return reinterpret_cast<uint32_t*>(p); };
+    if (c->passes == 0) return at;
+    for (int j = 0; j < 2; j++) c->key[j] = take(c->n * 4);
+    for (int j = 0; j < 2; j++) c->idx[j] = take(c->n * 4);
+    c->rank = take(c->n * 4);
+    c->hist = take((size_t)c->tiles * 256 * 4);
+    c->tot = take(256 * 4);
+    c->m = take(4);
+    return at;
+}
+
+size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
+    const auto take = [&](size_t b) { unsigned char* q = base + at; at += up256(b); return reinterpret_cast<uint32_t*>(q); };
+    const uint64_t vals = max_values(*p, c);
+    if (p->z_elem == 4) p->z = take(vals * 16);
+    for (int b = 0; b < 2; b++) {
+        p->st[b] = reinterpret_cast<uint4*>(take((size_t)p->n_keys * p->cap[b] * 16));
+        p->v[b] = p->kind == OBLIVGM_PRED_RANGE ? take((size_t)p->n_keys * p->cap[b] * 4) : nullptr;
+    }
+    if (p->dense) return at;
+    uint64_t runs = 0;
+    for (uint32_t s = 0; s + 1 < p->stages; s++) {
+        p->pre_off[s] = runs;
+        runs += max_runs(*p, c, s);
+    }
+    p->u = c.key[(c.passes + 1) & 1];
+    p->m = c.m;
+    p->pre = take(runs * 4);
+    p->par = take(runs * 4);
+    p->par_last = take(std::min<uint64_t>(p->chunk, vals) * 4);
+    p->blk = take((size_t)p->stages * p->blocks * 4);
+    p->cnt = take((size_t)p->stages * 4);
+    return at;
+}
+
+}  // namespace
+
+bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys,
+                 size_t scratch_cap, Staged* sg) {
+    *sg = Staged{};
+    sg->n_keys = (uint32_t)n_keys;
+    // columns: a share row of the first set
+    std::map<const uint32_t*, uint32_t> col_of;
+    std::vector<double> col_steps;                      // seconds per node of one level, over its predicates' keys
+    std::vector<uint32_t> pred_col(preds.size());
+    double fused = 0, combine = 0;
+    for (const GroupDesc& G : groups) {
+        if (G.n_elems == 0) continue;
+        if (G.n_elems > kMaxElems) return false;
+        for (uint32_t k = 0; k < G.n_preds; k++) {
+            const PredDesc& D = preds[G.pred_begin + k];
+            const uint64_t row = (uint64_t)D.attr * G.stride;
+            const auto ins = col_of.emplace(G.share[0] + row, (uint32_t)sg->cols.size());
+            if (ins.second) {
+                SgCol c{};
+                for (int j = 0; j < 3; j++) c.share[j] = G.share[j] + row;
+                c.n = G.n_elems;
+                c.radd = D.r[0] + D.r[1] + D.r[2];
+                c.mask = D.n_bits >= 32 ? 0xFFFFFFFFu : ((1u << D.n_bits) - 1u);
+                c.passes = (D.n_bits + 7) / 8;
+                c.tiles = (uint32_t)((c.n + kSortTile - 1) / kSortTile);
+                sg->cols.push_back(c);
+                col_steps.push_back(0);
+            }
+            pred_col[G.pred_begin + k] = ins.first->second;
+            const double step = D.kind == OBLIVGM_PRED_EQ ? 6 * kDpfStep : 12 * kDcfStep;
+            col_steps[ins.first->second] += step;
+            fused += step * D.n_bits * (double)G.n_elems;
+            combine += (k ? 6 : 3) * kPrfWord * (double)G.n_elems;
+        }
+    }
+    if (sg->cols.empty()) return false;
+    // per column: dense when the whole domain costs no more than its sorted values
+    std::vector<std::vector<uint8_t>> lev(sg->cols.size());
+    double staged = 0;
+    size_t most_stages = 0;
+    for (size_t c = 0; c < sg->cols.size(); c++) {
+        SgCol& C = sg->cols[c];
+        const int n = __builtin_popcount(C.mask);
+        std::vector<uint8_t> ld;
+        double cd = 1e300;
+        if (n <= kMaxDenseBits) cd = choose_stages(0, true, n, col_steps[c], &ld);
+        const double sort = (double)C.n * kSortKeyPass * C.passes;
+        const double cs = choose_stages((double)C.n, false, n, col_steps[c], &lev[c]) + sort;
+        if (cd <= cs + 6 * kLaunch) {
+            C.passes = 0;
+            lev[c] = ld;
+        }
+        // the columns' launches are shared, so they are counted once below
+        staged += std::min(cd, cs) - kLaunch * (double)lev[c].size();
+        most_stages = std::max(most_stages, lev[c].size());
+        if (C.passes) {
+            sg->sort_passes = std::max(sg->sort_passes, C.passes);
+            sg->sort_tiles = std::max(sg->sort_tiles, C.tiles);
+        }
+    }
+    staged += kLaunch * (double)(most_stages + 1 + (sg->sort_passes ? 6 + 3 * sg->sort_passes : 0));
+    if (staged + combine > 0.85 * (fused + combine)) { *sg = Staged{}; return false; }
+
+    size_t col_end = 0;
+    for (SgCol& C : sg->cols) col_end = layout_col(&C, nullptr, col_end);
+    // predicates in group order, cut into rounds whose states fit kRoundBytes
+    size_t at = col_end, most = col_end;
+    StagedRound R{};
+    const auto close = [&]() {
+        if (R.n_preds) sg->rounds.push_back(R);
+        R = StagedRound{};
+        R.pred_begin = (uint32_t)sg->preds.size();
+        R.group_begin = (uint32_t)sg->groups.size();
+        at = col_end;
+    };
+    for (const GroupDesc& G : groups) {
+        if (G.n_elems == 0) continue;
+        bool open = false;          // the group has an entry in the current round
+        for (uint32_t k = 0; k < G.n_preds; k++) {
+            const PredDesc& D = preds[G.pred_begin + k];
+            const SgCol& C = sg->cols[pred_col[G.pred_begin + k]];
+            SgPred p{};
+            p.kind = D.kind; p.n = D.n_bits; p.n_keys = D.n_keys; p.key_begin = D.key_begin;
+            p.mask = C.mask;
+            p.delta = D.r[0] + D.r[1] + D.r[2] - C.radd;
+            p.cbeta = D.cbeta;
+            p.dense = C.passes == 0;
+            p.col = pred_col[G.pred_begin + k];
+            p.slots = 3;
+            p.z_elem = 4;
+            p.z_slot = 1;
+            p.stages = (uint32_t)lev[p.col].size();
+            std::copy(lev[p.col].begin(), lev[p.col].end(), p.lev);
+            const uint64_t vals = max_values(p, C);
+            p.chunk = kRunBlock;
+            while (p.chunk < vals && p.chunk < kMaxChunk) p.chunk <<= 1;
+            p.blocks = p.chunk / kRunBlock;
+            for (uint32_t s = 0; s + 1 < p.stages; s++) p.cap[s & 1] = std::max(p.cap[s & 1], (uint32_t)max_runs(p, C, s));
+            if (R.n_preds && (R.n_preds >= kMaxRoundPreds || layout_pred(&p, C, nullptr, at) - col_end > kRoundBytes)) {
+                close();
+                open = false;
+            }
+            at = layout_pred(&p, C, nullptr, at);
+            most = std::max(most, at);
+            if (!open) {
+                SgGroup g{};
+                for (int j = 0; j < 3; j++) { g.share[j] = G.share[j]; g.out[j] = G.out[j]; }
+                g.stride = G.stride; g.n_elems = G.n_elems;
+                g.item_begin = R.items;
+                g.query_id = G.query_id; g.table_id = G.table_id;
+                g.pred_begin = (uint32_t)sg->preds.size();
+                g.first = k == 0 ? 1u : 0u;
+                sg->groups.push_back(g);
+                R.items += (G.n_elems + 31) / 32;
+                R.n_groups++;
+                open = true;
+            }
+            sg->groups.back().n_preds++;
+            SgFold f{};
+            f.step = D.step; f.lin = D.lin; f.prod = D.prod; f.attr = D.attr;
+            f.radd = D.r[0] + D.r[1] + D.r[2];
+            f.mask = p.mask;
+            f.dense = p.dense;
+            sg->preds.push_back(p);
+            sg->folds.push_back(f);
+            R.n_preds++;
+            R.max_stages = std::max(R.max_stages, p.stages);
+            R.chunks = std::max<uint32_t>(R.chunks, (uint32_t)((vals + p.chunk - 1) / p.chunk));
+            if (!p.dense) {
+                R.sparse = 1;
+                R.max_blocks = std::max(R.max_blocks, p.blocks);
+            }
+        }
+    }
+    close();
+    sg->scratch_bytes = most;
+    if (sg->scratch_bytes > scratch_cap) { *sg = Staged{}; return false; }
+    sg->off_preds = up256(sg->cols.size() * sizeof(SgCol));
+    sg->off_folds = sg->off_preds + up256(sg->preds.size() * sizeof(SgPred));
+    sg->off_groups = sg->off_folds + up256(sg->folds.size() * sizeof(SgFold));
+    sg->off_keys = sg->off_groups + up256(sg->groups.size() * sizeof(SgGroup));
+    sg->image_bytes = sg->off_keys + up256(n_keys * sizeof(DevKey));
+    return true;
+}
+
+void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::vector<unsigned char>* bytes) {
+    size_t col_end = 0;
+    for (SgCol& C : sg->cols) col_end = layout_col(&C, scratch, col_end);
+    for (const StagedRound& R : sg->rounds) {
+        size_t at = col_end;
+        for (uint32_t q = R.pred_begin; q < R.pred_begin + R.n_preds; q++) {
+            SgPred& p = sg->preds[q];
+            const SgCol& C = sg->cols[p.col];
+            at = layout_pred(&p, C, scratch, at);
+            sg->folds[q].rank = C.rank;
+            sg->folds[q].z = p.z;
+        }
+    }
+    bytes->assign(sg->image_bytes, 0);
+    std::memcpy(bytes->data(), sg->cols.data(), sg->cols.size() * sizeof(SgCol));
+    std::memcpy(bytes->data() + sg->off_preds, sg->preds.data(), sg->preds.size() * sizeof(SgPred));
+    std::memcpy(bytes->data() + sg->off_folds, sg->folds.data(), sg->folds.size() * sizeof(SgFold));
+    std::memcpy(bytes->data() + sg->off_groups, sg->groups.data(), sg->groups.size() * sizeof(SgGroup));
+    std::memcpy(bytes->data() + sg->off_keys, keys, sg->n_keys * sizeof(DevKey));
+}
+
+oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s) {
+    const SgCol* cols = reinterpret_cast<const SgCol*>(image);
+    const SgPred* preds = reinterpret_cast<const SgPred*>(image + sg.off_preds);
+    const unsigned nc = (unsigned)sg.cols.size(), sms = (unsigned)ctx->sm_count;
+    uint64_t launches = 0;
+    if (sg.sort_passes) {
+        for (uint32_t p = 0; p < sg.sort_passes; p++) {
+            k_sort_hist<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
+            k_sort_scan<<<dim3(256, nc), 256, 0, s>>>(cols, p);
+            k_sort_scatter<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
+        }
+        k_uniq_count<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
+        k_uniq_scan<<<nc, 256, 0, s>>>(cols);
+        k_uniq_emit<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
+        launches += 3 * sg.sort_passes + 3;
+    }
+    StageParams W{};
+    W.aes = ctx->aes;
+    W.te0 = ctx->d_te0;
+    W.keys = reinterpret_cast<const DevKey*>(image + sg.off_keys);
+    CombineParams F{};
+    std::memcpy(F.rk_prf, ctx->rk_prf, sizeof F.rk_prf);
+    F.te0 = ctx->d_te0;
+    F.folds = reinterpret_cast<const SgFold*>(image + sg.off_folds);
+    for (const StagedRound& R : sg.rounds) {
+        W.preds = preds + R.pred_begin;
+        W.n_preds = R.n_preds;
+        for (uint32_t c = 0; c < R.chunks; c++) {
+            if (R.sparse && R.max_stages > 1) {
+                k_run_count<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
+                k_run_scan<<<dim3(R.max_stages - 1, R.n_preds), 256, 0, s>>>(W.preds, c);
+                k_run_emit<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
+                launches += 3;
+            }
+            W.chunk = c;
+            for (uint32_t st = 0; st + 1 < R.max_stages; st++) {
+                W.stage = st;
+                k_stage<<<sms, kStageThreads, kTableBytes, s>>>(W);
+                launches++;
+            }
+            k_stage_last<<<sms, kStageThreads, kTableBytes, s>>>(W);
+            launches++;
+        }
+        F.groups = reinterpret_cast<const SgGroup*>(image + sg.off_groups) + R.group_begin;
+        F.n_groups = R.n_groups;
+        F.items = R.items;
+        const uint64_t want = (R.items + kStageThreads / 32 - 1) / (kStageThreads / 32);
+        k_combine<<<(unsigned)std::min<uint64_t>(sms, want), kStageThreads, kTableBytes, s>>>(F);
+        launches++;
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "staged launch");
+    ctx->launches += launches;
+    return OBLIVGM_OK;
+}
+
+oblivgm_status set_staged_attrs() {
+    cudaError_t e = cudaFuncSetAttribute(k_stage, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stage_last, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_combine, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+    return e == cudaSuccess ? OBLIVGM_OK : cuda_fail(e, "staged kernel attributes");
+}
+
+}  // namespace ogm
