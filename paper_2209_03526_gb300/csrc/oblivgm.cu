@@ -288,24 +288,33 @@ struct RawParams {
     uint32_t all_pairs;
 };
 
+// One CTA per SM (the tables take 128 KiB) strides over the (key, point) items.
+constexpr int kRawThreads = 768;
+
 template <uint32_t KIND>
-__global__ void __launch_bounds__(256) k_eval_raw(const __grid_constant__ RawParams P) {
+__global__ void __launch_bounds__(kRawThreads) k_eval_raw(const __grid_constant__ RawParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
     fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P.n_points) return;
-    const uint32_t key = P.all_pairs ? blockIdx.y : P.key_of_point[i];
-    uint64_t o = i;
-    if (P.all_pairs) o = (uint64_t)key * P.n_points + i;
-    if (key >= P.n_keys) { P.out[o] = 0u; return; }
-    const DevKey& K = P.keys[key];
-    const uint32_t mask = K.n >= 32 ? 0xFFFFFFFFu : ((1u << K.n) - 1u);
-    uint32_t x[1] = {P.points[i] & mask}, y[1];
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
-    if (KIND == OBLIVGM_KEY_DPF) dpf_walk<1>(T, P.aes, K, x, y);
-    else dcf_walk<1>(T, P.aes, K, x, y);
-    P.out[o] = y[0];
+    const uint64_t items = P.all_pairs ? (uint64_t)P.n_keys * P.n_points : P.n_points;
+    for (uint64_t o = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; o < items; o += (uint64_t)gridDim.x * blockDim.x) {
+        uint64_t i = o;
+        uint32_t key;
+        if (P.all_pairs) {
+            key = (uint32_t)(o / P.n_points);
+            i = o - key * P.n_points;
+        } else {
+            key = P.key_of_point[i];
+        }
+        if (key >= P.n_keys) { P.out[o] = 0u; continue; }
+        const DevKey& K = P.keys[key];
+        const uint32_t mask = K.n >= 32 ? 0xFFFFFFFFu : ((1u << K.n) - 1u);
+        uint32_t x[1] = {P.points[i] & mask}, y[1];
+        if (KIND == OBLIVGM_KEY_DPF) dpf_walk<1>(T, P.aes, K, x, y);
+        else dcf_walk<1>(T, P.aes, K, x, y);
+        P.out[o] = y[0];
+    }
 }
 
 }  // namespace ogm
@@ -1213,6 +1222,29 @@ static oblivgm_status eval_batch(oblivgm_ctx* ctx, uint32_t kind, const uint8_t*
             if (!repack_key(keys + (size_t)k * klen, klen, kind, n, &dk[k], &err)) return fail(OBLIVGM_EINVAL, err);
         OGM_CUDA(cudaMemcpyAsync(d_keys, dk.data(), dk.size() * sizeof(DevKey), cudaMemcpyHostToDevice, s), "key upload");
     }
+    // all keys at all points: the walks share tree nodes (staged.cu) where that pays and there
+    // is room for it
+    Staged sg;
+    if (all && staged_plan_raw(kind, (uint32_t)n, n_keys, points, n_points, ctx->scratch_cap, &sg)) {
+        unsigned char* scratch = nullptr;
+        const size_t img = (sg.image_bytes + 255) / 256 * 256;
+        const cudaError_t ae = cudaMallocAsync(reinterpret_cast<void**>(&scratch), img + sg.scratch_bytes, s);
+        if (ae == cudaSuccess) {
+            ScratchGuard scratch_guard(scratch, s);
+            std::vector<unsigned char> bytes;
+            staged_image(&sg, nullptr, scratch + img, &bytes);
+            OGM_CUDA(cudaMemcpyAsync(scratch, bytes.data(), bytes.size(), cudaMemcpyHostToDevice, s), "descriptor upload");
+            st = staged_launch_raw(ctx, sg, scratch, d_keys, out, s);
+            if (st != OBLIVGM_OK) return st;
+            scratch_guard.done();
+            OGM_CUDA(cudaFreeAsync(scratch, s), "scratch release");
+            guard.done();
+            OGM_CUDA(cudaFreeAsync(d_keys, s), "key buffer release");
+            return OBLIVGM_OK;
+        }
+        if (ae != cudaErrorMemoryAllocation) return cuda_fail(ae, "scratch allocation");
+        cudaGetLastError();
+    }
     RawParams P{};
     P.aes = ctx->aes;
     P.te0 = ctx->d_te0;
@@ -1223,11 +1255,13 @@ static oblivgm_status eval_batch(oblivgm_ctx* ctx, uint32_t kind, const uint8_t*
     P.n_points = n_points;
     P.n_keys = n_keys;
     P.all_pairs = all ? 1u : 0u;
-    const uint64_t blocks = (n_points + 255) / 256;
-    if (blocks > 0x7FFFFFFFull) return fail(OBLIVGM_EINVAL, "too many points");
-    dim3 grid((unsigned)blocks, all ? n_keys : 1);
-    if (kind == OBLIVGM_KEY_DPF) k_eval_raw<OBLIVGM_KEY_DPF><<<grid, 256, kTableBytes, s>>>(P);
-    else k_eval_raw<OBLIVGM_KEY_DCF><<<grid, 256, kTableBytes, s>>>(P);
+    if ((n_points + 255) / 256 > 0x7FFFFFFFull) return fail(OBLIVGM_EINVAL, "too many points");
+    // as many threads per SM as give every item one, in one CTA of at most 768
+    const uint64_t sms = (uint64_t)ctx->sm_count, per_sm = (need + sms - 1) / sms;
+    const unsigned threads = (unsigned)std::min<uint64_t>(kRawThreads, std::max<uint64_t>(128, (per_sm + 31) / 32 * 32));
+    const unsigned grid = (unsigned)std::min<uint64_t>((need + threads - 1) / threads, sms);
+    if (kind == OBLIVGM_KEY_DPF) k_eval_raw<OBLIVGM_KEY_DPF><<<grid, threads, kTableBytes, s>>>(P);
+    else k_eval_raw<OBLIVGM_KEY_DCF><<<grid, threads, kTableBytes, s>>>(P);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "k_eval_raw launch");
     ctx->launches++;

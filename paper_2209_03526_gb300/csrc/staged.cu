@@ -71,7 +71,9 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const SgCol* cols, u
             uint32_t k;
             if (pass == 0) {
                 // open x^ = <x>_1 + <x>_2 + <x>_3 + r mod 2^n
-                k = (__ldg(C.share[0] + e) + __ldg(C.share[1] + e) + __ldg(C.share[2] + e) + C.radd) & C.mask;
+                k = __ldg(C.share[0] + e);
+                if (C.share[1]) k += __ldg(C.share[1] + e) + __ldg(C.share[2] + e) + C.radd;
+                k &= C.mask;
                 C.key[0][e] = k;
             } else {
                 k = C.key[pass & 1][e];
@@ -597,6 +599,26 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
     }
 }
 
+// ------------------------------------------------------------------ raw evaluation
+
+// out[k * n_points + i] = z of key k at point i's value; grid y strides over the keys
+struct GatherParams {
+    const SgCol* col;
+    const uint32_t* z;
+    uint32_t* out;
+    uint64_t n_points, vals;
+    uint32_t n_keys;
+};
+
+__global__ void __launch_bounds__(256) k_gather_raw(const __grid_constant__ GatherParams P) {
+    const SgCol& C = *P.col;
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < P.n_points; i += (uint64_t)gridDim.x * 256) {
+        const uint32_t at = C.passes ? __ldg(C.rank + i) : __ldg(C.share[0] + i) & C.mask;
+        for (uint32_t k = blockIdx.y; k < P.n_keys; k += gridDim.y)
+            P.out[k * P.n_points + i] = __ldg(P.z + k * P.vals + at);
+    }
+}
+
 // ------------------------------------------------------------------ planning
 
 // GB300 figures the plan weighs: a DPF / DCF level step of one key at the T-table lookup rate,
@@ -666,7 +688,7 @@ size_t layout_col(SgCol* c, unsigned char* base, size_t at) {
 size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
     const auto take = [&](size_t b) { unsigned char* q = base + at; at += up256(b); return reinterpret_cast<uint32_t*>(q); };
     const uint64_t vals = max_values(*p, c);
-    if (p->z_elem == 4) p->z = take(vals * 16);
+    p->z = take(p->z_elem == 4 ? vals * 16 : vals * 4 * p->n_keys);
     for (int b = 0; b < 2; b++) {
         p->st[b] = reinterpret_cast<uint4*>(take((size_t)p->n_keys * p->cap[b] * 16));
         p->v[b] = p->kind == OBLIVGM_PRED_RANGE ? take((size_t)p->n_keys * p->cap[b] * 4) : nullptr;
@@ -842,6 +864,7 @@ void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::v
             SgPred& p = sg->preds[q];
             const SgCol& C = sg->cols[p.col];
             at = layout_pred(&p, C, scratch, at);
+            if (sg->raw) continue;
             sg->folds[q].rank = C.rank;
             sg->folds[q].z = p.z;
         }
@@ -851,61 +874,163 @@ void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::v
     std::memcpy(bytes->data() + sg->off_preds, sg->preds.data(), sg->preds.size() * sizeof(SgPred));
     std::memcpy(bytes->data() + sg->off_folds, sg->folds.data(), sg->folds.size() * sizeof(SgFold));
     std::memcpy(bytes->data() + sg->off_groups, sg->groups.data(), sg->groups.size() * sizeof(SgGroup));
-    std::memcpy(bytes->data() + sg->off_keys, keys, sg->n_keys * sizeof(DevKey));
+    if (keys) std::memcpy(bytes->data() + sg->off_keys, keys, sg->n_keys * sizeof(DevKey));
 }
 
-oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s) {
-    const SgCol* cols = reinterpret_cast<const SgCol*>(image);
-    const SgPred* preds = reinterpret_cast<const SgPred*>(image + sg.off_preds);
-    const unsigned nc = (unsigned)sg.cols.size(), sms = (unsigned)ctx->sm_count;
-    uint64_t launches = 0;
-    if (sg.sort_passes) {
-        for (uint32_t p = 0; p < sg.sort_passes; p++) {
-            k_sort_hist<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
-            k_sort_scan<<<dim3(256, nc), 256, 0, s>>>(cols, p);
-            k_sort_scatter<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
-        }
-        k_uniq_count<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
-        k_uniq_scan<<<nc, 256, 0, s>>>(cols);
-        k_uniq_emit<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
-        launches += 3 * sg.sort_passes + 3;
+namespace {
+
+uint64_t launch_sort(const Staged& sg, const SgCol* cols, cudaStream_t s) {
+    if (!sg.sort_passes) return 0;
+    const unsigned nc = (unsigned)sg.cols.size();
+    for (uint32_t p = 0; p < sg.sort_passes; p++) {
+        k_sort_hist<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
+        k_sort_scan<<<dim3(256, nc), 256, 0, s>>>(cols, p);
+        k_sort_scatter<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
     }
+    k_uniq_count<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
+    k_uniq_scan<<<nc, 256, 0, s>>>(cols);
+    k_uniq_emit<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
+    return 3 * sg.sort_passes + 3;
+}
+
+// the sums of a round's predicates at every distinct value
+uint64_t launch_round(const oblivgm_ctx* ctx, const StagedRound& R, const SgPred* preds, const DevKey* keys,
+                      cudaStream_t s) {
     StageParams W{};
     W.aes = ctx->aes;
     W.te0 = ctx->d_te0;
-    W.keys = reinterpret_cast<const DevKey*>(image + sg.off_keys);
+    W.keys = keys;
+    W.preds = preds + R.pred_begin;
+    W.n_preds = R.n_preds;
+    const unsigned sms = (unsigned)ctx->sm_count;
+    for (uint32_t c = 0; c < R.chunks; c++) {
+        if (R.sparse && R.max_stages > 1) {
+            k_run_count<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
+            k_run_scan<<<dim3(R.max_stages - 1, R.n_preds), 256, 0, s>>>(W.preds, c);
+            k_run_emit<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
+        }
+        W.chunk = c;
+        for (uint32_t st = 0; st + 1 < R.max_stages; st++) {
+            W.stage = st;
+            k_stage<<<sms, kStageThreads, kTableBytes, s>>>(W);
+        }
+        k_stage_last<<<sms, kStageThreads, kTableBytes, s>>>(W);
+    }
+    return R.chunks * (R.max_stages + (R.sparse && R.max_stages > 1 ? 3ull : 0ull));
+}
+
+}  // namespace
+
+oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s) {
+    uint64_t launches = launch_sort(sg, reinterpret_cast<const SgCol*>(image), s);
     CombineParams F{};
     std::memcpy(F.rk_prf, ctx->rk_prf, sizeof F.rk_prf);
     F.te0 = ctx->d_te0;
     F.folds = reinterpret_cast<const SgFold*>(image + sg.off_folds);
     for (const StagedRound& R : sg.rounds) {
-        W.preds = preds + R.pred_begin;
-        W.n_preds = R.n_preds;
-        for (uint32_t c = 0; c < R.chunks; c++) {
-            if (R.sparse && R.max_stages > 1) {
-                k_run_count<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
-                k_run_scan<<<dim3(R.max_stages - 1, R.n_preds), 256, 0, s>>>(W.preds, c);
-                k_run_emit<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
-                launches += 3;
-            }
-            W.chunk = c;
-            for (uint32_t st = 0; st + 1 < R.max_stages; st++) {
-                W.stage = st;
-                k_stage<<<sms, kStageThreads, kTableBytes, s>>>(W);
-                launches++;
-            }
-            k_stage_last<<<sms, kStageThreads, kTableBytes, s>>>(W);
-            launches++;
-        }
+        launches += launch_round(ctx, R, reinterpret_cast<const SgPred*>(image + sg.off_preds),
+                                 reinterpret_cast<const DevKey*>(image + sg.off_keys), s);
         F.groups = reinterpret_cast<const SgGroup*>(image + sg.off_groups) + R.group_begin;
         F.n_groups = R.n_groups;
         F.items = R.items;
         const uint64_t want = (R.items + kStageThreads / 32 - 1) / (kStageThreads / 32);
-        k_combine<<<(unsigned)std::min<uint64_t>(sms, want), kStageThreads, kTableBytes, s>>>(F);
+        k_combine<<<(unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, want), kStageThreads, kTableBytes, s>>>(F);
         launches++;
     }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "staged launch");
+    ctx->launches += launches;
+    return OBLIVGM_OK;
+}
+
+bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint32_t* points, uint64_t n_points,
+                     size_t scratch_cap, Staged* sg) {
+    *sg = Staged{};
+    if (n_points > kMaxElems) return false;
+    SgCol C{};
+    C.share[0] = points;
+    C.n = n_points;
+    C.mask = n_bits >= 32 ? 0xFFFFFFFFu : ((1u << n_bits) - 1u);
+    C.passes = (n_bits + 7) / 8;
+    C.tiles = (uint32_t)((n_points + kSortTile - 1) / kSortTile);
+    const bool dcf = kind == OBLIVGM_KEY_DCF;
+    // at most 64 keys a round; a round's launches are its own, the sort is shared
+    const double rounds = (n_keys + 63) / 64, step = n_keys / rounds * (dcf ? kDcfStep : kDpfStep);
+    std::vector<uint8_t> lev, ld;
+    double cs = rounds * choose_stages((double)C.n, false, (int)n_bits, step, &lev) +
+                (double)C.n * kSortKeyPass * C.passes + kLaunch * (3 + 3 * rounds + 3 * C.passes);
+    if ((int)n_bits <= kMaxDenseBits) {
+        const double cd = rounds * choose_stages(0, true, (int)n_bits, step, &ld);
+        if (cd <= cs) {
+            cs = cd;
+            C.passes = 0;
+            lev = ld;
+        }
+    }
+    if (cs + rounds * kLaunch > 0.85 * (rounds * step * n_bits * (double)n_points + kLaunch)) return false;
+    sg->raw = true;
+    const size_t col_end = layout_col(&C, nullptr, 0);
+    sg->sort_passes = C.passes;
+    sg->sort_tiles = C.passes ? C.tiles : 0;
+    sg->cols.push_back(C);
+    // one predicate per 64 keys at most and per round, fewer where their states would not fit
+    SgPred p{};
+    p.kind = dcf ? OBLIVGM_PRED_RANGE : OBLIVGM_PRED_EQ;
+    p.n = n_bits;
+    p.mask = C.mask;
+    p.dense = C.passes == 0;
+    p.stages = (uint32_t)lev.size();
+    std::copy(lev.begin(), lev.end(), p.lev);
+    const uint64_t vals = max_values(p, C);
+    p.z_elem = 1;
+    p.z_slot = vals;
+    p.chunk = kRunBlock;
+    while (p.chunk < vals && p.chunk < kMaxChunk) p.chunk <<= 1;
+    p.blocks = p.chunk / kRunBlock;
+    for (uint32_t s = 0; s + 1 < p.stages; s++) p.cap[s & 1] = std::max(p.cap[s & 1], (uint32_t)max_runs(p, C, s));
+    p.n_keys = std::min<uint32_t>(n_keys, 64);
+    while (p.n_keys > 1 && layout_pred(&p, C, nullptr, col_end) - col_end > kRoundBytes) p.n_keys = (p.n_keys + 1) / 2;
+    sg->scratch_bytes = layout_pred(&p, C, nullptr, col_end);
+    if (sg->scratch_bytes > scratch_cap) { *sg = Staged{}; return false; }
+    const uint32_t per = p.n_keys;
+    for (uint32_t k = 0; k < n_keys; k += per) {
+        p.key_begin = k;
+        p.n_keys = p.slots = std::min(per, n_keys - k);
+        StagedRound R{};
+        R.pred_begin = (uint32_t)sg->preds.size();
+        R.n_preds = 1;
+        R.max_stages = p.stages;
+        R.chunks = (uint32_t)((vals + p.chunk - 1) / p.chunk);
+        R.sparse = !p.dense;
+        R.max_blocks = p.blocks;
+        sg->preds.push_back(p);
+        sg->rounds.push_back(R);
+    }
+    sg->off_preds = up256(sizeof(SgCol));
+    sg->off_folds = sg->off_groups = sg->off_keys = sg->off_preds + up256(sg->preds.size() * sizeof(SgPred));
+    sg->image_bytes = sg->off_keys;
+    return true;
+}
+
+oblivgm_status staged_launch_raw(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, const DevKey* keys,
+                                 uint32_t* out, cudaStream_t s) {
+    uint64_t launches = launch_sort(sg, reinterpret_cast<const SgCol*>(image), s);
+    GatherParams G{};
+    G.col = reinterpret_cast<const SgCol*>(image);
+    G.n_points = sg.cols[0].n;
+    for (const StagedRound& R : sg.rounds) {
+        const SgPred& p = sg.preds[R.pred_begin];
+        launches += launch_round(ctx, R, reinterpret_cast<const SgPred*>(image + sg.off_preds), keys, s);
+        G.z = p.z;
+        G.vals = p.z_slot;
+        G.n_keys = p.n_keys;
+        G.out = out + (uint64_t)p.key_begin * G.n_points;
+        const unsigned gx = (unsigned)std::min<uint64_t>((G.n_points + 255) / 256, 8ull * ctx->sm_count);
+        k_gather_raw<<<dim3(gx, std::min<uint32_t>(p.n_keys, 8)), 256, 0, s>>>(G);
+        launches++;
+    }
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_fail(e, "staged evaluation launch");
     ctx->launches += launches;
     return OBLIVGM_OK;
 }

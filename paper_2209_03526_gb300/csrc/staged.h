@@ -40,7 +40,7 @@ constexpr int kSgMaxStages = 33;
 
 // One opened column of the launch (an attribute of a table, all its elements).
 struct SgCol {
-    const uint32_t* share[3];   // the column's three share rows
+    const uint32_t* share[3];   // the column's three share rows (points of a raw evaluation: one row, twice NULL)
     uint64_t n;                 // elements
     uint32_t radd;              // <r>_1 + <r>_2 + <r>_3 of the first predicate on it
     uint32_t mask;              // 2^n_bits - 1
@@ -116,6 +116,7 @@ struct Staged {
     std::vector<SgGroup> groups;
     std::vector<StagedRound> rounds;
     uint32_t n_keys = 0, sort_tiles = 0, sort_passes = 0;
+    bool raw = false;           // a raw evaluation: no combine, its keys are elsewhere on the device
     size_t off_preds = 0, off_folds = 0, off_groups = 0, off_keys = 0, image_bytes = 0;
     size_t scratch_bytes = 0;
 };
@@ -131,6 +132,13 @@ void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::v
 // Launches it on an image in device memory: no host work beyond the launches, no allocation,
 // capturable.
 oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s);
+
+// Raw evaluation of n_keys keys of one kind at the same n_points points (OBLIVGM_ALL_PAIRS):
+// plan (false: does not pay) and launch; out[k * n_points + i] = Eval(key k, points[i]).
+bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint32_t* points, uint64_t n_points,
+                     size_t scratch_cap, Staged* out);
+oblivgm_status staged_launch_raw(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, const DevKey* keys,
+                                 uint32_t* out, cudaStream_t s);
 
 oblivgm_status set_staged_attrs();
 

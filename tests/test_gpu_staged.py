@@ -137,3 +137,41 @@ def test_two_streams_at_once(ctx):
     torch.cuda.synchronize()
     for q in range(2):
         assert all(torch.equal(a, b) for a, b in zip(got[q][0], want[q][0]))
+
+
+@pytest.mark.parametrize("dcf,keys,points,bits", [(False, 3, 200001, 32), (True, 70, 40001, 32), (True, 5, 50000, 9),
+                                                  (False, 65, 100000, 17), (True, 2, 1, 32), (False, 129, 7, 4)])
+def test_raw_evaluation_of_all_pairs(ctx, dcf, keys, points, bits):
+    """Many keys at the same points: staged (sorted and dense points, more keys than a round
+    takes) and, for the few points of the last two, the per-item kernel; keys read from the
+    device and from the host; point bits above n are ignored."""
+    g = np.random.default_rng(points)
+    pairs = (keys + 1) // 2
+    kind = P.KEY_DCF if dcf else P.KEY_DPF
+    L = 28 + (24 if dcf else 20) * bits
+    pts = g.integers(0, 1 << 32, points, dtype=np.uint64).astype(np.uint32)
+    alpha = torch.from_numpy(g.integers(0, 1 << bits, pairs, dtype=np.uint64).astype(np.uint32).view(np.int32)).cuda()
+    alpha[0] = int(pts[0].astype(np.uint64) & ((1 << bits) - 1)) - (1 << 32 if pts[0] >> 31 and bits == 32 else 0)
+    beta = torch.arange(1, pairs + 1, dtype=torch.int32, device="cuda")
+    wire = torch.zeros(2 * pairs * L, dtype=torch.uint8, device="cuda")
+    ctx.keygen_device(kind, bits, alpha, beta, bytes(range(16)), wire)
+    d_pts = torch.from_numpy(pts.view(np.int32)).cuda()
+    out = torch.full((keys * points,), -1, dtype=torch.int32, device="cuda")
+    ctx.eval_device_keys(kind, bits, wire, keys, d_pts, out, all_pairs=True)
+    host = torch.full_like(out, -1)
+    raw = bytes(wire.cpu().numpy().tobytes())[:keys * L]
+    (ctx.eval_dcf_batch if dcf else ctx.eval_dpf_batch)(raw, keys, d_pts, host, all_pairs=True)
+    torch.cuda.synchronize()
+    ctx.sync()
+    assert torch.equal(out, host)
+    got = from_dev(out).reshape(keys, points)
+    sample = np.unique(np.concatenate([[0, points - 1], g.integers(0, points, 32)]))
+    x = pts[sample] & np.uint32((1 << bits) - 1)
+    for k in {0, 1, keys // 2, keys - 1}:
+        want = oracle.eval_many(raw[k * L:(k + 1) * L], x, oracle.KIND_DCF if dcf else oracle.KIND_DPF)
+        assert np.array_equal(got[k, sample], want), k
+    # a pair's two keys add up to beta [x == alpha] or beta [x < alpha] on every point
+    full = pts.astype(np.uint64) & ((1 << bits) - 1)
+    a0 = int(from_dev(alpha)[0])
+    if keys >= 2:
+        assert np.array_equal(got[0] + got[1], ((full < a0) if dcf else (full == a0)).astype(np.uint32))
