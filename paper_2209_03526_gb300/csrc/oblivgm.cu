@@ -854,7 +854,8 @@ oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& ta
         // large launches share tree nodes between elements where that pays; the key-staging
         // expiry hook is about the fused kernels' waits
         if (staged_ok && !ctx->test_expire_next)
-            plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->scratch_cap, &plan->sg);
+            plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap,
+                                       &plan->sg);
         return OBLIVGM_OK;
     }
     // a forced tile (oblivgm_set_walk_parallel_tile) skips the search: step 0
@@ -949,7 +950,8 @@ oblivgm_status launch_staged(oblivgm_ctx* ctx, Plan& plan, cudaStream_t st, bool
         ws_alloc(ctx, reinterpret_cast<void**>(&image), plan.sg.image_bytes, st, "workspace allocation");
     if (as != OBLIVGM_OK) return as;
     ScratchGuard guard(image, st);
-    const cudaError_t ae = cudaMallocAsync(reinterpret_cast<void**>(&scratch), plan.sg.scratch_bytes, st);
+    const cudaError_t ae =
+        cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), plan.sg.scratch_bytes, ctx->scratch_pool, st);
     if (ae == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         return OBLIVGM_OK;
@@ -1077,6 +1079,15 @@ oblivgm_status oblivgm_create(oblivgm_ctx** out, int32_t device, const oblivgm_c
         uint64_t keep = UINT64_MAX;
         if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
+    if (e == cudaSuccess) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        e = cudaMemPoolCreate(&ctx->scratch_pool, &props);
+        uint64_t keep = kScratchKeep;
+        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(ctx->scratch_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
     if (e != cudaSuccess) {
         st = cuda_fail(e, "context set-up");
         oblivgm_destroy(ctx);
@@ -1098,6 +1109,7 @@ oblivgm_status oblivgm_destroy(oblivgm_ctx* ctx) {
     if (ctx->d_te0) cudaFree(ctx->d_te0);
     if (ctx->d_te4) cudaFree(ctx->d_te4);
     if (ctx->d_error) cudaFree(ctx->d_error);
+    if (ctx->scratch_pool) cudaMemPoolDestroy(ctx->scratch_pool);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     delete ctx;
     return OBLIVGM_OK;
@@ -1228,7 +1240,8 @@ static oblivgm_status eval_batch(oblivgm_ctx* ctx, uint32_t kind, const uint8_t*
     if (all && staged_plan_raw(kind, (uint32_t)n, n_keys, points, n_points, ctx->scratch_cap, &sg)) {
         unsigned char* scratch = nullptr;
         const size_t img = (sg.image_bytes + 255) / 256 * 256;
-        const cudaError_t ae = cudaMallocAsync(reinterpret_cast<void**>(&scratch), img + sg.scratch_bytes, s);
+        const cudaError_t ae =
+            cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), img + sg.scratch_bytes, ctx->scratch_pool, s);
         if (ae == cudaSuccess) {
             ScratchGuard scratch_guard(scratch, s);
             std::vector<unsigned char> bytes;

@@ -44,6 +44,8 @@ struct ScratchGuard {
     ScratchGuard& operator=(const ScratchGuard&) = delete;
 };
 
+constexpr uint64_t kScratchKeep = 4ull << 30;
+
 struct Table {
     uint32_t* dev = nullptr;   // [share set j][attr][stride] uint32
     uint64_t n_elems = 0;
@@ -118,6 +120,7 @@ struct oblivgm_ctx {
     uint32_t elems_per_thread = 1;
     uint64_t wp_max_elems = 0;       // batches with at most this many elements in all run walk-parallel
     size_t scratch_cap = 0;          // most scratch a staged evaluation may take
+    cudaMemPool_t scratch_pool = nullptr;   // its stream-ordered scratch; keeps kScratchKeep bytes between calls
     uint32_t wp_tile = 0;            // walk-parallel elements per tile; 0 = chosen per launch
     std::atomic<uint64_t> launches{0};
     bool test_expire_next = false;      // failure-path test hook, one-shot

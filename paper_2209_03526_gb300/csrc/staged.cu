@@ -38,9 +38,10 @@ namespace ogm {
 namespace {
 
 constexpr int kSortThreads = 256;
-constexpr int kSortItems = 16;                               // keys per thread
-constexpr uint32_t kSortTile = kSortThreads * kSortItems;    // 4,096 keys per CTA
 constexpr int kSortWarps = kSortThreads / 32;
+// Keys per thread of a sort tile: 16 (4,096 keys per CTA) where that gives every SM a few CTAs,
+// else 4, which shortens the chain of a CTA that has an SM to itself.
+constexpr int kSortItemsLarge = 16, kSortItemsSmall = 4;
 constexpr uint32_t kRunBlock = 1024;                         // distinct values per CTA of the run kernels
 constexpr int kStageThreads = 768;                           // one CTA per SM (the tables take 128 KiB)
 constexpr uint32_t kMaxRoundPreds = 64;
@@ -54,18 +55,19 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
 // ------------------------------------------------------------------ opened columns, sorted
 //
 // Least-significant-digit radix sort, 8 bits a pass, of all the launch's sparse columns side
-// by side (grid y).  A pass is three launches: digit counts per 4,096-key tile, their sums
-// along the tiles, and the stable scatter.  It moves 24 bytes a key and pass.
+// by side (grid y).  A pass is three launches: digit counts per tile, their sums along the
+// tiles, and the stable scatter.  It moves 20 bytes a key and pass.
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const SgCol* cols, uint32_t pass) {
     __shared__ uint32_t h[256];
     const SgCol& C = cols[blockIdx.y];
     if (blockIdx.x >= C.tiles || pass >= C.passes) return;
     h[threadIdx.x] = 0;
     __syncthreads();
-    const uint64_t base = (uint64_t)blockIdx.x * kSortTile;
+    const uint64_t base = (uint64_t)blockIdx.x * (kSortThreads * ITEMS);
 #pragma unroll
-    for (int i = 0; i < kSortItems; i++) {
+    for (int i = 0; i < ITEMS; i++) {
         const uint64_t e = base + (uint32_t)i * kSortThreads + threadIdx.x;
         if (e < C.n) {
             uint32_t k;
@@ -129,26 +131,50 @@ __global__ void __launch_bounds__(256) k_sort_scan(const SgCol* cols, uint32_t p
     row_scan(C.hist + (uint64_t)blockIdx.x * C.tiles, C.tiles, C.tot + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const SgCol* cols, uint32_t pass) {
+// Lanes of the warp whose 9-bit value equals this lane's, by a ballot per bit: a match
+// instruction takes time per distinct value, which are many here.
+__device__ __forceinline__ uint32_t same_digit(uint32_t d) {
+    uint32_t m = 0xFFFFFFFFu;
+#pragma unroll
+    for (int b = 0; b < 9; b++) {
+        const uint32_t v = __ballot_sync(0xFFFFFFFFu, (d >> b) & 1u);
+        m &= (d >> b) & 1u ? v : ~v;
+    }
+    return m;
+}
+
+// The stable scatter.  Each warp ranks its keys among its own of the same digit; the tile's
+// keys then go through shared memory in digit order, so that a digit's keys leave as one
+// consecutive run of stores (16 of them in the mean at 4,096 keys and 256 digits): storing
+// each key straight from its thread took 416 us a pass on 2 x 10M keys (one sector per word).
+template <int ITEMS>
+__global__ void __launch_bounds__(kSortThreads, 3) k_sort_scatter(const SgCol* cols, uint32_t pass) {
+    constexpr uint32_t kTile = kSortThreads * ITEMS;
     __shared__ uint32_t cnt[kSortWarps][256];
+    __shared__ uint32_t skey[kTile], sidx[kTile];
+    __shared__ uint32_t base_of[256];      // output position of a digit's first key, less its place in the tile
     __shared__ uint32_t ws[8];
     const SgCol& C = cols[blockIdx.y];
     if (blockIdx.x >= C.tiles || pass >= C.passes) return;
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, shift = 8 * pass;
     for (int w = 0; w < kSortWarps; w++) cnt[w][threadIdx.x] = 0;
     __syncthreads();
-    // each warp owns 512 consecutive keys; a key's rank among its warp's keys of the same digit
     const uint32_t* src = C.key[pass & 1];
-    const uint32_t* sidx = C.idx[pass & 1];
-    const uint64_t base = (uint64_t)blockIdx.x * kSortTile + (uint64_t)warp * (32 * kSortItems) + lane;
-    uint32_t k[kSortItems], rk[kSortItems];
+    const uint32_t* isrc = C.idx[pass & 1];
+    const uint64_t tile0 = (uint64_t)blockIdx.x * kTile;
+    const uint64_t base = tile0 + warp * (32 * ITEMS) + lane;     // a warp owns 32 ITEMS consecutive keys
+    uint32_t k[ITEMS], rk[ITEMS];
 #pragma unroll
-    for (int i = 0; i < kSortItems; i++) {
+    for (int i = 0; i < ITEMS; i++) {
         const uint64_t e = base + 32u * i;
         const bool ok = e < C.n;
         k[i] = ok ? src[e] : 0u;
-        const uint32_t d = ok ? (k[i] >> (8 * pass)) & 255u : 256u;
-        const uint32_t same = __match_any_sync(0xFFFFFFFFu, d);
+    }
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+        const bool ok = base + 32u * i < C.n;
+        const uint32_t d = ok ? (k[i] >> shift) & 255u : 256u;
+        const uint32_t same = same_digit(d);
         const uint32_t old = ok ? cnt[warp][d] : 0u;
         __syncwarp();
         const uint32_t below = same & lanemask_lt();
@@ -157,10 +183,15 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const SgCol* cols
         __syncwarp();
     }
     __syncthreads();
-    // cnt[w][d] <- first output position of warp w's keys with digit d
-    uint32_t total;
-    uint32_t at = block_exclusive_256(C.tot[threadIdx.x], ws, &total) +
-                  C.hist[(uint64_t)threadIdx.x * C.tiles + blockIdx.x];
+    // thread d: the place of digit d's first key in the tile, and of each warp's first one
+    uint32_t mine = 0, total;
+#pragma unroll
+    for (int w = 0; w < kSortWarps; w++) mine += cnt[w][threadIdx.x];
+    uint32_t at = block_exclusive_256(mine, ws, &total);
+    const uint32_t tile_keys = total;
+    const uint32_t out = block_exclusive_256(C.tot[threadIdx.x], ws, &total) +
+                         C.hist[(uint64_t)threadIdx.x * C.tiles + blockIdx.x];
+    base_of[threadIdx.x] = out - at;
 #pragma unroll
     for (int w = 0; w < kSortWarps; w++) {
         const uint32_t c = cnt[w][threadIdx.x];
@@ -168,35 +199,46 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_scatter(const SgCol* cols
         at += c;
     }
     __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+        const uint64_t e = base + 32u * i;
+        if (e < C.n) {
+            const uint32_t o = cnt[warp][(k[i] >> shift) & 255u] + rk[i];
+            skey[o] = k[i];
+            sidx[o] = pass == 0 ? (uint32_t)e : isrc[e];
+        }
+    }
+    __syncthreads();
     uint32_t* dst = C.key[(pass + 1) & 1];
     uint32_t* didx = C.idx[(pass + 1) & 1];
 #pragma unroll
-    for (int i = 0; i < kSortItems; i++) {
-        const uint64_t e = base + 32u * i;
-        if (e < C.n) {
-            const uint32_t o = cnt[warp][(k[i] >> (8 * pass)) & 255u] + rk[i];
-            dst[o] = k[i];
-            didx[o] = pass == 0 ? (uint32_t)e : sidx[e];
+    for (int i = 0; i < ITEMS; i++) {
+        const uint32_t o = i * kSortThreads + threadIdx.x;
+        if (o < tile_keys) {
+            const uint32_t key = skey[o], to = base_of[(key >> shift) & 255u] + o;
+            dst[to] = key;
+            didx[to] = sidx[o];
         }
     }
 }
 
 // The sorted keys' distinct values: counts per tile, their sums, then the values and every
-// element's rank.  A warp owns 512 consecutive keys of its tile.
+// element's rank.  A warp owns 32 ITEMS consecutive keys of its tile.
 __device__ __forceinline__ bool starts_value(const uint32_t* key, uint64_t e, uint64_t n) {
     return e < n && (e == 0 || key[e] != key[e - 1]);
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_uniq_count(const SgCol* cols) {
     __shared__ uint32_t ws[kSortWarps];
     const SgCol& C = cols[blockIdx.y];
     if (blockIdx.x >= C.tiles || C.passes == 0) return;
     const uint32_t* key = C.key[C.passes & 1];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t base = (uint64_t)blockIdx.x * kSortTile + (uint64_t)warp * (32 * kSortItems) + lane;
+    const uint64_t base = (uint64_t)blockIdx.x * (kSortThreads * ITEMS) + warp * (32 * ITEMS) + lane;
     uint32_t c = 0;
 #pragma unroll 4
-    for (int i = 0; i < kSortItems; i++)
+    for (int i = 0; i < ITEMS; i++)
         c += __popc(__ballot_sync(0xFFFFFFFFu, starts_value(key, base + 32u * i, C.n)));
     if (lane == 0) ws[warp] = c;
     __syncthreads();
@@ -213,6 +255,7 @@ __global__ void __launch_bounds__(256) k_uniq_scan(const SgCol* cols) {
     row_scan(C.hist, C.tiles, C.m);
 }
 
+template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_uniq_emit(const SgCol* cols) {
     __shared__ uint32_t ws[kSortWarps];
     const SgCol& C = cols[blockIdx.y];
@@ -221,10 +264,10 @@ __global__ void __launch_bounds__(kSortThreads) k_uniq_emit(const SgCol* cols) {
     const uint32_t* idx = C.idx[C.passes & 1];
     uint32_t* u = C.key[(C.passes + 1) & 1];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t base = (uint64_t)blockIdx.x * kSortTile + (uint64_t)warp * (32 * kSortItems) + lane;
+    const uint64_t base = (uint64_t)blockIdx.x * (kSortThreads * ITEMS) + warp * (32 * ITEMS) + lane;
     uint32_t flags = 0, c = 0;     // bit i: this lane's key of step i starts a value
 #pragma unroll 4
-    for (int i = 0; i < kSortItems; i++) {
+    for (int i = 0; i < ITEMS; i++) {
         const bool f = starts_value(key, base + 32u * i, C.n);
         flags |= (f ? 1u : 0u) << i;
         c += __popc(__ballot_sync(0xFFFFFFFFu, f));
@@ -234,7 +277,7 @@ __global__ void __launch_bounds__(kSortThreads) k_uniq_emit(const SgCol* cols) {
     uint32_t at = C.hist[blockIdx.x];
     for (uint32_t w = 0; w < warp; w++) at += ws[w];
 #pragma unroll 4
-    for (int i = 0; i < kSortItems; i++) {
+    for (int i = 0; i < ITEMS; i++) {
         const uint64_t e = base + 32u * i;
         const bool f = (flags >> i) & 1u;
         const uint32_t b = __ballot_sync(0xFFFFFFFFu, f);
@@ -531,71 +574,127 @@ struct CombineParams {
     const uint32_t* te0;
     const SgGroup* groups;
     const SgFold* folds;
-    uint64_t items;             // warp items of 32 elements
+    uint64_t items;             // tiles of blockDim.x * per_thread elements
     uint32_t n_groups;
+    uint32_t per_thread;        // elements per thread of a tile
 };
 
-// One thread per element of a group: for each of the round's predicates the three servers'
-// sums at the element's value (z_i), r_i = z_i + F(k_i) - F(k_{i-1}) (Sec. III-B), and the fold
-// into the group's result with its re-share (Sec. V-D).
+// Dynamic shared memory: the tables, then a tile's counter prefixes, (predicate, pass, PRF key,
+// 256 elements) each 5 words.
+constexpr int kPrefixWords = 5;
+constexpr uint32_t kMaxTileSteps = 64;      // predicates of a group entry x elements per thread
+static_assert(kMaxTileSteps >= kMaxRoundPreds, "a round's predicates may all be of one group");
+constexpr int kMaxPrefixes = (int)kMaxTileSteps * 6 * (kStageThreads / 256);
+constexpr int kCombineSmem = kTableBytes + kMaxPrefixes * kPrefixWords * 4;
+
+// index of element e's value in a predicate's sums
+__device__ __forceinline__ uint32_t value_index(const SgGroup& G, const SgFold& D, uint64_t e) {
+    if (!D.dense) return __ldg(D.rank + e);
+    const uint64_t row = (uint64_t)D.attr * G.stride + e;
+    return (__ldg(G.share[0] + row) + __ldg(G.share[1] + row) + __ldg(G.share[2] + row) + D.radd) & D.mask;
+}
+
+// One thread per element of a tile: for each of the round's predicates the three servers' sums
+// at the element's value (z_i), r_i = z_i + F(k_i) - F(k_{i-1}) (Sec. III-B), and the fold into the
+// group's result with its re-share (Sec. V-D).  The PRF words bound it: 3 per predicate and 3
+// per fold, from the shared-memory tables.  Two things keep that pipe busy:
+//   * the counters' low byte runs over 256 consecutive elements, so a tile first computes what
+//     those share (ctr_prefix) and an element's word takes 121 lookups instead of 148;
+//   * the two dependent reads of the sums (rank, then a random 16 bytes) are issued one step
+//     ahead, the step after a tile's last predicate being the next tile's first.
 __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_constant__ CombineParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    uint4* pre_c = reinterpret_cast<uint4*>(smem + kTableBytes);
+    uint32_t* pre_n = reinterpret_cast<uint32_t*>(pre_c + kMaxPrefixes);
     fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
-    const uint32_t lane = threadIdx.x & 31;
-    const uint64_t step = (uint64_t)gridDim.x * (kStageThreads / 32);
+    const uint32_t tile = blockDim.x * P.per_thread, subs = tile >> 8;   // 256-element parts of a tile
     uint32_t g = 0;
-    for (uint64_t w = (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; w < P.items; w += step) {
-        while (g + 1 < P.n_groups && P.groups[g + 1].item_begin <= w) g++;
+    while (g + 1 < P.n_groups && P.groups[g + 1].item_begin <= blockIdx.x) g++;
+    uint4 zq = make_uint4(0, 0, 0, 0);
+    {
         const SgGroup& G = P.groups[g];
-        const uint64_t e = (w - G.item_begin) * 32 + lane;
-        if (e >= G.n_elems) continue;
-        uint32_t acc[3] = {0, 0, 0};
-        if (!G.first) {
-#pragma unroll
-            for (int i = 0; i < 3; i++) acc[i] = G.out[i][e];
+        const uint64_t e = (blockIdx.x - G.item_begin) * tile + threadIdx.x;
+        const SgFold& D = P.folds[G.pred_begin];
+        if (e < G.n_elems) zq = __ldg(reinterpret_cast<const uint4*>(D.z) + value_index(G, D, e));
+    }
+    for (uint64_t w = blockIdx.x; w < P.items;) {
+        const SgGroup& G = P.groups[g];
+        const uint64_t e0 = (w - G.item_begin) * tile;
+        for (uint32_t q = threadIdx.x; q < G.n_preds * 6 * subs; q += blockDim.x) {
+            // prefix q = ((predicate * subs + 256 elements) * 2 + pass) * 3 + key
+            const uint32_t key = q % 3, pass = q / 3 % 2, k = q / 6 / subs;
+            const uint64_t b = e0 + 256u * (q / 6 % subs);
+            const uint32_t in[4] = {(uint32_t)b, (uint32_t)(b >> 32),
+                                    (P.folds[G.pred_begin + k].step + 64u * pass) | (G.table_id << 16), G.query_id};
+            const CtrPrefix c = ctr_prefix(T, P.rk_prf[key], in);
+            pre_c[q] = c.c;
+            pre_n[q] = c.n0;
         }
-        for (uint32_t k = 0; k < G.n_preds; k++) {
-            const SgFold& D = P.folds[G.pred_begin + k];
-            uint32_t at;
-            if (D.dense) {
-                const uint64_t row = (uint64_t)D.attr * G.stride + e;
-                at = (__ldg(G.share[0] + row) + __ldg(G.share[1] + row) + __ldg(G.share[2] + row) + D.radd) & D.mask;
-            } else {
-                at = __ldg(D.rank + e);
-            }
-            const uint4 q = __ldg(reinterpret_cast<const uint4*>(D.z) + at);
-            uint32_t z[3] = {q.x, q.y, q.z};
-            const bool fold = !(G.first && k == 0);
-            uint32_t step_ctr = D.step;
-#pragma unroll 1
-            for (int pass = 0; pass < (fold ? 2 : 1); pass++) {
-                const uint32_t ctr[4] = {(uint32_t)e, (uint32_t)(e >> 32), step_ctr | (G.table_id << 16), G.query_id};
-                uint32_t r[3] = {z[0], z[1], z[2]};
-#pragma unroll 1
-                for (int i = 0; i < 3; i++) {
-                    const uint32_t f = aes_one_w0(T, P.rk_prf[i], ctr);   // F keeps bytes 0..3
-                    r[0] += i == 0 ? f : (i == 2 ? 0u - f : 0u);
-                    r[1] += i == 1 ? f : (i == 0 ? 0u - f : 0u);
-                    r[2] += i == 2 ? f : (i == 1 ? 0u - f : 0u);
-                }
-                if (fold && pass == 0) {
+        __syncthreads();
+        // the tile after this one
+        const uint64_t w2 = w + gridDim.x;
+        uint32_t g2 = g;
+        while (g2 + 1 < P.n_groups && P.groups[g2 + 1].item_begin <= w2) g2++;
+        for (uint32_t at_tile = threadIdx.x; at_tile < tile; at_tile += blockDim.x) {
+            const uint64_t e = e0 + at_tile;
+            const uint32_t sub = at_tile >> 8;
+            const bool mine = e < G.n_elems, tile_end = at_tile + blockDim.x >= tile;
+            uint32_t acc[3] = {0, 0, 0};
+            if (mine && !G.first) {
 #pragma unroll
+                for (int i = 0; i < 3; i++) acc[i] = G.out[i][e];
+            }
+            for (uint32_t k = 0; k < G.n_preds; k++) {
+                const SgFold& D = P.folds[G.pred_begin + k];
+                uint32_t z[3] = {zq.x, zq.y, zq.z};
+                // the next step's sums: its index now, the sums themselves after a PRF word
+                const bool last = k + 1 == G.n_preds, leave = last && tile_end;
+                const SgGroup& G2 = leave ? P.groups[g2] : G;
+                const SgFold& D2 = P.folds[G2.pred_begin + (last ? 0u : k + 1)];
+                const uint64_t e2 = leave ? (w2 - G2.item_begin) * tile + threadIdx.x : last ? e + blockDim.x : e;
+                const bool more = (!leave || w2 < P.items) && e2 < G2.n_elems;
+                const uint32_t at2 = more ? value_index(G2, D2, e2) : 0u;
+                if (!mine) {
+                    if (more) zq = __ldg(reinterpret_cast<const uint4*>(D2.z) + at2);
+                    continue;
+                }
+                const bool fold = !(G.first && k == 0);
+#pragma unroll 1
+                for (int pass = 0; pass < (fold ? 2 : 1); pass++) {
+                    uint32_t r[3] = {z[0], z[1], z[2]};
+#pragma unroll 1
                     for (int i = 0; i < 3; i++) {
-                        const int i1 = (i + 1) % 3;
-                        const uint32_t pr = acc[i] * r[i] + acc[i] * r[i1] + acc[i1] * r[i];
-                        z[i] = D.lin * (acc[i] + r[i]) + D.prod * pr;
+                        const uint32_t at_pre = ((k * subs + sub) * 2 + pass) * 3 + i;
+                        const CtrPrefix c{pre_n[at_pre], pre_c[at_pre]};
+                        const uint32_t f = ctr_w0(T, P.rk_prf[i], c, (uint32_t)e);   // F keeps bytes 0..3
+                        if (pass == 0 && i == 0 && more) zq = __ldg(reinterpret_cast<const uint4*>(D2.z) + at2);
+                        r[0] += i == 0 ? f : (i == 2 ? 0u - f : 0u);
+                        r[1] += i == 1 ? f : (i == 0 ? 0u - f : 0u);
+                        r[2] += i == 2 ? f : (i == 1 ? 0u - f : 0u);
                     }
-                    step_ctr = 64u + D.step;
-                } else {
+                    if (fold && pass == 0) {
 #pragma unroll
-                    for (int i = 0; i < 3; i++) acc[i] = r[i];
+                        for (int i = 0; i < 3; i++) {
+                            const int i1 = (i + 1) % 3;
+                            const uint32_t pr = acc[i] * r[i] + acc[i] * r[i1] + acc[i1] * r[i];
+                            z[i] = D.lin * (acc[i] + r[i]) + D.prod * pr;
+                        }
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 3; i++) acc[i] = r[i];
+                    }
                 }
             }
-        }
+            if (mine) {
 #pragma unroll
-        for (int i = 0; i < 3; i++) G.out[i][e] = acc[i];
+                for (int i = 0; i < 3; i++) G.out[i][e] = acc[i];
+            }
+        }
+        __syncthreads();
+        w = w2;
+        g = g2;
     }
 }
 
@@ -626,8 +725,8 @@ __global__ void __launch_bounds__(256) k_gather_raw(const __grid_constant__ Gath
 constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, kLaunch = 4.0e-6;
 constexpr double kSortKeyPass = 12e-12;
 constexpr uint64_t kMaxElems = 1ull << 28;
-constexpr uint32_t kMaxChunk = 1u << 21;      // distinct values evaluated together
-constexpr size_t kRoundBytes = 1ull << 30;    // states of the predicates evaluated together
+constexpr uint32_t kMaxChunk = 1u << 22;      // distinct values evaluated together
+constexpr size_t kRoundBytes = 5ull << 29;    // states of the predicates evaluated together (2.5 GiB)
 constexpr int kMaxDenseBits = 24;
 
 // distinct l-bit prefixes of n_vals uniform values, the most that a column can be expected to have
@@ -671,6 +770,19 @@ uint64_t max_runs(const SgPred& p, const SgCol& c, uint32_t s) {
     return std::min<uint64_t>(std::min<uint64_t>(p.chunk, max_values(p, c)), (1ull << p.lev[s]) + (p.dense ? 0 : 1));
 }
 
+// Sort tiles: large ones once the sparse columns fill the SMs' tiles several times over.
+void choose_tiles(Staged* sg) {
+    uint64_t keys = 0;
+    for (const SgCol& C : sg->cols) keys += C.passes ? C.n : 0;
+    const uint32_t large = kSortThreads * kSortItemsLarge, small = kSortThreads * kSortItemsSmall;
+    sg->sort_large = keys >= 512ull * large;
+    sg->sort_tiles = 0;
+    for (SgCol& C : sg->cols) {
+        C.tiles = (uint32_t)((C.n + (sg->sort_large ? large : small) - 1) / (sg->sort_large ? large : small));
+        if (C.passes) sg->sort_tiles = std::max(sg->sort_tiles, C.tiles);
+    }
+}
+
 // Lays out a sparse column / a predicate from byte `at` on and returns the end; sets the
 // pointers when there is a base.
 size_t layout_col(SgCol* c, unsigned char* base, size_t at) {
@@ -711,7 +823,7 @@ size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
 
 }  // namespace
 
-bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys,
+bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
                  size_t scratch_cap, Staged* sg) {
     *sg = Staged{};
     sg->n_keys = (uint32_t)n_keys;
@@ -734,7 +846,6 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
                 c.radd = D.r[0] + D.r[1] + D.r[2];
                 c.mask = D.n_bits >= 32 ? 0xFFFFFFFFu : ((1u << D.n_bits) - 1u);
                 c.passes = (D.n_bits + 7) / 8;
-                c.tiles = (uint32_t)((c.n + kSortTile - 1) / kSortTile);
                 sg->cols.push_back(c);
                 col_steps.push_back(0);
             }
@@ -765,16 +876,20 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         // the columns' launches are shared, so they are counted once below
         staged += std::min(cd, cs) - kLaunch * (double)lev[c].size();
         most_stages = std::max(most_stages, lev[c].size());
-        if (C.passes) {
-            sg->sort_passes = std::max(sg->sort_passes, C.passes);
-            sg->sort_tiles = std::max(sg->sort_tiles, C.tiles);
-        }
+        sg->sort_passes = std::max(sg->sort_passes, C.passes);
     }
     staged += kLaunch * (double)(most_stages + 1 + (sg->sort_passes ? 6 + 3 * sg->sort_passes : 0));
     if (staged + combine > 0.85 * (fused + combine)) { *sg = Staged{}; return false; }
 
+    choose_tiles(sg);
     size_t col_end = 0;
     for (SgCol& C : sg->cols) col_end = layout_col(&C, nullptr, col_end);
+    // elements per tile of the combine: narrower where that spreads a small launch over more SMs
+    uint64_t elems = 0;
+    for (const GroupDesc& G : groups) elems += G.n_elems;
+    sg->combine_threads = elems >= (uint64_t)kStageThreads * sm_count ? kStageThreads
+                          : elems >= 512ull * sm_count               ? 512
+                                                                     : 256;
     // predicates in group order, cut into rounds whose states fit kRoundBytes
     size_t at = col_end, most = col_end;
     StagedRound R{};
@@ -818,12 +933,10 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
                 SgGroup g{};
                 for (int j = 0; j < 3; j++) { g.share[j] = G.share[j]; g.out[j] = G.out[j]; }
                 g.stride = G.stride; g.n_elems = G.n_elems;
-                g.item_begin = R.items;
                 g.query_id = G.query_id; g.table_id = G.table_id;
                 g.pred_begin = (uint32_t)sg->preds.size();
                 g.first = k == 0 ? 1u : 0u;
                 sg->groups.push_back(g);
-                R.items += (G.n_elems + 31) / 32;
                 R.n_groups++;
                 open = true;
             }
@@ -845,6 +958,18 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         }
     }
     close();
+    // several elements per thread, so that a tile's barriers are rare, while every SM gets a few tiles
+    uint32_t most_preds = 1;
+    for (const SgGroup& g : sg->groups) most_preds = std::max(most_preds, g.n_preds);
+    const uint64_t spread = elems / (6ull * kStageThreads * sm_count);
+    sg->combine_per_thread = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({8, spread, kMaxTileSteps / most_preds}));
+    for (StagedRound& r : sg->rounds) {
+        const uint64_t tile = (uint64_t)sg->combine_threads * sg->combine_per_thread;
+        for (uint32_t g = r.group_begin; g < r.group_begin + r.n_groups; g++) {
+            sg->groups[g].item_begin = r.items;
+            r.items += (sg->groups[g].n_elems + tile - 1) / tile;
+        }
+    }
     sg->scratch_bytes = most;
     if (sg->scratch_bytes > scratch_cap) { *sg = Staged{}; return false; }
     sg->off_preds = up256(sg->cols.size() * sizeof(SgCol));
@@ -879,17 +1004,24 @@ void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::v
 
 namespace {
 
+template <int ITEMS>
+void launch_sort_tiles(const Staged& sg, const SgCol* cols, cudaStream_t s) {
+    const unsigned nc = (unsigned)sg.cols.size();
+    const dim3 grid(sg.sort_tiles, nc);
+    for (uint32_t p = 0; p < sg.sort_passes; p++) {
+        k_sort_hist<ITEMS><<<grid, kSortThreads, 0, s>>>(cols, p);
+        k_sort_scan<<<dim3(256, nc), 256, 0, s>>>(cols, p);
+        k_sort_scatter<ITEMS><<<grid, kSortThreads, 0, s>>>(cols, p);
+    }
+    k_uniq_count<ITEMS><<<grid, kSortThreads, 0, s>>>(cols);
+    k_uniq_scan<<<nc, 256, 0, s>>>(cols);
+    k_uniq_emit<ITEMS><<<grid, kSortThreads, 0, s>>>(cols);
+}
+
 uint64_t launch_sort(const Staged& sg, const SgCol* cols, cudaStream_t s) {
     if (!sg.sort_passes) return 0;
-    const unsigned nc = (unsigned)sg.cols.size();
-    for (uint32_t p = 0; p < sg.sort_passes; p++) {
-        k_sort_hist<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
-        k_sort_scan<<<dim3(256, nc), 256, 0, s>>>(cols, p);
-        k_sort_scatter<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols, p);
-    }
-    k_uniq_count<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
-    k_uniq_scan<<<nc, 256, 0, s>>>(cols);
-    k_uniq_emit<<<dim3(sg.sort_tiles, nc), kSortThreads, 0, s>>>(cols);
+    if (sg.sort_large) launch_sort_tiles<kSortItemsLarge>(sg, cols, s);
+    else launch_sort_tiles<kSortItemsSmall>(sg, cols, s);
     return 3 * sg.sort_passes + 3;
 }
 
@@ -927,14 +1059,14 @@ oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned 
     std::memcpy(F.rk_prf, ctx->rk_prf, sizeof F.rk_prf);
     F.te0 = ctx->d_te0;
     F.folds = reinterpret_cast<const SgFold*>(image + sg.off_folds);
+    F.per_thread = sg.combine_per_thread;
     for (const StagedRound& R : sg.rounds) {
         launches += launch_round(ctx, R, reinterpret_cast<const SgPred*>(image + sg.off_preds),
                                  reinterpret_cast<const DevKey*>(image + sg.off_keys), s);
         F.groups = reinterpret_cast<const SgGroup*>(image + sg.off_groups) + R.group_begin;
         F.n_groups = R.n_groups;
         F.items = R.items;
-        const uint64_t want = (R.items + kStageThreads / 32 - 1) / (kStageThreads / 32);
-        k_combine<<<(unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, want), kStageThreads, kTableBytes, s>>>(F);
+        k_combine<<<(unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, R.items), sg.combine_threads, kCombineSmem, s>>>(F);
         launches++;
     }
     const cudaError_t e = cudaGetLastError();
@@ -952,7 +1084,6 @@ bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint
     C.n = n_points;
     C.mask = n_bits >= 32 ? 0xFFFFFFFFu : ((1u << n_bits) - 1u);
     C.passes = (n_bits + 7) / 8;
-    C.tiles = (uint32_t)((n_points + kSortTile - 1) / kSortTile);
     const bool dcf = kind == OBLIVGM_KEY_DCF;
     // at most 64 keys a round; a round's launches are its own, the sort is shared
     const double rounds = (n_keys + 63) / 64, step = n_keys / rounds * (dcf ? kDcfStep : kDpfStep);
@@ -969,10 +1100,11 @@ bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint
     }
     if (cs + rounds * kLaunch > 0.85 * (rounds * step * n_bits * (double)n_points + kLaunch)) return false;
     sg->raw = true;
-    const size_t col_end = layout_col(&C, nullptr, 0);
     sg->sort_passes = C.passes;
-    sg->sort_tiles = C.passes ? C.tiles : 0;
     sg->cols.push_back(C);
+    choose_tiles(sg);
+    C = sg->cols[0];
+    const size_t col_end = layout_col(&C, nullptr, 0);
     // one predicate per 64 keys at most and per round, fewer where their states would not fit
     SgPred p{};
     p.kind = dcf ? OBLIVGM_PRED_RANGE : OBLIVGM_PRED_EQ;
@@ -1038,7 +1170,7 @@ oblivgm_status staged_launch_raw(oblivgm_ctx* ctx, const Staged& sg, const unsig
 oblivgm_status set_staged_attrs() {
     cudaError_t e = cudaFuncSetAttribute(k_stage, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stage_last, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_combine, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_combine, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineSmem);
     return e == cudaSuccess ? OBLIVGM_OK : cuda_fail(e, "staged kernel attributes");
 }
 

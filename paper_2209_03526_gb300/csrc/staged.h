@@ -45,7 +45,7 @@ struct SgCol {
     uint32_t radd;              // <r>_1 + <r>_2 + <r>_3 of the first predicate on it
     uint32_t mask;              // 2^n_bits - 1
     uint32_t passes;            // radix passes of 8 bits; 0: the column is dense (not sorted)
-    uint32_t tiles;             // sort tiles of kSortTile elements
+    uint32_t tiles;             // sort tiles
     uint32_t* key[2];           // opened values, ping-pong; key[(passes + 1) & 1] ends up as the distinct values
     uint32_t* idx[2];           // their elements
     uint32_t* hist;             // [256][tiles] digit counts, then their exclusive sums; [tiles] for the distinct count
@@ -87,7 +87,7 @@ struct SgGroup {
     const uint32_t* share[3];
     uint32_t* out[3];
     uint64_t stride, n_elems;
-    uint64_t item_begin;        // first warp item of the group in the round
+    uint64_t item_begin;        // first tile of the group in the round
     uint32_t query_id, table_id;
     uint32_t pred_begin, n_preds;   // in the launch's predicate list
     uint32_t first;             // 1: the group's first predicate is among them; 0: the result so far is in out
@@ -116,6 +116,8 @@ struct Staged {
     std::vector<SgGroup> groups;
     std::vector<StagedRound> rounds;
     uint32_t n_keys = 0, sort_tiles = 0, sort_passes = 0;
+    uint32_t combine_threads = 0, combine_per_thread = 1;
+    bool sort_large = false;    // sort tiles of 4,096 keys instead of 1,024
     bool raw = false;           // a raw evaluation: no combine, its keys are elsewhere on the device
     size_t off_preds = 0, off_folds = 0, off_groups = 0, off_keys = 0, image_bytes = 0;
     size_t scratch_bytes = 0;
@@ -123,7 +125,7 @@ struct Staged {
 
 // Plans the staged evaluation of a launch; false when it does not pay (or does not apply) and
 // the fused kernels should run.
-bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys,
+bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
                  size_t scratch_cap, Staged* out);
 
 // Sets the pointers for scratch at a device address and builds the descriptor image's bytes.
