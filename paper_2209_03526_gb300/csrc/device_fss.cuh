@@ -2,11 +2,18 @@
 // bank-replicated shared-memory T-tables, the fixed-key PRG, and one tree
 // walk of DPF Eval / DCF Eval per (key, input) for E inputs per thread.
 //
-// Shared-memory table layout (128 KiB, dynamic shared memory offset 0):
-//   table k in {0,1,2,3} = rotl(Te0, 8k); entry idx of table k for lane L sits
-//   at byte (k >> 1) * 65536 + idx * 256 + (k & 1) * 128 + L * 4, so every lane
-//   reads its own bank and a warp-wide lookup is conflict-free for any indices.
-//   One PRMT builds idx * 256 + L * 4 from a state byte and the lane offset.
+// Shared-memory tables (128 KiB, dynamic shared memory offset 0): table k in {0,1,2,3} =
+// rotl(Te0, 8k), each entry replicated for the 32 lanes, so every lane reads its own bank and
+// a warp-wide lookup is conflict-free for any indices.  Two layouts:
+//   SmemTab      entry idx of table k for lane L at byte k * 32768 + idx * 128 + L * 4.  One
+//                DP4A builds idx * 128 + L * 4 from a state byte and the lane offset; it runs on
+//                the FMA pipe, so the ALU pipe, which the XORs of a round and the key choice
+//                fill, is left to them.  The walks run at 0.97 of the lookup rate instead of
+//                0.95: the fresh-key filter 3.78 -> 3.70 ms (131,071 elements), the staged
+//                filter 31.4 -> 30.9 ms (2^20 vertices, 8 predicates).
+//   SmemTabPair  entry idx of table k at byte (k >> 1) * 65536 + idx * 256 + (k & 1) * 128 +
+//                L * 4, addressed by one PRMT on the ALU pipe.  Gen, which has no key choice,
+//                is faster with it: 1.71 ms against 2.14 for 50,000 elements' fresh tokens.
 #pragma once
 #include <cstdint>
 
@@ -22,6 +29,7 @@ __device__ __forceinline__ uint32_t lane_offset() { return (threadIdx.x & 31u) *
 // the 1,024 (table, entry) pairs is one word replicated for the 32 lanes (128 bytes): eight
 // threads write a pair with one 16-byte store each, so a warp's store covers four whole
 // 128-byte rows (four wavefronts, no bank conflict).
+template <bool PAIR = false>
 __device__ __forceinline__ void fill_tables(uint32_t* tab, const uint32_t* __restrict__ te0) {
 #pragma unroll 4
     for (int i = threadIdx.x; i < 4 * 256 * 8; i += blockDim.x) {
@@ -29,14 +37,25 @@ __device__ __forceinline__ void fill_tables(uint32_t* tab, const uint32_t* __res
         const int k = pair >> 8, idx = pair & 255;
         const uint32_t w = __ldg(te0 + idx);
         const uint32_t v = __funnelshift_l(w, w, 8 * k);
-        reinterpret_cast<uint4*>(tab + (k >> 1) * 16384 + idx * 64 + (k & 1) * 32)[chunk] = make_uint4(v, v, v, v);
+        uint32_t* row = PAIR ? tab + (k >> 1) * 16384 + idx * 64 + (k & 1) * 32 : tab + k * 8192 + idx * 32;
+        reinterpret_cast<uint4*>(row)[chunk] = make_uint4(v, v, v, v);
     }
 }
 
-// Table access policies.  SmemTab: the bank-replicated shared-memory tables above
-// (lookup of table TABLE at byte BYTE of column col).  GlobalTab: the four 1 KiB
-// tables read straight from global memory through L1 (the plain path's layout).
+// Table access policies: lookup of table TABLE at byte BYTE of column col in the two layouts
+// above.  GlobalTab: the four 1 KiB tables read straight from global memory through L1 (the
+// plain path's layout).
 struct SmemTab {
+    const char* T;
+    uint32_t lane4;
+    template <int BYTE, int TABLE>
+    __device__ __forceinline__ uint32_t lu(uint32_t col) const {
+        const uint32_t off = __dp4a(col, 0x80u << (8 * BYTE), lane4);          // byte * 128 + lane4
+        return *reinterpret_cast<const uint32_t*>(T + off + TABLE * 32768);
+    }
+};
+
+struct SmemTabPair {
     const char* T;
     uint32_t lane4;
     template <int BYTE, int TABLE>

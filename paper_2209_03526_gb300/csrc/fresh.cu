@@ -126,7 +126,7 @@ struct SoaSink {
 };
 
 // AES under the client seed of B(c, p, tag, j) = u64 c || u16 p || u16 tag || u32 j
-__device__ __forceinline__ void client_block(const SmemTab& T, const uint32_t* rk, uint64_t c, uint32_t p,
+__device__ __forceinline__ void client_block(const SmemTabPair& T, const uint32_t* rk, uint64_t c, uint32_t p,
                                              uint32_t tag, uint32_t j, uint32_t out[4]) {
     const uint32_t in[4] = {(uint32_t)c, (uint32_t)(c >> 32), p | (tag << 16), j};
     aes_one(T, rk, in, out);
@@ -136,9 +136,9 @@ __device__ __forceinline__ void client_block(const SmemTab& T, const uint32_t* r
 template <bool DCF>
 __global__ void __launch_bounds__(fresh_gen_threads<DCF>()) k_keygen_fresh(const __grid_constant__ FreshGenParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
-    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
-    const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
+    const SmemTabPair T{reinterpret_cast<const char*>(smem), lane_offset()};
     constexpr bool eq = !DCF;
     const uint32_t n = P.n;
     const uint32_t m = n >= 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);

@@ -23,7 +23,7 @@ struct GenRightKeys {
 
 // child of a seed under the round keys rk of its direction: seed with bit 0 of byte 0
 // cleared, control bit apart
-__device__ __forceinline__ void gen_expand(const SmemTab& T, const uint32_t* rk, const uint32_t s[4], uint32_t cs[4],
+__device__ __forceinline__ void gen_expand(const SmemTabPair& T, const uint32_t* rk, const uint32_t s[4], uint32_t cs[4],
                                            uint32_t& ct) {
     uint32_t o[4];
     aes_one(T, rk, s, o);
@@ -38,7 +38,7 @@ __device__ __forceinline__ void gen_expand(const SmemTab& T, const uint32_t* rk,
 // keep/lose choices are selects, so everything stays in registers.  One instance per
 // kind keeps the DPF loop free of the DCF's value blocks.
 template <bool DCF, class Sink>
-__device__ __forceinline__ void gen_pair(const SmemTab& T, const AesParams& A, const GenRightKeys& R, int n,
+__device__ __forceinline__ void gen_pair(const SmemTabPair& T, const AesParams& A, const GenRightKeys& R, int n,
                                          uint32_t alpha, uint32_t beta, uint32_t s0[4], uint32_t s1[4], Sink& sink) {
     constexpr bool dcf = DCF;
     uint32_t t0 = 0u, t1 = 1u, valpha = 0u;

@@ -80,9 +80,9 @@ struct WarpWireSink {
 template <int kThreads, bool DCF>
 __global__ void __launch_bounds__(kThreads) k_keygen(const __grid_constant__ KeygenParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
-    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
-    const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
+    const SmemTabPair T{reinterpret_cast<const char*>(smem), lane_offset()};
     const uint32_t L = P.key_len;
     const int n = (int)P.n;
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
