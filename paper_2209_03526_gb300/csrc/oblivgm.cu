@@ -596,6 +596,46 @@ void build_aes_params(AesParams* a) {
     }
 }
 
+// The staged evaluation's scratch pool of a device, shared by its contexts (a new context's
+// first call then finds memory that another one's calls have already mapped) and destroyed with
+// the last of them.  It keeps at most kScratchKeep bytes between calls.
+namespace {
+struct ScratchPool {
+    cudaMemPool_t pool = nullptr;
+    int users = 0;
+};
+std::mutex g_pool_mu;
+std::map<int, ScratchPool> g_pools;
+}  // namespace
+
+static cudaError_t scratch_pool_acquire(int device, cudaMemPool_t* out) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    ScratchPool& p = g_pools[device];
+    if (p.users == 0) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaError_t e = cudaMemPoolCreate(&p.pool, &props);
+        if (e != cudaSuccess) return e;
+        uint64_t keep = kScratchKeep;
+        e = cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(p.pool);
+            return e;
+        }
+    }
+    p.users++;
+    *out = p.pool;
+    return cudaSuccess;
+}
+
+static void scratch_pool_release(int device) {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    ScratchPool& p = g_pools[device];
+    if (--p.users == 0) cudaMemPoolDestroy(p.pool);
+}
+
 static oblivgm_status check_ctx(oblivgm_ctx* ctx) {
     if (!ctx) return fail(OBLIVGM_EINVAL, "NULL context");
     cudaError_t e = cudaSetDevice(ctx->device);
@@ -624,21 +664,39 @@ struct Plan {
 // the shortest makespan wins (the widest on ties).  Large item counts skip the search:
 // their tail is already a small fraction.
 // Makespan of the greedy schedule: items (group, tile) in group order, each taken by the CTA
-// that is free first (one persistent CTA per SM); tile_of(g) is group g's width.
+// that is free first (one persistent CTA per SM); tile_of(g) is group g's width.  A group's
+// items take equal times (but the last), so the CTAs stay in a few classes of equal finishing
+// times, and a class takes its items together: a heap of 152 CTAs and one step per item took
+// most of a small call's 240 us.
+struct CtaClass {
+    double t;      // when these CTAs are free
+    uint64_t n;    // how many they are
+};
+
+inline void place_items(std::vector<CtaClass>& free_at, uint64_t items, double time) {
+    while (items > 0) {
+        CtaClass& first = free_at.front();
+        const CtaClass moved{first.t + time, std::min(first.n, items)};
+        first.n -= moved.n;
+        items -= moved.n;
+        if (first.n == 0) free_at.erase(free_at.begin());
+        auto at = std::lower_bound(free_at.begin(), free_at.end(), moved.t,
+                                   [](const CtaClass& c, double t) { return c.t < t; });
+        if (at != free_at.end() && at->t == moved.t) at->n += moved.n;
+        else free_at.insert(at, moved);
+    }
+}
+
 template <typename NF, typename WF, typename TF>
 double simulate_makespan(size_t n_groups, NF n_elems_of, WF tile_of, TF item_time, int sm_count,
-                         std::vector<double>& finish) {
-    finish.assign((size_t)sm_count, 0.0);
-    std::make_heap(finish.begin(), finish.end(), std::greater<double>());
+                         std::vector<CtaClass>& free_at) {
+    free_at.assign(1, CtaClass{0.0, (uint64_t)sm_count});
     for (size_t g = 0; g < n_groups; g++) {
         const uint64_t n = n_elems_of(g), t = tile_of(g);
-        for (uint64_t e = 0; e < n; e += t) {
-            std::pop_heap(finish.begin(), finish.end(), std::greater<double>());
-            finish.back() += item_time(g, std::min<uint64_t>(t, n - e));
-            std::push_heap(finish.begin(), finish.end(), std::greater<double>());
-        }
+        if (n >= t) place_items(free_at, n / t, item_time(g, t));
+        if (n % t) place_items(free_at, 1, item_time(g, n % t));
     }
-    return *std::max_element(finish.begin(), finish.end());
+    return free_at.back().t;
 }
 
 template <typename NF, typename TF>
@@ -648,7 +706,7 @@ uint32_t choose_tile(size_t n_groups, NF n_elems_of, TF item_time, uint32_t max_
     if (items_at_max == 0 || items_at_max > 64ull * (uint64_t)sm_count || step == 0) return max_tile;
     uint32_t best_tile = max_tile;
     double best = -1.0;
-    std::vector<double> finish;
+    std::vector<CtaClass> finish;
     for (uint32_t t = max_tile; t >= step; t -= step) {
         if (best >= 0) {
             // skip a width whose work, spread evenly over the SMs, already takes longer
@@ -679,7 +737,7 @@ uint32_t choose_tile(size_t n_groups, NF n_elems_of, TF item_time, uint32_t max_
 template <typename NF, typename TF, typename MF>
 void choose_group_tiles(size_t n_groups, NF n_elems_of, TF item_time, MF max_tile_of, int sm_count,
                         std::vector<uint32_t>& tiles) {
-    std::vector<double> finish;
+    std::vector<CtaClass> finish;
     auto makespan = [&]() {
         return simulate_makespan(n_groups, n_elems_of, [&](size_t g) { return (uint64_t)tiles[g]; }, item_time,
                                  sm_count, finish);
@@ -737,7 +795,7 @@ double wp_item_time(const GroupCost& c, uint64_t width) {
 
 oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_queries, const uint32_t* query_ids,
                             const ParsedQuery* parsed, const uint32_t* n_groups, uint32_t* const* const* outs,
-                            uint32_t tile, uint32_t step, bool wp, int sm_count, Plan* plan) {
+                            const oblivgm_ctx* ctx, Plan* plan) {
     struct G { GroupDesc d; std::vector<const ParsedPred*> preds; GroupCost cost; };
     std::vector<G> all;
     for (uint32_t q = 0; q < n_queries; q++) {
@@ -790,12 +848,22 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
         }
     }
     std::stable_sort(all.begin(), all.end(), [](const G& a, const G& b) { return a.cost.walk_cost > b.cost.walk_cost; });
-    const uint32_t max_tile = tile;
+    // a batch whose groups hold at most ctx->wp_max_elems elements in all takes the walk-parallel
+    // kernel, in tiles of kWpElems elements (a forced tile, oblivgm_set_walk_parallel_tile, skips the
+    // search: step 0)
+    uint64_t total = 0;
+    for (const G& g : all) total += g.d.n_elems;
+    const bool wp = plan->wp = total != 0 && total <= ctx->wp_max_elems;
+    plan->elems_per_thread = wp ? 1 : ctx->elems_per_thread;
+    plan->threads = wp ? kWpThreads : ctx->threads;
+    const int sm_count = ctx->sm_count;
+    const uint32_t max_tile = !wp ? ctx->threads * ctx->elems_per_thread : ctx->wp_tile ? ctx->wp_tile : kWpElems;
+    const uint32_t step = !wp ? 32 * ctx->elems_per_thread : ctx->wp_tile ? 0 : 1;
     const auto n_of = [&](size_t i) { return all[i].d.n_elems; };
     const auto time_of = [&](size_t i, uint64_t w) {
         return wp ? wp_item_time(all[i].cost, w) : filter_item_time(all[i].cost, w);
     };
-    tile = choose_tile(all.size(), n_of, time_of, max_tile, step, sm_count);
+    const uint32_t tile = choose_tile(all.size(), n_of, time_of, max_tile, step, sm_count);
     std::vector<uint32_t> tiles(all.size(), tile);
     if (wp && step != 0 && all.size() > 1 && all.size() <= kWpTileGroups) {
         uint64_t items_at_max = 0;
@@ -839,32 +907,13 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
 oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& tables, uint32_t n_queries,
                            const uint32_t* query_ids, const ParsedQuery* parsed, const uint32_t* n_groups,
                            uint32_t* const* const* outs, bool staged_ok, Plan* plan) {
-    const uint32_t threads = ctx->threads, E = ctx->elems_per_thread;
     plan->staged = false;
-    plan->elems_per_thread = E;
-    plan->threads = threads;
-    plan->wp = false;
-    oblivgm_status s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, threads * E, 32 * E,
-                                    false, ctx->sm_count, plan);
-    if (s != OBLIVGM_OK) return s;
-    uint64_t total = 0;
-    for (const GroupDesc& g : plan->groups) total += g.n_elems;
-    if (total == 0) return OBLIVGM_OK;
-    if (total > ctx->wp_max_elems) {
-        // large launches share tree nodes between elements where that pays; the key-staging
-        // expiry hook is about the fused kernels' waits
-        if (staged_ok && !ctx->test_expire_next)
-            plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap,
-                                       &plan->sg);
-        return OBLIVGM_OK;
-    }
-    // a forced tile (oblivgm_set_walk_parallel_tile) skips the search: step 0
-    s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, ctx->wp_tile ? ctx->wp_tile : kWpElems,
-                     ctx->wp_tile ? 0 : 1, true, ctx->sm_count, plan);
-    if (s != OBLIVGM_OK) return s;
-    plan->wp = true;
-    plan->threads = kWpThreads;
-    plan->elems_per_thread = 1;
+    const oblivgm_status s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, ctx, plan);
+    if (s != OBLIVGM_OK || plan->wp) return s;
+    // large launches share tree nodes between elements where that pays; the key-staging expiry
+    // hook is about the fused kernels' waits
+    if (staged_ok && !ctx->test_expire_next)
+        plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap, &plan->sg);
     return OBLIVGM_OK;
 }
 
@@ -1079,15 +1128,7 @@ oblivgm_status oblivgm_create(oblivgm_ctx** out, int32_t device, const oblivgm_c
         uint64_t keep = UINT64_MAX;
         if (e == cudaSuccess) e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
-    if (e == cudaSuccess) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = device;
-        e = cudaMemPoolCreate(&ctx->scratch_pool, &props);
-        uint64_t keep = kScratchKeep;
-        if (e == cudaSuccess) e = cudaMemPoolSetAttribute(ctx->scratch_pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    }
+    if (e == cudaSuccess) e = scratch_pool_acquire(device, &ctx->scratch_pool);
     if (e != cudaSuccess) {
         st = cuda_fail(e, "context set-up");
         oblivgm_destroy(ctx);
@@ -1109,7 +1150,7 @@ oblivgm_status oblivgm_destroy(oblivgm_ctx* ctx) {
     if (ctx->d_te0) cudaFree(ctx->d_te0);
     if (ctx->d_te4) cudaFree(ctx->d_te4);
     if (ctx->d_error) cudaFree(ctx->d_error);
-    if (ctx->scratch_pool) cudaMemPoolDestroy(ctx->scratch_pool);
+    if (ctx->scratch_pool) scratch_pool_release(ctx->device);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     delete ctx;
     return OBLIVGM_OK;
