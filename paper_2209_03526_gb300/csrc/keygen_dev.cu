@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(kThreads) k_keygen(const __grid_constant__ Key
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t* stage = reinterpret_cast<uint32_t*>(smem + kTableBytes) + warp * 32 * WarpWireSink<DCF>::kWords;
     const uint64_t warps_total = (uint64_t)gridDim.x * (blockDim.x >> 5);
-    for (uint64_t chunk = (uint64_t)blockIdx.x * (blockDim.x >> 5) + warp; chunk * 32 < P.n_pairs;
+    // consecutive chunks go to different SMs, so every SM gets the same number of them but one
+    for (uint64_t chunk = (uint64_t)warp * gridDim.x + blockIdx.x; chunk * 32 < P.n_pairs;
          chunk += warps_total) {
         const uint64_t first = chunk * 32;
         const uint64_t i = first + lane < P.n_pairs ? first + lane : P.n_pairs - 1;
@@ -159,12 +160,12 @@ extern "C" oblivgm_status oblivgm_keygen_device(oblivgm_ctx* ctx, uint32_t kind,
     P.n = n_bits;
     P.kind = kind;
     P.key_len = L;
-    const unsigned grid =
-        (unsigned)std::min<uint64_t>((n_pairs + kKeygenThreads - 1) / kKeygenThreads, (uint64_t)ctx->sm_count);
+    const unsigned threads = even_threads(n_pairs, ctx->sm_count, kKeygenThreads);
+    const unsigned grid = (unsigned)std::min<uint64_t>((n_pairs + threads - 1) / threads, (uint64_t)ctx->sm_count);
     if (kind == OBLIVGM_KEY_DCF)
-        k_keygen<kKeygenThreads, true><<<grid, kKeygenThreads, kKeygenSmem, static_cast<cudaStream_t>(stream)>>>(P);
+        k_keygen<kKeygenThreads, true><<<grid, threads, kKeygenSmem, static_cast<cudaStream_t>(stream)>>>(P);
     else
-        k_keygen<kKeygenThreads, false><<<grid, kKeygenThreads, kKeygenSmem, static_cast<cudaStream_t>(stream)>>>(P);
+        k_keygen<kKeygenThreads, false><<<grid, threads, kKeygenSmem, static_cast<cudaStream_t>(stream)>>>(P);
     ctx->launches++;
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_fail(ce, "k_keygen launch");

@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <condition_variable>
 #include <cstdint>
@@ -132,6 +133,16 @@ struct oblivgm_ctx {
 };
 
 namespace ogm {
+
+// Threads per CTA for a persistent grid of one CTA per SM over `items` items: as many as give
+// its waves equal widths, so that the last one does not run on a few warps (131,071 items on 152
+// SMs of 768 threads: a full wave and one of 12 %).
+inline unsigned even_threads(uint64_t items, int sm_count, unsigned max_threads) {
+    const uint64_t per_sm = (items + sm_count - 1) / sm_count;
+    const uint64_t waves = std::max<uint64_t>(1, (per_sm + max_threads - 1) / max_threads);
+    const uint64_t t = (per_sm + waves - 1) / waves;
+    return (unsigned)std::min<uint64_t>(max_threads, std::max<uint64_t>(64, (t + 31) / 32 * 32));
+}
 
 oblivgm_status fail(oblivgm_status st, const std::string& msg);
 const std::string& last_error_text();   // the calling thread's last failure text

@@ -589,7 +589,8 @@ constexpr int kCombineSmem = kTableBytes + kMaxPrefixes * kPrefixWords * 4;
 
 // index of element e's value in a predicate's sums
 __device__ __forceinline__ uint32_t value_index(const SgGroup& G, const SgFold& D, uint64_t e) {
-    if (!D.dense) return __ldg(D.rank + e);
+    if (D.index == kIndexRank) return __ldg(D.rank + e);
+    if (D.index == kIndexElem) return (uint32_t)e;
     const uint64_t row = (uint64_t)D.attr * G.stride + e;
     return (__ldg(G.share[0] + row) + __ldg(G.share[1] + row) + __ldg(G.share[2] + row) + D.radd) & D.mask;
 }
@@ -726,7 +727,6 @@ constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, 
 constexpr double kSortKeyPass = 12e-12;
 constexpr uint64_t kMaxElems = 1ull << 28;
 constexpr uint32_t kMaxChunk = 1u << 22;      // distinct values evaluated together
-constexpr size_t kRoundBytes = 5ull << 29;    // states of the predicates evaluated together (2.5 GiB)
 constexpr int kMaxDenseBits = 24;
 
 // distinct l-bit prefixes of n_vals uniform values, the most that a column can be expected to have
@@ -823,6 +823,41 @@ size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
 
 }  // namespace
 
+// Elements per tile of the combine: narrower CTAs where that spreads a small launch over more
+// SMs, several elements per thread, so that a tile's barriers are rare, where every SM still
+// gets a few tiles.
+CombineShape combine_shape(uint64_t elems, uint32_t most_preds, int sm_count) {
+    CombineShape c;
+    c.threads = elems >= (uint64_t)kStageThreads * sm_count ? kStageThreads : elems >= 512ull * sm_count ? 512 : 256;
+    const uint64_t spread = elems / (6ull * kStageThreads * sm_count);
+    c.per_thread = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({8, spread, kMaxTileSteps / most_preds}));
+    return c;
+}
+
+uint64_t combine_tiles(const CombineShape& c, SgGroup* groups, uint32_t n_groups) {
+    const uint64_t tile = (uint64_t)c.threads * c.per_thread;
+    uint64_t items = 0;
+    for (uint32_t g = 0; g < n_groups; g++) {
+        groups[g].item_begin = items;
+        items += (groups[g].n_elems + tile - 1) / tile;
+    }
+    return items;
+}
+
+void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* groups, uint32_t n_groups,
+                    const SgFold* folds, uint64_t items, cudaStream_t s) {
+    CombineParams F{};
+    std::memcpy(F.rk_prf, ctx->rk_prf, sizeof F.rk_prf);
+    F.te0 = ctx->d_te0;
+    F.folds = folds;
+    F.groups = groups;
+    F.n_groups = n_groups;
+    F.items = items;
+    F.per_thread = c.per_thread;
+    k_combine<<<(unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, items), c.threads, kCombineSmem, s>>>(F);
+    ctx->launches++;
+}
+
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
                  size_t scratch_cap, Staged* sg) {
     *sg = Staged{};
@@ -884,12 +919,6 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
     choose_tiles(sg);
     size_t col_end = 0;
     for (SgCol& C : sg->cols) col_end = layout_col(&C, nullptr, col_end);
-    // elements per tile of the combine: narrower where that spreads a small launch over more SMs
-    uint64_t elems = 0;
-    for (const GroupDesc& G : groups) elems += G.n_elems;
-    sg->combine_threads = elems >= (uint64_t)kStageThreads * sm_count ? kStageThreads
-                          : elems >= 512ull * sm_count               ? 512
-                                                                     : 256;
     // predicates in group order, cut into rounds whose states fit kRoundBytes
     size_t at = col_end, most = col_end;
     StagedRound R{};
@@ -945,7 +974,7 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
             f.step = D.step; f.lin = D.lin; f.prod = D.prod; f.attr = D.attr;
             f.radd = D.r[0] + D.r[1] + D.r[2];
             f.mask = p.mask;
-            f.dense = p.dense;
+            f.index = p.dense ? kIndexDense : kIndexRank;
             sg->preds.push_back(p);
             sg->folds.push_back(f);
             R.n_preds++;
@@ -958,18 +987,14 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         }
     }
     close();
-    // several elements per thread, so that a tile's barriers are rare, while every SM gets a few tiles
     uint32_t most_preds = 1;
-    for (const SgGroup& g : sg->groups) most_preds = std::max(most_preds, g.n_preds);
-    const uint64_t spread = elems / (6ull * kStageThreads * sm_count);
-    sg->combine_per_thread = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({8, spread, kMaxTileSteps / most_preds}));
-    for (StagedRound& r : sg->rounds) {
-        const uint64_t tile = (uint64_t)sg->combine_threads * sg->combine_per_thread;
-        for (uint32_t g = r.group_begin; g < r.group_begin + r.n_groups; g++) {
-            sg->groups[g].item_begin = r.items;
-            r.items += (sg->groups[g].n_elems + tile - 1) / tile;
-        }
+    uint64_t elems = 0;
+    for (const SgGroup& g : sg->groups) {
+        most_preds = std::max(most_preds, g.n_preds);
+        elems += g.first ? g.n_elems : 0;
     }
+    sg->shape = combine_shape(elems, most_preds, sm_count);
+    for (StagedRound& r : sg->rounds) r.items = combine_tiles(sg->shape, sg->groups.data() + r.group_begin, r.n_groups);
     sg->scratch_bytes = most;
     if (sg->scratch_bytes > scratch_cap) { *sg = Staged{}; return false; }
     sg->off_preds = up256(sg->cols.size() * sizeof(SgCol));
@@ -1055,19 +1080,11 @@ uint64_t launch_round(const oblivgm_ctx* ctx, const StagedRound& R, const SgPred
 
 oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s) {
     uint64_t launches = launch_sort(sg, reinterpret_cast<const SgCol*>(image), s);
-    CombineParams F{};
-    std::memcpy(F.rk_prf, ctx->rk_prf, sizeof F.rk_prf);
-    F.te0 = ctx->d_te0;
-    F.folds = reinterpret_cast<const SgFold*>(image + sg.off_folds);
-    F.per_thread = sg.combine_per_thread;
     for (const StagedRound& R : sg.rounds) {
         launches += launch_round(ctx, R, reinterpret_cast<const SgPred*>(image + sg.off_preds),
                                  reinterpret_cast<const DevKey*>(image + sg.off_keys), s);
-        F.groups = reinterpret_cast<const SgGroup*>(image + sg.off_groups) + R.group_begin;
-        F.n_groups = R.n_groups;
-        F.items = R.items;
-        k_combine<<<(unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, R.items), sg.combine_threads, kCombineSmem, s>>>(F);
-        launches++;
+        launch_combine(ctx, sg.shape, reinterpret_cast<const SgGroup*>(image + sg.off_groups) + R.group_begin, R.n_groups,
+                       reinterpret_cast<const SgFold*>(image + sg.off_folds), R.items, s);
     }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "staged launch");

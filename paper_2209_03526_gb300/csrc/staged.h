@@ -37,6 +37,7 @@ struct PredDesc {
 };
 
 constexpr int kSgMaxStages = 33;
+constexpr size_t kRoundBytes = 5ull << 29;    // scratch of the predicates evaluated together (2.5 GiB)
 
 // One opened column of the launch (an attribute of a table, all its elements).
 struct SgCol {
@@ -96,10 +97,25 @@ struct SgGroup {
 
 struct SgFold {                 // per predicate, next to SgPred
     uint32_t step, lin, prod, attr;
-    uint32_t radd, mask, dense, pad;
+    uint32_t radd, mask;
+    uint32_t index;             // kIndexRank, kIndexDense or kIndexElem: which sums are element e's
+    uint32_t pad;
     const uint32_t* rank;
-    const uint32_t* z;
+    const uint32_t* z;          // four words per value: the three servers' sums
 };
+constexpr uint32_t kIndexRank = 0;    // those of value rank[e]
+constexpr uint32_t kIndexDense = 1;   // those of value x^, opened from the shares
+constexpr uint32_t kIndexElem = 2;    // those of element e (fresh keys)
+
+// The re-share and fold over predicates' sums: tile shape for `elems` elements in all with at most
+// most_preds predicates in a group entry, the entries' first tiles (returns the tiles), launch.
+struct CombineShape {
+    uint32_t threads = 0, per_thread = 1;
+};
+CombineShape combine_shape(uint64_t elems, uint32_t most_preds, int sm_count);
+uint64_t combine_tiles(const CombineShape& c, SgGroup* groups, uint32_t n_groups);
+void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* groups, uint32_t n_groups,
+                    const SgFold* folds, uint64_t items, cudaStream_t s);
 
 struct StagedRound {
     uint32_t pred_begin = 0, n_preds = 0;
@@ -116,7 +132,7 @@ struct Staged {
     std::vector<SgGroup> groups;
     std::vector<StagedRound> rounds;
     uint32_t n_keys = 0, sort_tiles = 0, sort_passes = 0;
-    uint32_t combine_threads = 0, combine_per_thread = 1;
+    CombineShape shape;
     bool sort_large = false;    // sort tiles of 4,096 keys instead of 1,024
     bool raw = false;           // a raw evaluation: no combine, its keys are elsewhere on the device
     size_t off_preds = 0, off_folds = 0, off_groups = 0, off_keys = 0, image_bytes = 0;
