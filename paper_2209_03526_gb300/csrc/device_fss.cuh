@@ -12,8 +12,8 @@
 //                0.95: the fresh-key filter 3.78 -> 3.70 ms (131,071 elements), the staged
 //                filter 31.4 -> 30.9 ms (2^20 vertices, 8 predicates).
 //   SmemTabPair  entry idx of table k at byte (k >> 1) * 65536 + idx * 256 + (k & 1) * 128 +
-//                L * 4, addressed by one PRMT on the ALU pipe.  Gen, which has no key choice,
-//                is faster with it: 1.71 ms against 2.14 for 50,000 elements' fresh tokens.
+//                L * 4, addressed by one PRMT on the ALU pipe: the shuffle's, whose mask blocks
+//                have no key choice.
 #pragma once
 #include <cstdint>
 

@@ -2,7 +2,7 @@
 // attribute value (Sec. V-C, the basic approach): predicate p meets element c with its
 // own mask r_{c,p} and its own three key pairs, so no two opened values x^ share a mask.
 //
-//   k_keygen_fresh  the client's Gen, one thread per (element, predicate, pair, key):
+//   k_keygen_fresh  the client's Gen, two lanes per (element, predicate, pair, key):
 //                   mask block and root seeds from AES under the client seed, then the
 //                   DPF / DCF Gen of gen_device.cuh, written level-major so that the
 //                   servers' reads are coalesced.
@@ -38,12 +38,12 @@ namespace {
 constexpr uint32_t kFreshMagic = 0x464D474Fu;
 constexpr int kFreshMaxPreds = 64;
 constexpr int kFreshMaxJobs = kFreshMaxPreds * 6;
-// client Gen: one CTA per SM (the tables take 128 KiB); both instances need more than the
-// 80 registers a 768-thread CTA leaves
+// client Gen: one CTA per SM (the tables take 128 KiB).  512 threads leave a DCF pair's lane its
+// 100 registers: 50,000 elements' tokens take 1.62 ms, 1.76 with 768 threads and 80.
 #ifndef OGM_FRESH_GEN_THREADS
 #define OGM_FRESH_GEN_THREADS 512
 #endif
-template <bool DCF> constexpr int fresh_gen_threads() { return OGM_FRESH_GEN_THREADS; }
+constexpr int kFreshGenThreads = OGM_FRESH_GEN_THREADS;
 #ifndef OGM_FRESH_EVAL_THREADS
 #define OGM_FRESH_EVAL_THREADS 768
 #endif
@@ -86,7 +86,6 @@ struct GenJob {
 
 struct FreshGenParams {
     AesParams aes;
-    GenRightKeys right;
     uint32_t rk_client[44];
     const uint32_t* te0;
     uint32_t n, n_jobs;
@@ -100,58 +99,56 @@ __device__ __forceinline__ void st_u128(uint8_t* p, const uint32_t w[4]) {
     *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// level-major key blocks: element c's words of both keys of the pair
+// level-major key blocks: element c's words of this lane's key of the pair
 struct SoaSink {
-    uint8_t* b[2];         // key block of party 0 and party 1
-    uint64_t N, N4, c;
+    uint8_t* b;            // the key's block; its owner's
+    const FreshLayout& L;  // in the launch parameters: the strides take no registers
     uint32_t n, tlw, trw;
-    bool dcf;
+    uint64_t c;
+    bool dcf, real;        // real: false for a lane past the last pair, which stores nothing
     __device__ __forceinline__ void level(int lv, const uint32_t scw[4], uint32_t tl, uint32_t tr, uint32_t vcw) {
-        const uint64_t o = 16 * N + 16 * ((uint64_t)lv * N + c);
-        st_u128(b[0] + o, scw);
-        st_u128(b[1] + o, scw);
         tlw |= tl << lv;
         trw |= tr << lv;
-        if (dcf) {
-            const uint64_t ov = 16 * N + 16 * (uint64_t)n * N + 8 * N4 + 4 * ((uint64_t)lv * N4 + c);
-            st_u32(b[0] + ov, vcw);
-            st_u32(b[1] + ov, vcw);
-        }
+        if (!real) return;
+        st_u128(b + 16 * ((uint64_t)(lv + 1) * L.N + c), scw);
+        if (dcf) st_u32(b + 16 * (uint64_t)(n + 1) * L.N + 4 * ((uint64_t)(lv + 2) * L.N4 + c), vcw);
     }
     __device__ __forceinline__ void final(uint32_t cw) {
-        const uint64_t ot = 16 * N + 16 * (uint64_t)n * N;
-        const uint64_t oc = ot + 8 * N4 + (dcf ? 4 * (uint64_t)n * N4 : 0);
-        for (int k = 0; k < 2; k++) {
-            st_u32(b[k] + ot + 4 * c, tlw);
-            st_u32(b[k] + ot + 4 * N4 + 4 * c, trw);
-            st_u32(b[k] + oc + 4 * c, cw);
-        }
+        if (!real) return;
+        uint8_t* t = b + 16 * (uint64_t)(n + 1) * L.N + 4 * c;
+        st_u32(t, tlw);
+        st_u32(t + 4 * L.N4, trw);
+        st_u32(t + 4 * (2 + (dcf ? (uint64_t)n : 0)) * L.N4, cw);
     }
 };
 
 // AES under the client seed of B(c, p, tag, j) = u64 c || u16 p || u16 tag || u32 j
-__device__ __forceinline__ void client_block(const SmemTabPair& T, const uint32_t* rk, uint64_t c, uint32_t p,
+__device__ __forceinline__ void client_block(const SmemTab& T, const uint32_t* rk, uint64_t c, uint32_t p,
                                              uint32_t tag, uint32_t j, uint32_t out[4]) {
     const uint32_t in[4] = {(uint32_t)c, (uint32_t)(c >> 32), p | (tag << 16), j};
     aes_one(T, rk, in, out);
 }
 
-// one instance per predicate kind (EQ: DPF keys, RANGE: DCF keys), launched on its own jobs
+// one instance per predicate kind (EQ: DPF keys, RANGE: DCF keys), launched on its own jobs; a
+// pair of lanes per (job, element)
 template <bool DCF>
-__global__ void __launch_bounds__(fresh_gen_threads<DCF>()) k_keygen_fresh(const __grid_constant__ FreshGenParams P) {
+__global__ void __launch_bounds__(kFreshGenThreads) k_keygen_fresh(const __grid_constant__ FreshGenParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
-    fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
+    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
-    const SmemTabPair T{reinterpret_cast<const char*>(smem), lane_offset()};
+    const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
     constexpr bool eq = !DCF;
     const uint32_t n = P.n;
     const uint32_t m = n >= 32 ? 0xFFFFFFFFu : ((1u << n) - 1u);
     constexpr int nsub = eq ? 1 : 2;
-    // one persistent grid over all (job, element) items of the launch, so no CTA waits on
-    // a short last wave
-    const uint64_t total = P.job_start[P.n_jobs];
-    for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-         idx += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t lane = threadIdx.x & 31, party = lane & 1u;
+    // one persistent grid over all (job, element) items of the launch, 16 to a warp, so no CTA
+    // waits on a short last wave; whole warps stay in the loop (gen_pair's exchange)
+    const uint64_t total = P.job_start[P.n_jobs], step = (uint64_t)gridDim.x * (blockDim.x >> 5) * 16;
+    for (uint64_t first = ((uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 16; first < total; first += step) {
+        const uint64_t mine = first + (lane >> 1);
+        const bool real = mine < total;
+        const uint64_t idx = real ? mine : total - 1;
         uint32_t lo = 0, hi = P.n_jobs - 1;
         while (lo < hi) {
             const uint32_t mid = (lo + hi + 1) >> 1;
@@ -161,17 +158,17 @@ __global__ void __launch_bounds__(fresh_gen_threads<DCF>()) k_keygen_fresh(const
         const FreshPred& Q = P.preds[J.pred];
         const FreshLayout& L = Q.lay;
         const uint64_t c = idx - P.job_start[lo];
-        // owners (server, half) of the pair's two keys, from the assignment
+        // owner (server, half) of this lane's key, from the assignment
         // CS1 (1,0),(2,0); CS2 (2,1),(3,0); CS3 (3,1),(1,1): party 0 of pairs 1, 2, 3 sits with
         // CS1 A, CS1 B, CS2 B; party 1 with CS3 B, CS2 A, CS3 A
-        const uint32_t srv0 = J.pair == 2 ? 1u : 0u, half0 = J.pair == 0 ? 0u : 1u;
-        const uint32_t srv1 = J.pair == 1 ? 1u : 2u, half1 = J.pair == 0 ? 1u : 0u;
+        const uint32_t srv = party ? (J.pair == 1 ? 1u : 2u) : (J.pair == 2 ? 1u : 0u);
+        const uint32_t half = (J.pair == 0) == (party != 0) ? 1u : 0u;
         uint32_t w[4];
         client_block(T, P.rk_client, c, Q.step, 1u, 0u, w);
         const uint32_t r = w[0] & m;
-        const uint32_t rs[3] = {w[1] & m, w[2] & m, (r - (w[1] & m) - (w[2] & m)) & m};
         const uint32_t a0 = (Q.lo + r) & m, a1 = (Q.hi + 1u + r) & m;
-        if (J.pair == 0 && J.sub == 0) {
+        if (real && party == 0 && J.pair == 0 && J.sub == 0) {
+            const uint32_t rs[3] = {w[1] & m, w[2] & m, (r - (w[1] & m) - (w[2] & m)) & m};
 #pragma unroll
             for (int i = 0; i < 3; i++) {
                 st_u32(Q.data[i] + 4 * c, rs[i]);
@@ -181,21 +178,11 @@ __global__ void __launch_bounds__(fresh_gen_threads<DCF>()) k_keygen_fresh(const
         }
         const uint32_t alpha = eq ? a0 : (J.sub == 0 ? a1 : a0);
         const uint32_t beta = (eq || J.sub == 0) ? kBetaPrime : 0u - kBetaPrime;
-        uint32_t s0[4], s1[4];
-        client_block(T, P.rk_client, c, Q.step, 2u, 4u * J.pair + 2u * J.sub + 0u, s0);
-        client_block(T, P.rk_client, c, Q.step, 2u, 4u * J.pair + 2u * J.sub + 1u, s1);
-        SoaSink sink;
-        sink.b[0] = Q.data[srv0] + L.keys_at + (uint64_t)(half0 * nsub + J.sub) * L.key_block;
-        sink.b[1] = Q.data[srv1] + L.keys_at + (uint64_t)(half1 * nsub + J.sub) * L.key_block;
-        st_u128(sink.b[0] + 16 * c, s0);
-        st_u128(sink.b[1] + 16 * c, s1);
-        sink.N = L.N;
-        sink.N4 = L.N4;
-        sink.c = c;
-        sink.n = n;
-        sink.tlw = sink.trw = 0;
-        sink.dcf = !eq;
-        gen_pair<DCF>(T, P.aes, P.right, (int)n, alpha, beta, s0, s1, sink);
+        uint32_t s[4];
+        client_block(T, P.rk_client, c, Q.step, 2u, 4u * J.pair + 2u * J.sub + party, s);
+        SoaSink sink{Q.data[srv] + L.keys_at + (uint64_t)(half * nsub + J.sub) * L.key_block, L, n, 0u, 0u, c, !eq, real};
+        if (real) st_u128(sink.b + 16 * c, s);
+        gen_pair<DCF>(T, P.aes, (int)n, alpha, beta, party, s, sink);
     }
 }
 
@@ -491,10 +478,6 @@ extern "C" oblivgm_status oblivgm_keygen_fresh(oblivgm_ctx* ctx, const oblivgm_p
     FreshGenParams P;
     std::memset(&P, 0, sizeof P);
     P.aes = ctx->aes;
-    for (int w = 0; w < 44; w++) {
-        P.right.st[w] = ctx->aes.rk_st[w] ^ ctx->aes.d_st[w];
-        P.right.v[w] = ctx->aes.rk_v[w] ^ ctx->aes.d_v[w];
-    }
     const RoundKeys rk = expand_key(seed);
     std::memcpy(P.rk_client, rk.w, sizeof P.rk_client);
     P.te0 = ctx->d_te0;
@@ -559,9 +542,9 @@ extern "C" oblivgm_status oblivgm_keygen_fresh(oblivgm_ctx* ctx, const oblivgm_p
         P.job_start[0] = 0;
         for (uint32_t j = 0; j < P.n_jobs; j++) P.job_start[j + 1] = P.job_start[j] + P.preds[jl[j].pred].lay.N;
         if (P.job_start[P.n_jobs] == 0) continue;
-        const uint64_t threads = even_threads(P.job_start[P.n_jobs], ctx->sm_count,
-                                              kind ? fresh_gen_threads<true>() : fresh_gen_threads<false>());
-        const uint64_t grid = std::min<uint64_t>((P.job_start[P.n_jobs] + threads - 1) / threads, ctx->sm_count);
+        const uint64_t lanes = 2 * P.job_start[P.n_jobs];
+        const uint64_t threads = even_threads(lanes, ctx->sm_count, kFreshGenThreads);
+        const uint64_t grid = std::min<uint64_t>((lanes + threads - 1) / threads, ctx->sm_count);
         if (kind) k_keygen_fresh<true><<<(unsigned)grid, (unsigned)threads, kTableBytes, s>>>(P);
         else k_keygen_fresh<false><<<(unsigned)grid, (unsigned)threads, kTableBytes, s>>>(P);
         ctx->launches++;

@@ -13,73 +13,71 @@
 
 namespace ogm {
 
-// The round keys of the right-child PRG keys (K_R for the seed / control-bit block, K_vR
-// for the DCF value block); the left-child ones are AesParams::rk_st and rk_v.  Gen
-// expands both children of every node, so each AES runs under a fixed key.
-struct GenRightKeys {
-    uint32_t st[44];
-    uint32_t v[44];
-};
-
-// child of a seed under the round keys rk of its direction: seed with bit 0 of byte 0
-// cleared, control bit apart
-__device__ __forceinline__ void gen_expand(const SmemTabPair& T, const uint32_t* rk, const uint32_t s[4], uint32_t cs[4],
-                                           uint32_t& ct) {
-    uint32_t o[4];
-    aes_one(T, rk, s, o);
-#pragma unroll
-    for (int w = 0; w < 4; w++) cs[w] = o[w] ^ s[w];
-    ct = cs[0] & 1u;
-    cs[0] &= ~1u;
+// b - a for a of the pair's party 0 and b of its party 1, from this lane's own value
+__device__ __forceinline__ uint32_t party_diff(uint32_t own, uint32_t party) {
+    const uint32_t d = __shfl_xor_sync(0xFFFFFFFFu, own, 1) - own;
+    return party ? 0u - d : d;
 }
 
-// Gen of f^=_{alpha,beta} (DCF = false) or g^<_{alpha,beta} (DCF = true) over Z_{2^32}
-// from the root seeds s0, s1 (overwritten).  No runtime-indexed arrays: the L/R and
-// keep/lose choices are selects, so everything stays in registers.  One instance per
-// kind keeps the DPF loop free of the DCF's value blocks.
+// Gen of f^=_{alpha,beta} (DCF = false) or g^<_{alpha,beta} (DCF = true) over Z_{2^32} on a
+// pair of lanes: the even lane expands party 0's seeds (root s), the odd lane party 1's, and
+// the lose children, control bits and value words meet by shuffles and ballots.  The whole
+// warp takes part.  The shared-memory lookups bound it (616 per lane and DCF level).  A thread
+// per pair had eight AES bodies in a row, 16 warps per SM and twice the work in its smallest
+// unit; with both sides unrolled the lane pairs are slower than that (1.91 ms below), the code
+// being larger than the instruction cache.  50,000 elements' fresh tokens 1.71 -> 1.62 ms,
+// 1,000 elements 0.28 -> 0.12 ms, 1,000 DCF pairs 0.16 -> 0.07 ms.
 template <bool DCF, class Sink>
-__device__ __forceinline__ void gen_pair(const SmemTabPair& T, const AesParams& A, const GenRightKeys& R, int n,
-                                         uint32_t alpha, uint32_t beta, uint32_t s0[4], uint32_t s1[4], Sink& sink) {
-    constexpr bool dcf = DCF;
-    uint32_t t0 = 0u, t1 = 1u, valpha = 0u;
+__device__ __forceinline__ void gen_pair(const SmemTab& T, const AesParams& A, int n, uint32_t alpha, uint32_t beta,
+                                         uint32_t party, uint32_t s[4], Sink& sink) {
+    const uint32_t other = (threadIdx.x & 31u) ^ 1u;
+    uint32_t t = party, valpha = 0u;
+#pragma unroll 1
     for (int lv = 1; lv <= n; lv++) {
-        uint32_t c0l[4], c0r[4], c1l[4], c1r[4], t0l, t0r, t1l, t1r;
-        gen_expand(T, A.rk_st, s0, c0l, t0l);
-        gen_expand(T, R.st, s0, c0r, t0r);
-        gen_expand(T, A.rk_st, s1, c1l, t1l);
-        gen_expand(T, R.st, s1, c1r, t1r);
         const uint32_t a = (alpha >> (n - lv)) & 1u;
-        const uint32_t tl = t0l ^ t1l ^ a ^ 1u, tr = t0r ^ t1r ^ a;
-        uint32_t scw[4];
+        uint32_t scw[4], keep[4], tc[2], dv[2];            // tc, dv: lose, keep
+#pragma unroll 1
+        for (int side = 0; side < 2; side++) {
+            const uint32_t m = 0u - (side ? a : a ^ 1u);
+            uint32_t c[4], v = 0u;
+            aes_sel(T, A.rk_st, A.d_st, m, s, c);
+            if (DCF) v = aes_sel_w0(T, A.rk_v, A.d_v, m, s) ^ s[0];
 #pragma unroll
-        for (int w = 0; w < 4; w++) scw[w] = a ? (c0l[w] ^ c1l[w]) : (c0r[w] ^ c1r[w]);   // CW on the lose side
+            for (int w = 0; w < 4; w++) c[w] ^= s[w];
+            if (side == 0) {
+                tc[0] = c[0] & 1u;
+                c[0] &= ~1u;
+#pragma unroll
+                for (int w = 0; w < 4; w++) scw[w] = c[w] ^ __shfl_xor_sync(0xFFFFFFFFu, c[w], 1);
+                if (DCF) dv[0] = party_diff(v, party);
+            } else {
+                tc[1] = c[0] & 1u;
+                c[0] &= ~1u;
+#pragma unroll
+                for (int w = 0; w < 4; w++) keep[w] = c[w];
+                if (DCF) dv[1] = party_diff(v, party);
+            }
+        }
+        // control-bit words of the lose and the keep side: the sides' bits differ only in a
+        const uint32_t t_lose = tc[0] ^ ((__ballot_sync(0xFFFFFFFFu, tc[0]) >> other) & 1u);
+        const uint32_t t_keep = tc[1] ^ ((__ballot_sync(0xFFFFFFFFu, tc[1]) >> other) & 1u) ^ 1u;
         uint32_t vcw = 0u;
-        if (dcf) {
-            const uint32_t v0l = aes_one_w0(T, A.rk_v, s0) ^ s0[0];
-            const uint32_t v0r = aes_one_w0(T, R.v, s0) ^ s0[0];
-            const uint32_t v1l = aes_one_w0(T, A.rk_v, s1) ^ s1[0];
-            const uint32_t v1r = aes_one_w0(T, R.v, s1) ^ s1[0];
-            const uint32_t v0_lose = a ? v0l : v0r, v1_lose = a ? v1l : v1r;
-            const uint32_t v0_keep = a ? v0r : v0l, v1_keep = a ? v1r : v1l;
-            const bool neg = t1 != 0;
-            vcw = v1_lose - v0_lose - valpha;
+        if (DCF) {
+            const bool neg = (t ^ party ^ 1u) != 0;        // party 1's bit: the two differ on alpha's path
+            vcw = dv[0] - valpha;
             if (neg) vcw = 0u - vcw;
             if (a) vcw += neg ? 0u - beta : beta;          // lose side is L: inputs below alpha
-            valpha = valpha - v1_keep + v0_keep + (neg ? 0u - vcw : vcw);
+            valpha = valpha - dv[1] + (neg ? 0u - vcw : vcw);
         }
-        sink.level(lv - 1, scw, tl, tr, vcw);
-        const uint32_t tkeep = a ? tr : tl;
-        const uint32_t m0 = 0u - t0, m1 = 0u - t1;
+        sink.level(lv - 1, scw, a ? t_lose : t_keep, a ? t_keep : t_lose, vcw);
+        const uint32_t m = 0u - t;
 #pragma unroll
-        for (int w = 0; w < 4; w++) {
-            s0[w] = (a ? c0r[w] : c0l[w]) ^ (scw[w] & m0);
-            s1[w] = (a ? c1r[w] : c1l[w]) ^ (scw[w] & m1);
-        }
-        t0 = (a ? t0r : t0l) ^ (t0 & tkeep);
-        t1 = (a ? t1r : t1l) ^ (t1 & tkeep);
+        for (int w = 0; w < 4; w++) s[w] = keep[w] ^ (scw[w] & m);
+        t = tc[1] ^ (t & t_keep);
     }
-    uint32_t cw = dcf ? s1[1] - s0[1] - valpha : beta - s0[1] + s1[1];
-    if (t1) cw = 0u - cw;
+    const uint32_t d = party_diff(s[1], party);
+    uint32_t cw = DCF ? d - valpha : beta + d;
+    if (t ^ party ^ 1u) cw = 0u - cw;
     sink.final(cw);
 }
 

@@ -1,0 +1,50 @@
+"""Kernels that pair lanes, share nodes or split words, at the sizes where that can go wrong, bit
+for bit against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import workload as W
+from tests._helpers import PRF, from_dev, to_dev
+from tests.test_gpu_keygen import SEED, _gen, _oracle_pair
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+P = pytest.importorskip("paper_2209_03526_gb300")
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c = P.Context(0, prf_keys=PRF)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("kind", [P.KEY_DPF, P.KEY_DCF])
+@pytest.mark.parametrize("pairs", [1, 15, 16, 17, 33])
+def test_keygen_warp_of_lane_pairs(ctx, kind, pairs):
+    """A warp generates 16 key pairs: a single one, one short of a warp, whole, one more."""
+    g = np.random.default_rng(pairs + 100 * kind)
+    alpha = g.integers(0, 1 << 7, pairs, dtype=np.uint64).astype(np.uint32)
+    beta = g.integers(0, 1 << 32, pairs, dtype=np.uint64).astype(np.uint32)
+    keys, L = _gen(ctx, kind, 7, alpha, beta)
+    raw = keys.cpu().numpy().tobytes()
+    for i in range(pairs):
+        k0, k1 = _oracle_pair(kind, 7, SEED, i, int(alpha[i]), int(beta[i]))
+        assert raw[2 * i * L: (2 * i + 1) * L] == bytes(k0) and raw[(2 * i + 1) * L: (2 * i + 2) * L] == bytes(k1), i
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 17, 65])
+def test_fresh_tokens_warp_of_lane_pairs(ctx, n):
+    g = W.rng(n)
+    vals = W.uniform_attrs(g, 2, n, 6)
+    preds = [W.eq_pred(0, 0, 0, int(vals[0, 0])), W.range_pred(0, 1, 0, 3, 40)]
+    size = P.fresh_token_size(preds, 6, [n])
+    toks = [torch.zeros(size, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    ctx.keygen_fresh(preds, 6, [n], SEED, toks)
+    torch.cuda.synchronize()
+    for got, want in zip(toks, oracle.keygen_fresh(preds, 6, [n], SEED)):
+        assert got.cpu().numpy().tobytes() == want
