@@ -58,8 +58,10 @@ struct ShufParams {
     uint32_t half_bits;         // h of the Feistel network
     uint32_t ds, ps, os;
     uint32_t vec_d, vec_s;      // 16-byte accesses fit the input / output rows
-    // secFetch case II: CS1's rows come straight from columns x, (id), attributes
-    const uint32_t* cols[2][kShufMaxWidth];
+    // secFetch case II: the input rows come straight from columns x, (id), attributes, and word 0
+    // of the output rows also goes to columns, which the opening reads
+    const uint32_t* cols[3][kShufMaxWidth];
+    uint32_t* x_out[3];
     uint32_t from_cols;
     MaskPrefix pre[kMaskStreams][kShufMaxWidth / 4];
 };
@@ -194,10 +196,26 @@ __device__ __forceinline__ void store_words(uint32_t* row, uint32_t q, uint32_t 
     }
 }
 
-// CS1 runs over its input rows (two rows of D read in order, one row of X1 written at
-// pi31(pi12(i))); CS2 and CS3 run over their output rows and gather the input row the
-// permutations bring there, so their row writes are in order.  A row's words are read before
-// the AES calls, which then cover the reads.
+// words 4 q .. of row i of share set j of the input; a record is (x, id, attributes), the id c
+// shared as (c, 0, 0)
+__device__ __forceinline__ void load_input(const ShufParams& P, int j, uint64_t i, uint32_t q, uint32_t need,
+                                           uint32_t v[4]) {
+    if (P.from_cols) {
+#pragma unroll
+        for (uint32_t e = 0; e < 4; e++) {
+            const uint32_t w = 4 * q + e;
+            v[e] = w == 1 ? (j == 0 ? (uint32_t)i : 0u) : e < need ? __ldg(P.cols[j][w] + i) : 0u;
+        }
+    } else {
+        load_words(P.d[j] + i * P.ds, q, need, P.vec_d, v);
+    }
+}
+
+// The input rows are read in order and written, padded, at their permuted place: an unaligned
+// or column-wise input never has to be gathered.  (secFetch case II packed CS2's share set into
+// rows for a gather before: 16 us of 409 at 2^20 x 6 words.)  The rows that come from another
+// server are gathered instead, so that those writes are in order.  A row's words are read
+// before the AES calls, which then cover the reads.
 
 // CS1: X1[k] = (D1 + D2 + T12)[i] + T31[j], j = pi12(i), k = pi31(j)
 template <bool FAST>
@@ -214,17 +232,8 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs1(const __grid_const
         for (uint32_t q = 0; q * 4 < W; q++) {
             const uint32_t need = min(4u, W - 4 * q);
             uint32_t a[4], b[4], t12[4], t31[4];
-            if (P.from_cols) {      // record (x, id, attributes); the id c is shared as (c, 0, 0)
-#pragma unroll
-                for (uint32_t e = 0; e < 4; e++) {
-                    const uint32_t w = 4 * q + e;
-                    a[e] = w == 1 ? (uint32_t)i : e < need ? __ldg(P.cols[0][w] + i) : 0u;
-                    b[e] = e < need && w != 1 ? __ldg(P.cols[1][w] + i) : 0u;
-                }
-            } else {
-                load_words(P.d[0] + i * P.ds, q, need, P.vec_d, a);
-                load_words(P.d[1] + i * P.ds, q, need, P.vec_d, b);
-            }
+            load_input(P, 0, i, q, need, a);
+            load_input(P, 1, i, q, need, b);
             mask_words<FAST>(T, P, kT12, i, q, need, t12);
             mask_words<FAST>(T, P, kT31, j, q, need, t31);
 #pragma unroll
@@ -234,7 +243,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs1(const __grid_const
     }
 }
 
-// CS2: items 0..n-1: Y1[j] = D3[i] - T12[i], i = pi12^-1(j);
+// CS2: items 0..n-1: Y1[j] = D3[i] - T12[i], j = pi12(i);
 //      items n..2n-1 (l = item - n): C1[l] = X1[k] + T23[k] - R2[l], k = pi23^-1(l); output R2[l]
 template <bool FAST>
 __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs2(const __grid_constant__ ShufParams P) {
@@ -248,11 +257,11 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs2(const __grid_const
     for (uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; t < 2 * P.n;
          t += (uint64_t)gridDim.x * blockDim.x) {
         if (t < P.n) {
-            const uint64_t j = t, i = p12.inv(j);
+            const uint64_t i = t, j = p12.fwd(i);
             for (uint32_t q = 0; q * 4 < W; q++) {
                 const uint32_t need = min(4u, W - 4 * q);
                 uint32_t a[4], t12[4];
-                load_words(P.d[2] + i * P.ds, q, need, P.vec_d, a);
+                load_input(P, 2, i, q, need, a);
                 mask_words<FAST>(T, P, kT12, i, q, need, t12);
 #pragma unroll
                 for (int e = 0; e < 4; e++) a[e] = op_sub(g, a[e], t12[e]);
@@ -270,6 +279,7 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs2(const __grid_const
                 for (int e = 0; e < 4; e++) a[e] = op_sub(g, op_add(g, a[e], t23[e]), r2[e]);
                 store_words(P.c1 + l * P.ps, q, need, true, a);
                 store_words(P.s[1] + l * P.os, q, need, P.vec_s, r2);
+                if (P.from_cols && q == 0) P.x_out[1][l] = r2[0];
             }
         }
     }
@@ -303,38 +313,22 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs3(const __grid_const
             }
             store_words(P.s[2] + l * P.os, q, need, P.vec_s, a);
             store_words(P.s[0] + l * P.os, q, need, P.vec_s, r1);
+            if (P.from_cols && q == 0) {
+                P.x_out[0][l] = r1[0];
+                P.x_out[2][l] = a[0];
+            }
         }
     }
 }
 
 // ------------------------------------------------------------------ secFetch case II
 
-// CS2's record rows D3 = (x, 0, attributes), padded to 16-byte groups for the gather; CS1 reads
-// its two share sets from their columns directly.
-struct PackParams {
-    const uint32_t* cols[kShufMaxWidth];    // the record's columns, NULL for the id
-    uint32_t* d;
-    uint64_t n;
-    uint32_t groups;                        // 16-byte groups per row
-    uint32_t width;
-};
-
-__global__ void __launch_bounds__(256) k_fetch_pack(const __grid_constant__ PackParams P) {
-    const uint32_t q = blockIdx.y;
-    for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < P.n; c += (uint64_t)gridDim.x * blockDim.x) {
-        uint32_t v[4];
-#pragma unroll
-        for (uint32_t e = 0; e < 4; e++) {
-            const uint32_t w = 4 * q + e;
-            v[e] = w < P.width && P.cols[w] ? __ldg(P.cols[w] + c) : 0u;
-        }
-        reinterpret_cast<uint4*>(P.d)[c * P.groups + q] = make_uint4(v[0], v[1], v[2], v[3]);
-    }
-}
-
 constexpr int kCompactRows = 1024;   // rows per block of the open-and-compact pass
 
+// The opening reads word 0 of the shuffled rows from columns that CS2 and CS3 wrote beside them:
+// 12 bytes a row instead of three rows' sectors, 16.4 + 19.7 us for the two passes before.
 struct CompactParams {
+    const uint32_t* x[3];
     const uint32_t* s[3];
     uint32_t* out[3];
     uint32_t* block_count;      // per block: rows with x^ = 1
@@ -343,7 +337,7 @@ struct CompactParams {
 };
 
 __device__ __forceinline__ bool opened_one(const CompactParams& P, uint64_t l) {
-    return l < P.n && P.s[0][l * P.stride] + P.s[1][l * P.stride] + P.s[2][l * P.stride] == 1u;
+    return l < P.n && P.x[0][l] + P.x[1][l] + P.x[2][l] == 1u;
 }
 
 // open x^ for a block of rows and count the ones
@@ -434,10 +428,12 @@ static MaskPrefix mask_prefix(const uint32_t* rk, uint32_t tag, uint32_t q) {
     return p;
 }
 
-// Rows of the shuffle's input and output, and where CS1's input comes from.
+// Rows of the shuffle's input and output; secFetch case II has input columns instead of rows, and
+// columns for word 0 of the output rows.
 struct ShufRows {
     uint32_t ds, os;                            // row strides in words
-    const uint32_t* const* cols[2];             // CS1's columns (secFetch case II), or NULL
+    const uint32_t* const* cols[3];
+    uint32_t* x_out[3];
 };
 
 // the shuffle on device buffers; scratch from the stream-ordered pool
@@ -468,8 +464,10 @@ oblivgm_status shuffle_device(oblivgm_ctx* ctx, uint32_t group, uint64_t n, uint
     }
     if (rows.cols[0]) {
         P.from_cols = 1;
-        for (int k = 0; k < 2; k++)
+        for (int k = 0; k < 3; k++) {
+            P.x_out[k] = rows.x_out[k];
             for (uint32_t w = 0; w < width; w++) P.cols[k][w] = rows.cols[k][w];
+        }
     }
     uint32_t bits = 0;
     for (uint64_t v = n - 1; v; v >>= 1) bits++;
@@ -547,7 +545,7 @@ extern "C" oblivgm_status oblivgm_shuffle(oblivgm_ctx* ctx, uint32_t group, uint
     }
     const cudaError_t ce = cudaSetDevice(ctx->device);
     if (ce != cudaSuccess) return cuda_fail(ce, "cudaSetDevice");
-    return shuffle_device(ctx, group, n_rows, width, in, seeds, out, ShufRows{width, width, {nullptr, nullptr}},
+    return shuffle_device(ctx, group, n_rows, width, in, seeds, out, ShufRows{width, width, {}, {}},
                           static_cast<cudaStream_t>(stream));
 }
 
@@ -575,7 +573,8 @@ extern "C" oblivgm_status oblivgm_fetch_multi(oblivgm_ctx* ctx, uint32_t table_i
     const uint32_t n_blocks = (uint32_t)((n + kCompactRows - 1) / kCompactRows);
     const uint32_t stride = (W + 3) / 4 * 4;      // rows padded to 16-byte groups
     const size_t tab = ((size_t)n * stride * 4 + 255) & ~size_t(255);
-    const size_t total = 4 * tab + ((size_t)(n_blocks + 1) * 4 + 255);
+    const size_t col = ((size_t)n * 4 + 255) & ~size_t(255);
+    const size_t total = 3 * (tab + col) + ((size_t)(n_blocks + 1) * 4 + 255);
     uint8_t* scratch = nullptr;
     {
         const oblivgm_status as = ws_alloc(ctx, reinterpret_cast<void**>(&scratch), total, s, "fetch scratch");
@@ -583,27 +582,19 @@ extern "C" oblivgm_status oblivgm_fetch_multi(oblivgm_ctx* ctx, uint32_t table_i
     }
     // the records' columns: x, id, attributes
     const uint32_t* cols[3][kShufMaxWidth] = {};
-    uint32_t* sh[3];
+    uint32_t *sh[3], *xs[3];
     for (int j = 0; j < 3; j++) {
-        sh[j] = reinterpret_cast<uint32_t*>(scratch + (1 + j) * tab);
+        sh[j] = reinterpret_cast<uint32_t*>(scratch + j * tab);
+        xs[j] = reinterpret_cast<uint32_t*>(scratch + 3 * tab + j * col);
         cols[j][0] = x[j];
         for (uint32_t a = 0; a < n_attrs; a++)
             cols[j][2 + a] = tb.dev + ((uint64_t)j * tb.n_attrs + attrs[a]) * tb.stride;
     }
-    uint32_t* counts = reinterpret_cast<uint32_t*>(scratch + 4 * tab);
-    PackParams K;
-    std::memset(&K, 0, sizeof K);
-    std::memcpy(K.cols, cols[2], sizeof K.cols);
-    K.d = reinterpret_cast<uint32_t*>(scratch);
-    K.n = n;
-    K.groups = stride / 4;
-    K.width = W;
-    k_fetch_pack<<<dim3((unsigned)std::min<uint64_t>((n + 255) / 256, 8ull * ctx->sm_count), K.groups), 256, 0, s>>>(K);
-    ctx->launches++;
-    const uint32_t* din[3] = {nullptr, nullptr, K.d};
+    uint32_t* counts = reinterpret_cast<uint32_t*>(scratch + 3 * (tab + col));
+    const uint32_t* din[3] = {nullptr, nullptr, nullptr};
     uint32_t* dout[3] = {sh[0], sh[1], sh[2]};
     oblivgm_status st = shuffle_device(ctx, OBLIVGM_SHUFFLE_ADD, n, W, din, seeds, dout,
-                                       ShufRows{stride, stride, {cols[0], cols[1]}}, s);
+                                       ShufRows{stride, stride, {cols[0], cols[1], cols[2]}, {xs[0], xs[1], xs[2]}}, s);
     if (st) {
         cudaFreeAsync(scratch, s);
         return st;
@@ -611,6 +602,7 @@ extern "C" oblivgm_status oblivgm_fetch_multi(oblivgm_ctx* ctx, uint32_t table_i
     CompactParams C;
     std::memset(&C, 0, sizeof C);
     for (int j = 0; j < 3; j++) {
+        C.x[j] = xs[j];
         C.s[j] = sh[j];
         C.out[j] = out[j];
     }

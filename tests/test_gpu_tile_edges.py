@@ -48,3 +48,21 @@ def test_fresh_tokens_warp_of_lane_pairs(ctx, n):
     torch.cuda.synchronize()
     for got, want in zip(toks, oracle.keygen_fresh(preds, 6, [n], SEED)):
         assert got.cpu().numpy().tobytes() == want
+
+
+@pytest.mark.parametrize("n,attrs", [(1, []), (33, [0]), (1025, [1, 0]), (2048, [2, 1, 0]), (515, [0, 1, 2, 0, 1, 2, 0])])
+def test_fetch_multi_record_widths(ctx, n, attrs):
+    """Records of 2, 3, 4, 5 and 9 words (part of a 16-byte group, whole, several), row counts on
+    both sides of an opening block."""
+    g = W.rng(n)
+    vals = W.uniform_attrs(g, 3, n, 16)
+    tab = W.table(vals, 16, g)
+    ctx.load_shares(0, [to_dev(s) for s in tab["shares"]], 16)
+    flags = vals[0] % 3 == 0
+    xs = W.table(flags.astype(np.uint32)[None], 32, g)["shares"]
+    outs = [torch.zeros((n, 1 + len(attrs)), dtype=torch.int32, device="cuda") for _ in range(3)]
+    m = ctx.fetch_multi(0, [to_dev(x[0]) for x in xs], attrs, bytes(range(100, 148)), outs)
+    wm, want = oracle.fetch_multi([x[0] for x in xs], (tab["shares"], 16), attrs, bytes(range(100, 148)), cap=n)
+    assert m == wm == int(flags.sum())
+    for j in range(3):
+        assert np.array_equal(from_dev(outs[j][:m]), want[j])
