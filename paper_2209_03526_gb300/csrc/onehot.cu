@@ -279,17 +279,23 @@ __global__ void __launch_bounds__(512) k_onehot_dots(const __grid_constant__ Dot
     }
 }
 
-// The same pass for rows of W = 128 * warps words (2^12 <= D <= 2^16), persistent (one
-// CTA per SM walks the 32-element words wd = blockIdx.x, + gridDim.x, ...) with the element
-// rows staged through shared memory so that two batches are always in flight while a
-// third is combined, across word boundaries too.  Lane l of warp q owns words
-// [128 q + 4 l, 128 q + 4 l + 4) of every row: it copies them with its own 16-byte
-// cp.async into its own slots and reads back only those, so the pipeline needs no
-// barrier.  A step is one share set and 8 elements; a word's 32 elements and 3 share sets
-// take 12 steps.  The next share set's half-vector slices are loaded into registers
-// during the last step of the current one.
+// The same pass for rows of W = 128 * WARPS words (2^12 <= D <= 2^16), persistent, with the
+// element rows staged through shared memory so that two batches are always in flight while a
+// third is combined, across words too.  Lane l of warp q owns words [128 q + 4 l, 128 q + 4 l + 4)
+// of every row: it copies them with its own 16-byte cp.async into its own slots and reads back
+// only those, so the pipeline needs no barrier.  A CTA takes a run of 16-element halves of output
+// words (a 45th half is 2 % of a CTA's share of 107,614 elements, a 23rd word was 4 %), as
+// chunks of 32 elements; a step is 8 elements of one share set.  Two chunks share the
+// half-vector slices that their share set needs, loaded into registers a few steps ahead.
+// With four predicates the AND / XOR work on the ALU pipe bounds it (4 bytes read are 8 such
+// operations), so everything else is kept off that pipe: a compile-time row length makes a
+// step's addresses immediates, one warp reduction instruction replaces five shuffle / XOR
+// steps, popcounts are placed by multiply-adds.  107,614 elements, n = 16, four predicates:
+// 453 -> 412 us, 6.4 TB/s.  (The binary matrix instruction m16n8k256 would do a step's work
+// in 4 of them, but takes 127 cycles of an SM each: 3.5 times too slow.)
 constexpr int kPipeStages = 3;
-constexpr int kPipeSteps = 3 * (32 / kDotBatch);
+constexpr int kGroupChunks = 2;                       // 32-element chunks per load of the half vectors
+constexpr int kBatches = 32 / kDotBatch;              // steps per (chunk, share set)
 constexpr uint32_t kPipeSmemPerWarp = kPipeStages * kDotBatch * 32 * 16;
 
 __device__ __forceinline__ void load_halves(const DotParams& P, uint32_t W, uint32_t w0, uint32_t np, int j,
@@ -316,143 +322,180 @@ __device__ __forceinline__ uint32_t xor_and(uint32_t acc, uint32_t a, uint32_t b
     return d;
 }
 
-__global__ void __launch_bounds__(512) k_onehot_dots_pipe(const __grid_constant__ DotParams P) {
+// A CTA's steps in order: groups of kGroupChunks chunks, their share sets, their chunks, their
+// batches of kDotBatch elements (a last chunk of one half has two).
+struct DotSteps {
+    uint32_t chunks, last_batches;     // chunks of the CTA; batches of its last one
+    uint32_t group, share, chunk, batch;
+    __device__ __forceinline__ uint32_t group_chunks() const {
+        return min((uint32_t)kGroupChunks, chunks - group * kGroupChunks);
+    }
+    __device__ __forceinline__ uint32_t at() const { return group * kGroupChunks + chunk; }
+    __device__ __forceinline__ uint32_t batches() const { return at() + 1 == chunks ? last_batches : (uint32_t)kBatches; }
+    __device__ __forceinline__ bool done() const { return group * kGroupChunks >= chunks; }
+    __device__ __forceinline__ void next() {
+        if (++batch < batches()) return;
+        batch = 0;
+        if (++chunk < group_chunks()) return;
+        chunk = 0;
+        if (++share < 3) return;
+        share = 0;
+        group++;
+    }
+};
+
+template <int WARPS>
+__global__ void __launch_bounds__(WARPS * 32) k_onehot_dots_pipe(const __grid_constant__ DotParams P) {
     extern __shared__ __align__(16) unsigned char dsmem[];
+    constexpr uint32_t W = 128 * WARPS;
     // 2^i for i < 32 from the launch parameters: a runtime factor, so that shifts into place
     // are multiply-adds on the FMA pipe and leave the ALU pipe to the AND / XOR work
     const uint32_t* pw = P.pow2;
-    __shared__ uint32_t zs[2][16][kDotPreds][3][2];    // by word parity: per warp, masks per (pred, share, half)
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-    const uint32_t W = P.words, np = P.n_preds;
-    const uint64_t nwords = (P.n_elems + 31) / 32;
-    if (blockIdx.x >= nwords) return;
-    const uint64_t my_words = (nwords - 1 - blockIdx.x) / gridDim.x + 1;
-    const uint64_t total = my_words * kPipeSteps;
+    // by group parity: masks per (chunk, share, warp, predicate and half)
+    __shared__ __align__(16) uint32_t zs[2][kGroupChunks][3][WARPS][2 * kDotPreds];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t np = P.n_preds;
+    const uint64_t nwords = (P.n_elems + 31) / 32, halves = 2 * nwords;
+    const uint64_t half0 = blockIdx.x * halves / gridDim.x, half1 = (blockIdx.x + 1) * halves / gridDim.x;
+    if (half0 >= half1) return;
+    const uint32_t mine_halves = (uint32_t)(half1 - half0);
+    DotSteps F{};                                     // the next step to fetch
+    F.chunks = (mine_halves + 1) / 2;
+    F.last_batches = mine_halves % 2 ? kBatches / 2 : kBatches;
     const uint32_t w0 = warp * 128 + lane * 4;
     // slot (stage s, element b) of this lane: mine[(s * kDotBatch + b) * 32]
-    uint4* mine = reinterpret_cast<uint4*>(dsmem + (size_t)warp * kPipeSmemPerWarp) + lane;
-    // step T: word blockIdx.x + (T / 12) gridDim.x, share set (T % 12) / 4, elements 8 (T % 4) ..
-    auto issue = [&](uint64_t T) {
-        const int t = (int)(T % kPipeSteps), st = (int)(T % kPipeStages);
-        const int j = t / (32 / kDotBatch), c0 = (t % (32 / kDotBatch)) * kDotBatch;
-        const uint64_t e0 = (blockIdx.x + (T / kPipeSteps) * gridDim.x) * 32 + c0;
-        uint4* dst = mine + st * kDotBatch * 32;
-        const uint32_t* src = P.share[j] + e0 * W + w0;
-        if (e0 + kDotBatch <= P.n_elems) {
+    uint4* const mine = reinterpret_cast<uint4*>(dsmem + (size_t)warp * kPipeSmemPerWarp) + lane;
+    uint32_t fetch_stage = 0, stage = 0;
+    const auto fetch = [&]() {
+        if (!F.done()) {
+            const uint64_t e0 = half0 * 16 + F.at() * 32u + F.batch * kDotBatch;
+            uint4* dst = mine + fetch_stage * kDotBatch * 32;
+            const uint32_t* src = P.share[F.share] + e0 * W + w0;
+            if (e0 + kDotBatch <= P.n_elems) {
 #pragma unroll
-            for (int b = 0; b < kDotBatch; b++) cp_async16(dst + b * 32, src + (size_t)b * W, 16u);
-        } else {
-            // the table's last word: rows past its end are zero-filled, nothing read
-            const uint32_t* row0 = P.share[j] + (e0 - c0) * W + w0;
+                for (int b = 0; b < kDotBatch; b++) cp_async16(dst + b * 32, src + (size_t)b * W, 16u);
+            } else {
+                // rows past the table's end are zero-filled, nothing read
 #pragma unroll
-            for (int b = 0; b < kDotBatch; b++) {
-                const bool ok = e0 + b < P.n_elems;
-                cp_async16(dst + b * 32, ok ? src + (size_t)b * W : row0, ok ? 16u : 0u);
+                for (int b = 0; b < kDotBatch; b++) {
+                    const bool ok = e0 + b < P.n_elems;
+                    cp_async16(dst + b * 32, ok ? src + (size_t)b * W : P.share[F.share] + w0, ok ? 16u : 0u);
+                }
             }
+            F.next();
         }
-        cp_async_commit();
+        cp_async_commit();                            // an empty group keeps the count uniform
+        fetch_stage = fetch_stage + 1 == kPipeStages ? 0 : fetch_stage + 1;
     };
-    for (int d = 0; d < kPipeStages - 1; d++) {
-        if ((uint64_t)d < total) issue(d);
-        else cp_async_commit();                       // an empty group keeps the count uniform
-    }
+    for (int d = 0; d < kPipeStages - 1; d++) fetch();
     uint32_t h[kDotPreds][2][4], hn[kDotPreds][2][4];
     load_halves(P, W, w0, np, 0, h);
-    constexpr int kBatches = 32 / kDotBatch;          // steps per (word, share set)
+    const uint32_t chunks = F.chunks, last_batches = F.last_batches;
 #pragma unroll 1
-    for (uint64_t T4 = 0; T4 < total; T4 += kBatches) {
-        const int j = (int)((T4 / kBatches) % 3);
-        const uint32_t par = (uint32_t)(T4 / kPipeSteps) & 1u;
-        uint32_t pl[kDotPreds][2];
+    for (uint32_t c0 = 0; c0 < chunks; c0 += kGroupChunks) {
+        const uint32_t nch = min((uint32_t)kGroupChunks, chunks - c0), par = (c0 / kGroupChunks) & 1u;
+#pragma unroll 1
+        for (int j = 0; j < 3; j++) {
+#pragma unroll 1
+            for (uint32_t ch = 0; ch < nch; ch++) {
+                const uint32_t nb = c0 + ch + 1 == chunks ? last_batches : (uint32_t)kBatches;
+                uint32_t pl[kDotPreds][2];
 #pragma unroll
-        for (int k = 0; k < kDotPreds; k++) pl[k][0] = pl[k][1] = 0;
+                for (int k = 0; k < kDotPreds; k++) pl[k][0] = pl[k][1] = 0;
 #pragma unroll
-        for (int cb = 0; cb < kBatches; cb++) {
-            const uint64_t T = T4 + cb;
-            if (T + kPipeStages - 1 < total) issue(T + kPipeStages - 1);
-            else cp_async_commit();
-            cp_async_wait<kPipeStages - 1>();         // this lane's copies of step T have landed
-            if (cb == kBatches - 1) load_halves(P, W, w0, np, j < 2 ? j + 1 : 0, hn);
-            const uint4* slot = mine + (int)(T % kPipeStages) * kDotBatch * 32;
-            uint32_t v[kDotBatch][4];
-#pragma unroll
-            for (int b = 0; b < kDotBatch; b++) {
-                const uint4 x = slot[b * 32];
-                v[b][0] = x.x; v[b][1] = x.y; v[b][2] = x.z; v[b][3] = x.w;
-            }
-#pragma unroll
-            for (int k = 0; k < kDotPreds; k++) {
-                if ((uint32_t)k >= np) break;
-#pragma unroll
-                for (int hh = 0; hh < 2; hh++) {
-                    uint32_t cnt[kDotBatch / 4] = {};
+                for (int cb = 0; cb < kBatches; cb++) {
+                    if (cb >= kBatches / 2 && cb >= (int)nb) break;
+                    fetch();
+                    cp_async_wait<kPipeStages - 1>();     // this lane's copies of the step have landed
+                    if (cb == 1 && ch + 1 == nch) load_halves(P, W, w0, np, j < 2 ? j + 1 : 0, hn);
+                    const uint4* slot = mine + stage * kDotBatch * 32;
+                    stage = stage + 1 == kPipeStages ? 0 : stage + 1;
+                    uint32_t v[kDotBatch][4];
 #pragma unroll
                     for (int b = 0; b < kDotBatch; b++) {
-                        uint32_t a = v[b][0] & h[k][hh][0];
-                        a = xor_and(a, v[b][1], h[k][hh][1]);
-                        a = xor_and(a, v[b][2], h[k][hh][2]);
-                        a = xor_and(a, v[b][3], h[k][hh][3]);
-                        // popcount into byte b % 4 by a multiply-add (the FMA pipe, not the ALU)
-                        cnt[b / 4] = (uint32_t)__popc(a) * pw[8 * (b % 4)] + cnt[b / 4];
+                        const uint4 x = slot[b * 32];
+                        v[b][0] = x.x; v[b][1] = x.y; v[b][2] = x.z; v[b][3] = x.w;
                     }
-                    // bit 8 f + q, q = cb * (kDotBatch / 4) + (b / 4): shifted by a multiply
 #pragma unroll
-                    for (int q = 0; q < kDotBatch / 4; q++) {
-                        constexpr uint32_t M = 0x01010101u;
-                        const int sh = cb * (kDotBatch / 4) + q;
-                        pl[k][hh] = xor_and(pl[k][hh], cnt[q] * pw[sh], M << sh);
+                    for (int k = 0; k < kDotPreds; k++) {
+                        if ((uint32_t)k >= np) break;
+#pragma unroll
+                        for (int hh = 0; hh < 2; hh++) {
+                            uint32_t cnt[kDotBatch / 4] = {};
+#pragma unroll
+                            for (int b = 0; b < kDotBatch; b++) {
+                                uint32_t a = v[b][0] & h[k][hh][0];
+                                a = xor_and(a, v[b][1], h[k][hh][1]);
+                                a = xor_and(a, v[b][2], h[k][hh][2]);
+                                a = xor_and(a, v[b][3], h[k][hh][3]);
+                                // popcount into byte b % 4 by a multiply-add (the FMA pipe, not the ALU)
+                                cnt[b / 4] = (uint32_t)__popc(a) * pw[8 * (b % 4)] + cnt[b / 4];
+                            }
+                            // bit 8 f + q, q = cb * (kDotBatch / 4) + (b / 4): shifted by a multiply
+#pragma unroll
+                            for (int q = 0; q < kDotBatch / 4; q++) {
+                                constexpr uint32_t M = 0x01010101u;
+                                const int sh = cb * (kDotBatch / 4) + q;
+                                pl[k][hh] = xor_and(pl[k][hh], cnt[q] * pw[sh], M << sh);
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < kDotPreds; k++) {
+                    if ((uint32_t)k >= np) break;
+#pragma unroll
+                    for (int hh = 0; hh < 2; hh++) {
+                        const uint32_t m = __reduce_xor_sync(0xFFFFFFFFu, pl[k][hh]);
+                        if (lane == 0) zs[par][ch][j][warp][2 * k + hh] = m;
                     }
                 }
             }
+#pragma unroll
+            for (int k = 0; k < kDotPreds; k++)
+#pragma unroll
+                for (int hh = 0; hh < 2; hh++)
+#pragma unroll
+                    for (int r = 0; r < 4; r++) h[k][hh][r] = hn[k][hh][r];
         }
+        // the group's masks are complete: combine the warps' and write the packed bits, a half
+        // word at a time.  zs is double-buffered by group parity, so one barrier per group suffices.
+        __syncthreads();
+        for (uint32_t t = threadIdx.x; t < nch * np * 3; t += WARPS * 32) {
+            const uint32_t ch = t / (np * 3), k = t / 3 % np, i = t % 3;
+            uint32_t zp = 0;
 #pragma unroll
-        for (int k = 0; k < kDotPreds; k++) {
-            if ((uint32_t)k >= np) break;
+            for (int q = 0; q < WARPS; q++) zp ^= zs[par][ch][i][q][2 * k] ^ zs[par][ch][(i + 1) % 3][q][2 * k + 1];
+            // element c sits at bit 8 (c % 4) + c / 4
+            uint32_t z = 0;
 #pragma unroll
-            for (int hh = 0; hh < 2; hh++) {
-                uint32_t m = pl[k][hh];
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) m ^= __shfl_xor_sync(0xFFFFFFFFu, m, off);
-                if (lane == 0) zs[par][warp][k][j][hh] = m;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < kDotPreds; k++)
-#pragma unroll
-            for (int hh = 0; hh < 2; hh++)
-#pragma unroll
-                for (int r = 0; r < 4; r++) h[k][hh][r] = hn[k][hh][r];
-        if (j == 2) {
-            // the word's masks are complete: combine the warps' and write the packed bits.
-            // zs is double-buffered by word parity, so one barrier per word suffices.
-            __syncthreads();
-            if (threadIdx.x < np * 3) {
-                const uint64_t wd = blockIdx.x + (T4 / kPipeSteps) * gridDim.x;
-                const uint32_t k = threadIdx.x / 3, i = threadIdx.x % 3;
-                uint32_t zp = 0;
-                for (uint32_t q = 0; q < warps; q++) zp ^= zs[par][q][k][i][0] ^ zs[par][q][k][(i + 1) % 3][1];
-                // element c sits at bit 8 (c % 4) + c / 4
-                uint32_t z = 0;
-#pragma unroll
-                for (uint32_t c = 0; c < 32; c++) z |= ((zp >> (8 * (c % 4) + c / 4)) & 1u) << c;
-                P.zbits[k][(uint64_t)i * nwords + wd] = z;
-            }
+            for (uint32_t c = 0; c < 32; c++) z |= ((zp >> (8 * (c % 4) + c / 4)) & 1u) << c;
+            uint16_t* out = reinterpret_cast<uint16_t*>(P.zbits[k] + (uint64_t)i * nwords) + half0 + 2 * (c0 + ch);
+            out[0] = (uint16_t)z;
+            if (c0 + ch + 1 < chunks || last_batches == kBatches) out[1] = (uint16_t)(z >> 16);
         }
     }
     cp_async_wait<0>();
 }
 
+template <int WARPS>
+void launch_dots_pipe(const DotParams& D, uint64_t nwords, int sm_count, cudaStream_t s) {
+    // persistent: as many CTAs as fit on the SMs (one of 16 warps per SM at D = 2^16)
+    constexpr uint32_t smem = WARPS * kPipeSmemPerWarp;
+    const uint32_t per_sm = std::max<uint32_t>(1, std::min<uint32_t>(227u * 1024 / (smem + 4096), 32 / WARPS));
+    const uint64_t grid = std::min<uint64_t>(nwords, (uint64_t)sm_count * per_sm);
+    k_onehot_dots_pipe<WARPS><<<(unsigned)grid, WARPS * 32, smem, s>>>(D);
+}
+
 void launch_dots(const DotParams& D, uint64_t nwords, int sm_count, cudaStream_t s) {
-    if (D.words >= 128 && D.words <= 128 * 16) {
-        // persistent: as many CTAs as fit on the SMs (one of 16 warps per SM at D = 2^16)
-        const uint32_t warps = D.words / 128;
-        const uint32_t per_sm = std::max<uint32_t>(1, std::min<uint32_t>(227u * 1024 / (warps * kPipeSmemPerWarp + 4096), 32 / warps));
-        const uint64_t grid = std::min<uint64_t>(nwords, (uint64_t)sm_count * per_sm);
-        k_onehot_dots_pipe<<<(unsigned)grid, warps * 32, warps * kPipeSmemPerWarp, s>>>(D);
-        return;
+    switch (D.words / 128) {
+        case 1: return launch_dots_pipe<1>(D, nwords, sm_count, s);
+        case 2: return launch_dots_pipe<2>(D, nwords, sm_count, s);
+        case 4: return launch_dots_pipe<4>(D, nwords, sm_count, s);
+        case 8: return launch_dots_pipe<8>(D, nwords, sm_count, s);
+        case 16: return launch_dots_pipe<16>(D, nwords, sm_count, s);
+        default: k_onehot_dots<<<(unsigned)nwords, 32, 0, s>>>(D);      // D < 2^12: one warp's words at most
     }
-    const uint32_t warps = D.words >= 128 ? std::min<uint32_t>(16, D.words / 128) : 1u;
-    k_onehot_dots<<<(unsigned)nwords, warps * 32, 0, s>>>(D);
 }
 
 // All groups of a query in one launch: each element's predicate bits are re-shared in
@@ -815,10 +858,19 @@ extern "C" oblivgm_status oblivgm_filter_onehot(oblivgm_ctx* ctx, uint32_t query
 
 namespace ogm {
 
+template <int WARPS>
+static cudaError_t dots_pipe_attr() {
+    return cudaFuncSetAttribute(k_onehot_dots_pipe<WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                WARPS * (int)kPipeSmemPerWarp);
+}
+
 oblivgm_status set_onehot_attrs() {
     cudaError_t e = cudaFuncSetAttribute(k_onehot_evalall_et, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_onehot_dots_pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * kPipeSmemPerWarp);
+    if (e == cudaSuccess) e = dots_pipe_attr<1>();
+    if (e == cudaSuccess) e = dots_pipe_attr<2>();
+    if (e == cudaSuccess) e = dots_pipe_attr<4>();
+    if (e == cudaSuccess) e = dots_pipe_attr<8>();
+    if (e == cudaSuccess) e = dots_pipe_attr<16>();
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_onehot_fold, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
     return e == cudaSuccess ? OBLIVGM_OK : cuda_fail(e, "one-hot kernel attributes");

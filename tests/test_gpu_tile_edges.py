@@ -50,6 +50,28 @@ def test_fresh_tokens_warp_of_lane_pairs(ctx, n):
         assert got.cpu().numpy().tobytes() == want
 
 
+@pytest.mark.parametrize("n,n_elems,n_preds", [(12, 1, 1), (13, 16, 2), (14, 17, 5), (15, 48, 3), (16, 331, 4)])
+def test_onehot_halves_of_words(ctx, n, n_elems, n_preds):
+    """Every width of the staged dot pass, CTAs with one half of an output word, tables that end
+    inside either half."""
+    g = W.rng(n)
+    vals = W.uniform_attrs(g, 1, n_elems, n)
+    tab = W.onehot_table(vals, n, g)
+    ctx.load_onehot(0, [to_dev(s) for s in tab["shares"]], n)
+    preds = [W.eq_pred(0, 0, p, int(vals[0, p % n_elems])) for p in range(n_preds)]
+    toks = P.keygen_onehot(preds, n, bytes([n]) * 16)
+    outs = [[torch.full(((n_elems + 31) // 32,), -1, dtype=torch.int32, device="cuda") for _ in range(3)] for _ in preds]
+    ctx.filter_onehot(3, toks, outs)
+    ctx.sync()
+    for grp in (0, n_preds - 1):
+        words = np.stack([from_dev(t) for t in outs[grp]])
+        got = ((words[:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(3, -1)
+        idx = np.arange(n_elems) if n < 15 else np.unique([0, n_elems // 2, n_elems - 1])
+        assert np.array_equal(got[:, idx], oracle.filter_onehot(toks, 3, PRF, [(tab["shares"], n)], grp, idx))
+        assert np.array_equal(oracle.reconstruct_bits(got[:, :n_elems]), oracle.plain_group([preds[grp]], grp, vals))
+        assert not got[:, n_elems:].any()
+
+
 @pytest.mark.parametrize("n,attrs", [(1, []), (33, [0]), (1025, [1, 0]), (2048, [2, 1, 0]), (515, [0, 1, 2, 0, 1, 2, 0])])
 def test_fetch_multi_record_widths(ctx, n, attrs):
     """Records of 2, 3, 4, 5 and 9 words (part of a 16-byte group, whole, several), row counts on
