@@ -338,6 +338,12 @@ namespace ogm {
 // as in k_filter; the walks' outputs meet in shared memory, and the element's first slot
 // thread sums them per server, re-shares and folds exactly as k_filter does.
 
+//
+// The elements of a tile pass through the same nodes near the root, so the first levels visit
+// nodes instead: while a level has at most as many nodes as the tile has elements, each node's
+// step is made once per key, from the parent's state in shared memory, four or five levels of
+// the usual tiles.  Path query on 1,000 / 4,000 elements, n = 16: 41.0 -> 39.0 us.
+
 constexpr int kWpSlots = 12;                          // key walks per element
 constexpr int kWpElems = 40;                          // elements per CTA (tile)
 constexpr int kWpWalks = kWpSlots * kWpElems;         // 480 seed threads, then 480 value threads
@@ -347,7 +353,7 @@ constexpr int kWpThreads = 2 * kWpWalks;              // 960
 static_assert(kWpWalks % 32 == 0 && kWpWalks / 32 <= 15, "one named barrier (1..15) per walk pair of warps");
 constexpr int kWpPrf = 6;                             // re-share PRF words per element: 2 passes x 3 keys
 constexpr int kWpResidentOff = kFilterSmem + (kWpWalks + kWpEqElems * kWpPrf) * 4 +   // walk outputs, PRF words
-                               2 * kWpWalks * 16 + 2 * kWpWalks * 4 + kWpWalks * 4; // seed / control-bit hand-over, V
+                               2 * kWpWalks * 16 + 2 * kWpWalks * 4 + 2 * kWpWalks * 4; // seed / control-bit hand-over, V
 constexpr int kWpResidentBytes = 48 * 1024;   // descriptors, keys and tile offsets of a small launch
 constexpr int kWpSmem = kWpResidentOff + kWpResidentBytes;
 static_assert(kWpResidentOff % 16 == 0, "bulk copies need 16-byte aligned destinations");
@@ -355,6 +361,14 @@ static_assert(kWpResidentOff % 16 == 0, "bulk copies need 16-byte aligned destin
 constexpr uint64_t kWpDefaultElemsPerSm = 128;
 // launches of at most this many groups get a tile width per group (walk-parallel kernel)
 constexpr size_t kWpTileGroups = 4;
+
+// levels below the root whose nodes a tile of `elems` elements shares: as many as have at most
+// that many nodes
+__host__ __device__ inline int wp_shared_levels(uint32_t elems, int n) {
+    int top = 0;
+    while (top < n && (2u << top) <= elems) top++;
+    return top;
+}
 
 // The seed warp w (< 15) and the value warp 15 + w of a walk pair meet at named barrier
 // 1 + w (64 threads): the per-level hand-over needs only the two of them, so pairs do not
@@ -371,7 +385,7 @@ __global__ void __launch_bounds__(kWpThreads, 1) k_filter_wp(const __grid_consta
     uint32_t* fprf = part + kWpWalks;                                      // [element][pass * 3 + key]
     uint4* sbuf = reinterpret_cast<uint4*>(fprf + kWpEqElems * kWpPrf);    // [2][walk]: s_i
     uint32_t* tbuf = reinterpret_cast<uint32_t*>(sbuf + 2 * kWpWalks);     // [2][walk]: t_i
-    uint32_t* vbuf = tbuf + 2 * kWpWalks;                                  // [walk]: the value sum V
+    uint32_t* vbuf = tbuf + 2 * kWpWalks;                                  // [2][walk]: the value sum V
     unsigned char* wsm = smem + kWpResidentOff;                            // resident copy of the workspace
     __shared__ __align__(8) uint64_t mbar;
     __shared__ unsigned long long item_sh;
@@ -427,7 +441,7 @@ __global__ void __launch_bounds__(kWpThreads, 1) k_filter_wp(const __grid_consta
         const GroupDesc& G = groups[lo];
         const uint32_t tile = G.tile, sw = G.slots;   // elements per item, walk threads per element
         const uint32_t el = walk / sw, slot = walk % sw;
-        const uint64_t e = (item - item_start[lo]) * tile + el;
+        const uint64_t e_first = (item - item_start[lo]) * tile, e = e_first + el;
         const uint64_t n_elems = G.n_elems;
         const bool valid = el < tile && e < n_elems;
         const uint32_t table = G.table_id, query = G.query_id;
@@ -472,16 +486,65 @@ __global__ void __launch_bounds__(kWpThreads, 1) k_filter_wp(const __grid_consta
             const int n = (int)D.n_bits;
             const uint32_t party = K.party;
             uint32_t s[4] = {0, 0, 0, 0}, t = party, V = 0;
-            if (active && !value_thread) {
-#pragma unroll
-                for (int w = 0; w < 4; w++) s[w] = K.seed[w];
-                if (!eq) {
-                    sbuf[walk] = make_uint4(s[0], s[1], s[2], s[3]);
-                    tbuf[walk] = t;
+            // the shared levels 0 .. top - 1: node v of level l and key k at slot nk * v + k of the
+            // buffers of parity l
+            const uint32_t nk = 6 * nsub, kk = walk % nk, node = walk / nk;
+            const int top = wp_shared_levels((uint32_t)min((unsigned long long)tile, (unsigned long long)(n_elems - e_first)), n);
+            if (top > 0) {
+                const DevKey& N = pkeys[kk];
+                if (walk < nk) {
+                    if (!value_thread) {
+                        sbuf[walk] = *reinterpret_cast<const uint4*>(N.seed);
+                        tbuf[walk] = N.party;
+                    } else {
+                        vbuf[walk] = 0u;
+                    }
+                }
+                __syncthreads();
+                for (int i = 0; i < top; i++) {
+                    if (node < (2u << i)) {
+                        const uint32_t at = (i & 1) * kWpWalks + (node >> 1) * nk + kk, to = ((i + 1) & 1) * kWpWalks + walk;
+                        const uint4 sp = sbuf[at];
+                        const uint32_t dir = node & 1u, m = 0u - dir, tp = tbuf[at];
+                        const uint32_t sv[4] = {sp.x, sp.y, sp.z, sp.w};
+                        if (!value_thread) {
+                            uint32_t o[4];
+                            aes_sel(T, P.aes.rk_st, P.aes.d_st, m, sv, o);
+                            const uint4 cw = *reinterpret_cast<const uint4*>(N.scw[i]);
+                            const uint32_t tm = 0u - tp;
+                            const uint32_t c0 = o[0] ^ sp.x;
+                            sbuf[to] = make_uint4((c0 & ~1u) ^ (cw.x & tm), o[1] ^ sp.y ^ (cw.y & tm),
+                                                  o[2] ^ sp.z ^ (cw.z & tm), o[3] ^ sp.w ^ (cw.w & tm));
+                            tbuf[to] = (c0 & 1u) ^ (tp & (((dir ? N.tr : N.tl) >> i) & 1u));
+                        } else if (!eq) {
+                            const uint32_t v0 = aes_sel_w0(T, P.aes.rk_v, P.aes.d_v, m, sv);
+                            const uint32_t term = (v0 ^ sp.x) + (tp ? N.vcw[i] : 0u);
+                            vbuf[to] = vbuf[at] + (N.party ? 0u - term : term);
+                        }
+                    }
+                    __syncthreads();
                 }
             }
+            if (active && top > 0) {
+                const uint32_t at = (top & 1) * kWpWalks + (xh >> (n - top)) * nk + slot;
+                if (!value_thread) {
+                    const uint4 sp = sbuf[at];
+                    s[0] = sp.x; s[1] = sp.y; s[2] = sp.z; s[3] = sp.w;
+                    t = tbuf[at];
+                } else if (!eq) {
+                    V = vbuf[at];
+                }
+            } else if (active && !value_thread) {
+#pragma unroll
+                for (int w = 0; w < 4; w++) s[w] = K.seed[w];
+            }
+            if (top > 0) __syncthreads();                  // the nodes are read before the hand-over takes their place
+            if (active && !value_thread && !eq) {
+                sbuf[(top & 1) * kWpWalks + walk] = make_uint4(s[0], s[1], s[2], s[3]);
+                tbuf[(top & 1) * kWpWalks + walk] = t;
+            }
             if (!eq) wp_pair_sync(walk);
-            for (int i = 0; i < n; i++) {
+            for (int i = top; i < n; i++) {
                 const uint32_t dir = (xh >> (n - 1 - i)) & 1u;
                 const uint32_t m = 0u - dir;
                 if (active && !value_thread) {
@@ -776,12 +839,13 @@ void choose_group_tiles(size_t n_groups, NF n_elems_of, TF item_time, MF max_til
 //  about two warps per SM the walks' own latency, not the shared-memory pipe, sets it.
 //  k_filter_wp: one thread per walk (two per DCF walk); per predicate of n bits a fixed
 //  cost (the key staging, the walk chain of one PRG call per level, the combine: about
-//  656 n ns for EQ, 719 n ns for RANGE on GB300) plus a per-element term (20 n / 54 n ns:
-//  the shared-memory lookups of an EQ / RANGE element).  Fitted to sweeps of tiles of 1..40
-//  elements, one and two items per SM, n = 16 and 32.
+//  656 n ns for EQ, 719 n ns for RANGE on GB300) plus a term per level and element, or node
+//  in the shared levels (20 / 54 ns: the shared-memory lookups of an EQ / RANGE element).
+//  Fitted to sweeps of tiles of 1..40 elements, one and two items per SM, n = 16 and 32.
 struct GroupCost {
     uint64_t walk_cost = 0;            // k_filter: sum over predicates of 6 n (EQ) / 24 n (RANGE)
     uint64_t wp_lat = 0, wp_slope = 0; // k_filter_wp: latency and per-element terms, ns
+    int n_bits = 1;
 };
 
 double filter_item_time(const GroupCost& c, uint64_t width) {
@@ -790,7 +854,10 @@ double filter_item_time(const GroupCost& c, uint64_t width) {
 }
 
 double wp_item_time(const GroupCost& c, uint64_t width) {
-    return (double)c.wp_lat + (double)c.wp_slope * (double)width;
+    // nodes of the shared levels, elements of the others
+    const int top = wp_shared_levels((uint32_t)width, c.n_bits);
+    const double per_level = (double)(2u << top) - 2.0 + (double)(c.n_bits - top) * (double)width;
+    return (double)c.wp_lat + (double)c.wp_slope / c.n_bits * per_level;
 }
 
 oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_queries, const uint32_t* query_ids,
@@ -823,6 +890,7 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
                 cost.walk_cost += (eq ? 6ull : 24ull) * p->n;
                 cost.wp_lat += (eq ? 656ull : 719ull) * p->n;
                 cost.wp_slope += (eq ? 20ull : 54ull) * p->n;
+                cost.n_bits = (int)p->n;
             }
             G gr{};
             for (int j = 0; j < 3; j++) {

@@ -50,6 +50,33 @@ def test_fresh_tokens_warp_of_lane_pairs(ctx, n):
         assert got.cpu().numpy().tobytes() == want
 
 
+@pytest.mark.parametrize("bits", [1, 3, 9, 32])
+@pytest.mark.parametrize("tile", [1, 2, 31, 32, 33, 40])
+def test_walk_parallel_shared_levels(ctx, bits, tile):
+    """Tiles on both sides of a level of nodes, domains smaller than a tile (every level is shared)
+    and ragged last tiles; a group of equality predicates, one of both kinds."""
+    g = W.rng(bits * 64 + tile)
+    n = 3 * tile + max(1, tile // 3)
+    vals = W.uniform_attrs(g, 2, n, bits)
+    tab = W.table(vals, bits, g)
+    ctx.load_shares(0, [to_dev(s) for s in tab["shares"]], bits)
+    top = (1 << bits) - 1
+    preds = [W.eq_pred(0, 0, 0, int(vals[0, 0])), W.range_pred(0, 1, 1, top // 3, top),
+             W.eq_pred(0, 0, 1, int(vals[0, -1]), W.COMBINE_OR), W.eq_pred(0, 1, 0, int(vals[1, 0]))]
+    toks = P.keygen(preds, bits, bytes(range(3, 19)))
+    prev, prev_tile = ctx.set_walk_parallel((1 << 64) - 1), ctx.set_walk_parallel_tile(tile)
+    try:
+        outs = [[torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(3)] for _ in range(2)]
+        ctx.filter_and_combine(9, toks, outs)
+        ctx.sync()
+    finally:
+        ctx.set_walk_parallel(prev)
+        ctx.set_walk_parallel_tile(prev_tile)
+    for grp in range(2):
+        got = np.stack([from_dev(t) for t in outs[grp]])
+        assert np.array_equal(got, oracle.filter_group(toks, 9, PRF, [(tab["shares"], bits)], grp, np.arange(n), threads=4))
+
+
 @pytest.mark.parametrize("n,n_elems,n_preds", [(12, 1, 1), (13, 16, 2), (14, 17, 5), (15, 48, 3), (16, 331, 4)])
 def test_onehot_halves_of_words(ctx, n, n_elems, n_preds):
     """Every width of the staged dot pass, CTAs with one half of an output word, tables that end
