@@ -270,6 +270,14 @@ oblivgm_status oblivgm_release(oblivgm_ctx* ctx, uint64_t ticket) {
         for (auto& kv : q->tables) S.table_refs[kv.first]--;
     }
     cudaSetDevice(ctx->device);
+    // Work that the caller queued on the default stream before this call (a copy of the result) may
+    // not have run yet, while the next batch on the serve stream could already reuse the memory:
+    // the release waits for it on the device.
+    cudaEvent_t read = nullptr;
+    if (cudaEventCreateWithFlags(&read, cudaEventDisableTiming) == cudaSuccess) {
+        if (cudaEventRecord(read, cudaStreamLegacy) == cudaSuccess) cudaStreamWaitEvent(S.streams[q->stream], read, 0);
+        cudaEventDestroy(read);
+    }
     for (uint32_t* p : q->outs)
         if (p) cudaFreeAsync(p, S.streams[q->stream]);
     S.cv_work.notify_all();
