@@ -28,17 +28,20 @@ __device__ __forceinline__ uint32_t lane_offset() { return (threadIdx.x & 31u) *
 // Fill the replicated tables from the compact Te0 (256 words in global memory).  Each of
 // the 1,024 (table, entry) pairs is one word replicated for the 32 lanes (128 bytes): eight
 // threads write a pair with one 16-byte store each, so a warp's store covers four whole
-// 128-byte rows (four wavefronts, no bank conflict).
+// 128-byte rows (four wavefronts, no bank conflict).  A thread reads an entry once for its four
+// tables, and its reads (two or three) are under way together.
 template <bool PAIR = false>
 __device__ __forceinline__ void fill_tables(uint32_t* tab, const uint32_t* __restrict__ te0) {
 #pragma unroll 4
-    for (int i = threadIdx.x; i < 4 * 256 * 8; i += blockDim.x) {
-        const int pair = i >> 3, chunk = i & 7;
-        const int k = pair >> 8, idx = pair & 255;
+    for (int i = threadIdx.x; i < 256 * 8; i += blockDim.x) {
+        const int idx = i >> 3, chunk = i & 7;
         const uint32_t w = __ldg(te0 + idx);
-        const uint32_t v = __funnelshift_l(w, w, 8 * k);
-        uint32_t* row = PAIR ? tab + (k >> 1) * 16384 + idx * 64 + (k & 1) * 32 : tab + k * 8192 + idx * 32;
-        reinterpret_cast<uint4*>(row)[chunk] = make_uint4(v, v, v, v);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const uint32_t v = __funnelshift_l(w, w, 8 * k);
+            uint32_t* row = PAIR ? tab + (k >> 1) * 16384 + idx * 64 + (k & 1) * 32 : tab + k * 8192 + idx * 32;
+            reinterpret_cast<uint4*>(row)[chunk] = make_uint4(v, v, v, v);
+        }
     }
 }
 

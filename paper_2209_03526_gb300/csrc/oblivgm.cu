@@ -345,18 +345,26 @@ namespace ogm {
 // the usual tiles.  Path query on 1,000 / 4,000 elements, n = 16: 41.0 -> 39.0 us.
 
 constexpr int kWpSlots = 12;                          // key walks per element
-constexpr int kWpElems = 40;                          // elements per CTA (tile)
-constexpr int kWpWalks = kWpSlots * kWpElems;         // 480 seed threads, then 480 value threads
 constexpr int kWpEqSlots = 6;                         // walk threads per element of a group of equality predicates
-constexpr int kWpEqElems = kWpWalks / kWpEqSlots;     // such a group's tile: up to 80 elements
-constexpr int kWpThreads = 2 * kWpWalks;              // 960
-static_assert(kWpWalks % 32 == 0 && kWpWalks / 32 <= 15, "one named barrier (1..15) per walk pair of warps");
 constexpr int kWpPrf = 6;                             // re-share PRF words per element: 2 passes x 3 keys
-constexpr int kWpResidentOff = kFilterSmem + (kWpWalks + kWpEqElems * kWpPrf) * 4 +   // walk outputs, PRF words
-                               2 * kWpWalks * 16 + 2 * kWpWalks * 4 + 2 * kWpWalks * 4; // seed / control-bit hand-over, V
-constexpr int kWpResidentBytes = 48 * 1024;   // descriptors, keys and tile offsets of a small launch
-constexpr int kWpSmem = kWpResidentOff + kWpResidentBytes;
-static_assert(kWpResidentOff % 16 == 0, "bulk copies need 16-byte aligned destinations");
+constexpr int kWpResidentBytes = 48 * 1024;           // descriptors, keys and tile offsets of a small launch
+// Elements per CTA (tile): 32 leave a thread 80 registers, which take a level's lookups with
+// fewer waits than the 64 that 40 leave (path query 39.3 -> 37.5 us), and 24 to 32 elements
+// take the same time, three warp pairs per SM sub-partition.  Tiles of 33 to 40 are for launches
+// of fewer waves with them, and for oblivgm_set_walk_parallel_tile.
+constexpr int kWpElems = 32, kWpMaxElems = 40;
+
+template <int ELEMS>
+struct WpShape {
+    static constexpr int kWalks = kWpSlots * ELEMS;           // seed threads, then as many value threads
+    static constexpr int kEqElems = kWalks / kWpEqSlots;      // tile of a group of equality predicates only
+    static constexpr int kThreads = 2 * kWalks;
+    static constexpr int kResidentOff = kFilterSmem + (kWalks + kEqElems * kWpPrf) * 4 +   // walk outputs, PRF words
+                                        2 * kWalks * 16 + 2 * kWalks * 4 + 2 * kWalks * 4; // seed / control-bit hand-over, V
+    static constexpr int kSmem = kResidentOff + kWpResidentBytes;
+    static_assert(kWalks % 32 == 0 && kWalks / 32 <= 15, "one named barrier (1..15) per walk pair of warps");
+    static_assert(kResidentOff % 16 == 0, "bulk copies need 16-byte aligned destinations");
+};
 // default switch-over: batches of at most this many elements per SM in all
 constexpr uint64_t kWpDefaultElemsPerSm = 128;
 // launches of at most this many groups get a tile width per group (walk-parallel kernel)
@@ -370,14 +378,16 @@ __host__ __device__ inline int wp_shared_levels(uint32_t elems, int n) {
     return top;
 }
 
-// The seed warp w (< 15) and the value warp 15 + w of a walk pair meet at named barrier
+// The seed warp w and the value warp kWalks / 32 + w of a walk pair meet at named barrier
 // 1 + w (64 threads): the per-level hand-over needs only the two of them, so pairs do not
 // wait for one another and drift apart, which keeps the lookup and logic pipes busy.
 __device__ __forceinline__ void wp_pair_sync(uint32_t walk) {
     asm volatile("bar.sync %0, 64;" ::"r"(1u + walk / 32u) : "memory");
 }
 
-__global__ void __launch_bounds__(kWpThreads, 1) k_filter_wp(const __grid_constant__ FilterParams P) {
+template <int ELEMS>
+__global__ void __launch_bounds__(WpShape<ELEMS>::kThreads, 1) k_filter_wp(const __grid_constant__ FilterParams P) {
+    constexpr int kWpWalks = WpShape<ELEMS>::kWalks, kWpEqElems = WpShape<ELEMS>::kEqElems;
     extern __shared__ __align__(128) unsigned char smem[];
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
     DevKey* kbuf = reinterpret_cast<DevKey*>(smem + kTableBytes);
@@ -386,7 +396,7 @@ __global__ void __launch_bounds__(kWpThreads, 1) k_filter_wp(const __grid_consta
     uint4* sbuf = reinterpret_cast<uint4*>(fprf + kWpEqElems * kWpPrf);    // [2][walk]: s_i
     uint32_t* tbuf = reinterpret_cast<uint32_t*>(sbuf + 2 * kWpWalks);     // [2][walk]: t_i
     uint32_t* vbuf = tbuf + 2 * kWpWalks;                                  // [2][walk]: the value sum V
-    unsigned char* wsm = smem + kWpResidentOff;                            // resident copy of the workspace
+    unsigned char* wsm = smem + WpShape<ELEMS>::kResidentOff;                            // resident copy of the workspace
     __shared__ __align__(8) uint64_t mbar;
     __shared__ unsigned long long item_sh;
 
@@ -427,8 +437,11 @@ __global__ void __launch_bounds__(kWpThreads, 1) k_filter_wp(const __grid_consta
     const uint32_t walk = threadIdx.x % kWpWalks;
     const uint64_t n_items = failed ? 0 : item_start[P.n_groups];
     // the first item of CTA b is item b (the grid has at most n_items CTAs); later ones come
-    // from the work counter, past the first gridDim.x
+    // from the work counter, past the first gridDim.x.  A launch of one wave needs neither the
+    // counter nor its reset, two round trips to memory at the end.
+    const bool one_wave = n_items <= gridDim.x;
     for (uint32_t round = 0;; round++) {
+        if (one_wave && round > 0) return;
         if (threadIdx.x == 0) item_sh = round == 0 ? blockIdx.x : gridDim.x + atomicAdd(P.counter, 1ull);
         __syncthreads();
         const uint64_t item = item_sh;
@@ -923,24 +936,47 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
     for (const G& g : all) total += g.d.n_elems;
     const bool wp = plan->wp = total != 0 && total <= ctx->wp_max_elems;
     plan->elems_per_thread = wp ? 1 : ctx->elems_per_thread;
-    plan->threads = wp ? kWpThreads : ctx->threads;
     const int sm_count = ctx->sm_count;
-    const uint32_t max_tile = !wp ? ctx->threads * ctx->elems_per_thread : ctx->wp_tile ? ctx->wp_tile : kWpElems;
     const uint32_t step = !wp ? 32 * ctx->elems_per_thread : ctx->wp_tile ? 0 : 1;
     const auto n_of = [&](size_t i) { return all[i].d.n_elems; };
     const auto time_of = [&](size_t i, uint64_t w) {
         return wp ? wp_item_time(all[i].cost, w) : filter_item_time(all[i].cost, w);
     };
-    const uint32_t tile = choose_tile(all.size(), n_of, time_of, max_tile, step, sm_count);
-    std::vector<uint32_t> tiles(all.size(), tile);
-    if (wp && step != 0 && all.size() > 1 && all.size() <= kWpTileGroups) {
-        uint64_t items_at_max = 0;
-        for (const G& g : all) items_at_max += (g.d.n_elems + max_tile - 1) / max_tile;
-        if (items_at_max <= 4ull * (uint64_t)sm_count)
+    // items at the widest tiles; with a width per group those of equality predicates take twice as many elements
+    const bool group_tiles = wp && step != 0 && all.size() > 1 && all.size() <= kWpTileGroups;
+    const auto items_of = [&](uint32_t width, uint32_t eq_width) {
+        uint64_t items = 0;
+        for (const G& g : all) {
+            const uint32_t w = g.d.slots == (uint32_t)kWpEqSlots ? eq_width : width;
+            items += (g.d.n_elems + w - 1) / w;
+        }
+        return items;
+    };
+    const auto tiles_of = [&](uint32_t max_tile) {
+        std::vector<uint32_t> tiles(all.size(), choose_tile(all.size(), n_of, time_of, max_tile, step, sm_count));
+        if (group_tiles && items_of(max_tile, max_tile) <= 4ull * (uint64_t)sm_count)
             choose_group_tiles(all.size(), n_of, time_of,
-                               [&](size_t i) { return all[i].d.slots == (uint32_t)kWpEqSlots ? (uint32_t)kWpEqElems : max_tile; },
+                               [&](size_t i) { return all[i].d.slots == (uint32_t)kWpEqSlots ? 2 * max_tile : max_tile; },
                                sm_count, tiles);
+        return tiles;
+    };
+    const uint32_t max_tile = !wp ? ctx->threads * ctx->elems_per_thread : ctx->wp_tile ? ctx->wp_tile : (uint32_t)kWpElems;
+    std::vector<uint32_t> tiles = tiles_of(max_tile);
+    bool wp_wide = wp && max_tile > (uint32_t)kWpElems;
+    if (wp && step != 0 && items_of(kWpElems, group_tiles ? 2 * kWpElems : kWpElems) > (uint64_t)sm_count) {
+        // more than one wave of 32-element tiles: 40-element ones, 6 % slower otherwise, where they
+        // take fewer waves (5,000 elements, n = 32, EQ AND RANGE: 134 us against 166)
+        std::vector<uint32_t> wide = tiles_of(kWpMaxElems);
+        std::vector<CtaClass> finish;
+        const auto makespan = [&](const std::vector<uint32_t>& t) {
+            return simulate_makespan(all.size(), n_of, [&](size_t g) { return (uint64_t)t[g]; }, time_of, sm_count, finish);
+        };
+        if (1.06 * makespan(wide) < makespan(tiles)) {
+            tiles = std::move(wide);
+            wp_wide = true;
+        }
     }
+    plan->threads = !wp ? ctx->threads : (uint32_t)(wp_wide ? WpShape<kWpMaxElems>::kThreads : WpShape<kWpElems>::kThreads);
     plan->groups.clear(); plan->preds.clear(); plan->keys.clear(); plan->item_start.clear();
     plan->tile = *std::max_element(tiles.begin(), tiles.end());
     uint64_t items = 0;
@@ -990,7 +1026,10 @@ cudaError_t launch_filter_kernel(const FilterParams& P, uint64_t n_items, int sm
                                  bool wp, cudaStream_t st) {
     const unsigned grid = (unsigned)std::min<uint64_t>(n_items, (uint64_t)sm_count);
     if (wp) {
-        k_filter_wp<<<grid, kWpThreads, kWpSmem, st>>>(P);
+        if (threads == (uint32_t)WpShape<kWpElems>::kThreads)
+            k_filter_wp<kWpElems><<<grid, threads, WpShape<kWpElems>::kSmem, st>>>(P);
+        else
+            k_filter_wp<kWpMaxElems><<<grid, WpShape<kWpMaxElems>::kThreads, WpShape<kWpMaxElems>::kSmem, st>>>(P);
     } else {
         switch (E) {
             case 1: k_filter<1><<<grid, threads, kFilterSmem, st>>>(P); break;
@@ -1125,7 +1164,10 @@ oblivgm_status set_filter_attrs() {
     OGM_CUDA(cudaFuncSetAttribute(k_filter<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFilterSmem), "smem attr");
     OGM_CUDA(cudaFuncSetAttribute(k_filter<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFilterSmem), "smem attr");
     OGM_CUDA(cudaFuncSetAttribute(k_filter<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kFilterSmem), "smem attr");
-    OGM_CUDA(cudaFuncSetAttribute(k_filter_wp, cudaFuncAttributeMaxDynamicSharedMemorySize, kWpSmem), "smem attr");
+    OGM_CUDA(cudaFuncSetAttribute(k_filter_wp<kWpElems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  WpShape<kWpElems>::kSmem), "smem attr");
+    OGM_CUDA(cudaFuncSetAttribute(k_filter_wp<kWpMaxElems>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  WpShape<kWpMaxElems>::kSmem), "smem attr");
     OGM_CUDA(cudaFuncSetAttribute(k_eval_raw<OBLIVGM_KEY_DPF>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes), "smem attr");
     OGM_CUDA(cudaFuncSetAttribute(k_eval_raw<OBLIVGM_KEY_DCF>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes), "smem attr");
     return OBLIVGM_OK;
@@ -1540,7 +1582,7 @@ oblivgm_status oblivgm_set_schedule(oblivgm_ctx* ctx, uint32_t threads, uint32_t
 oblivgm_status oblivgm_set_walk_parallel_tile(oblivgm_ctx* ctx, uint32_t tile, uint32_t* previous) {
     oblivgm_status st = check_ctx(ctx);
     if (st) return st;
-    if (tile > (uint32_t)kWpElems) return fail(OBLIVGM_EINVAL, "the walk-parallel tile is at most 40 elements");
+    if (tile > (uint32_t)kWpMaxElems) return fail(OBLIVGM_EINVAL, "the walk-parallel tile is at most 40 elements");
     if (previous) *previous = ctx->wp_tile;
     ctx->wp_tile = tile;
     return OBLIVGM_OK;
