@@ -28,6 +28,7 @@
 #include "gen_device.cuh"
 #include "host_crypto.h"
 #include "oblivgm.h"
+#include "ptx_async.cuh"
 #include "runtime.h"
 #include "staged.h"
 
@@ -283,6 +284,7 @@ struct FreshWalkParams {
 // 1.91 -> 0.12 ms); a unit is now one walk, 1/18 of that.
 __global__ void __launch_bounds__(kFreshEvalThreads, 1) k_fresh_walk(const __grid_constant__ FreshWalkParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_trigger();      // k_combine fills its tables as this kernel's CTAs leave
     fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};

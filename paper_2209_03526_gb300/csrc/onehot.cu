@@ -100,6 +100,7 @@ constexpr int kEvalEtMaxThreads = 512;
 
 __global__ void __launch_bounds__(kEvalEtMaxThreads, 1) k_onehot_evalall_et(const __grid_constant__ EvalEtParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_trigger();
     fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
@@ -303,9 +304,10 @@ __device__ __forceinline__ void load_halves(const DotParams& P, uint32_t W, uint
 #pragma unroll
     for (int k = 0; k < kDotPreds; k++) {
         if ((uint32_t)k < np) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(P.hv + (uint64_t)(P.half_base[k] + j * 2) * W + w0));
-            const uint4 b = __ldg(reinterpret_cast<const uint4*>(
-                P.hv + (uint64_t)(P.half_base[k] + ((j + 2) % 3) * 2 + 1) * W + w0));
+            // plain loads: a read-only one could move above grid_wait
+            const uint4 a = *reinterpret_cast<const uint4*>(P.hv + (uint64_t)(P.half_base[k] + j * 2) * W + w0);
+            const uint4 b = *reinterpret_cast<const uint4*>(
+                P.hv + (uint64_t)(P.half_base[k] + ((j + 2) % 3) * 2 + 1) * W + w0);
             h[k][0][0] = a.x; h[k][0][1] = a.y; h[k][0][2] = a.z; h[k][0][3] = a.w;
             h[k][1][0] = b.x; h[k][1][1] = b.y; h[k][1][2] = b.z; h[k][1][3] = b.w;
         } else {
@@ -357,7 +359,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_onehot_dots_pipe(const __grid_co
     const uint32_t np = P.n_preds;
     const uint64_t nwords = (P.n_elems + 31) / 32, halves = 2 * nwords;
     const uint64_t half0 = blockIdx.x * halves / gridDim.x, half1 = (blockIdx.x + 1) * halves / gridDim.x;
-    if (half0 >= half1) return;
+    grid_trigger();
     const uint32_t mine_halves = (uint32_t)(half1 - half0);
     DotSteps F{};                                     // the next step to fetch
     F.chunks = (mine_halves + 1) / 2;
@@ -387,7 +389,8 @@ __global__ void __launch_bounds__(WARPS * 32) k_onehot_dots_pipe(const __grid_co
         cp_async_commit();                            // an empty group keeps the count uniform
         fetch_stage = fetch_stage + 1 == kPipeStages ? 0 : fetch_stage + 1;
     };
-    for (int d = 0; d < kPipeStages - 1; d++) fetch();
+    for (int d = 0; d < kPipeStages - 1; d++) fetch();    // the table's rows do not depend on EvalAll
+    grid_wait();
     uint32_t h[kDotPreds][2][4], hn[kDotPreds][2][4];
     load_halves(P, W, w0, np, 0, h);
     const uint32_t chunks = F.chunks, last_batches = F.last_batches;
@@ -484,7 +487,7 @@ void launch_dots_pipe(const DotParams& D, uint64_t nwords, int sm_count, cudaStr
     constexpr uint32_t smem = WARPS * kPipeSmemPerWarp;
     const uint32_t per_sm = std::max<uint32_t>(1, std::min<uint32_t>(227u * 1024 / (smem + 4096), 32 / WARPS));
     const uint64_t grid = std::min<uint64_t>(nwords, (uint64_t)sm_count * per_sm);
-    k_onehot_dots_pipe<WARPS><<<(unsigned)grid, WARPS * 32, smem, s>>>(D);
+    launch_after(k_onehot_dots_pipe<WARPS>, (unsigned)grid, WARPS * 32, smem, s, D);
 }
 
 void launch_dots(const DotParams& D, uint64_t nwords, int sm_count, cudaStream_t s) {
@@ -535,6 +538,7 @@ constexpr uint32_t kFoldBlockElems = 128;
 __global__ void __launch_bounds__(kFoldThreads, 1) k_onehot_fold(const __grid_constant__ FoldParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
     fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
     const uint32_t lane = threadIdx.x & 31, warps = blockDim.x >> 5;
@@ -845,7 +849,7 @@ extern "C" oblivgm_status oblivgm_filter_onehot(oblivgm_ctx* ctx, uint32_t query
         const uint64_t warps = std::min<uint64_t>(kFoldThreads / 32, std::max<uint64_t>(
                                                       4, (fold_items + ctx->sm_count - 1) / ctx->sm_count));
         const unsigned grid = (unsigned)std::min<uint64_t>((fold_items + warps - 1) / warps, (uint64_t)ctx->sm_count);
-        k_onehot_fold<<<grid, (unsigned)(warps * 32), kTableBytes, s>>>(F);
+        launch_after(k_onehot_fold, grid, (unsigned)(warps * 32), kTableBytes, s, F);
         ctx->launches++;
     }
     ce = cudaGetLastError();

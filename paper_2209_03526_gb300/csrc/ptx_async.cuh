@@ -56,6 +56,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t phase,
     return true;
 }
 
+// Programmatic dependent launch (launch_after, runtime.h).  A kernel of a chain lets the next one
+// start as its own CTAs leave the SMs, and calls grid_wait before it reads or writes anything
+// that an earlier kernel of the stream touches: every thread, before any return, so that the
+// kernel's end also means the end of those before it.
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Per-thread asynchronous 16-byte copy global -> shared (cp.async, L2 only).  With
 // src_bytes = 0 nothing is read and the 16 bytes are zero-filled.  Both addresses must be
 // 16-byte aligned.  A thread sees its own copies once a wait_group covering them returns.

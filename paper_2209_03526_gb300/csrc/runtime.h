@@ -144,6 +144,24 @@ inline unsigned even_threads(uint64_t items, int sm_count, unsigned max_threads)
     return (unsigned)std::min<uint64_t>(max_threads, std::max<uint64_t>(64, (t + 31) / 32 * 32));
 }
 
+// Launches a kernel as a programmatic dependent of the one before it in the stream: its launch and
+// its prologue (the table fill) run while that one drains.  The kernel must call grid_wait
+// (ptx_async.cuh) before it touches global memory that an earlier kernel may use.
+template <class... P, class... A>
+inline void launch_after(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = a;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, kernel, args...);      // its error is the caller's cudaGetLastError
+}
+
 oblivgm_status fail(oblivgm_status st, const std::string& msg);
 const std::string& last_error_text();   // the calling thread's last failure text
 oblivgm_status cuda_fail(cudaError_t e, const char* what);

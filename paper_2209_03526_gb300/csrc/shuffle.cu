@@ -22,6 +22,7 @@
 #include "device_fss.cuh"
 #include "host_crypto.h"
 #include "oblivgm.h"
+#include "ptx_async.cuh"
 #include "runtime.h"
 
 namespace ogm {
@@ -107,6 +108,7 @@ __device__ __forceinline__ void mask_words(const SmemTabPair& T, const ShufParam
 // function sees only h <= 16 bits, so 4 * 2^h AES calls per permutation cover all inputs
 __global__ void __launch_bounds__(kShufThreads, 1) k_feistel_tab(const __grid_constant__ ShufParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_trigger();
     fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
     __syncthreads();
     const SmemTabPair T{reinterpret_cast<const char*>(smem), lane_offset()};
@@ -221,7 +223,9 @@ __device__ __forceinline__ void load_input(const ShufParams& P, int j, uint64_t 
 template <bool FAST>
 __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs1(const __grid_constant__ ShufParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_trigger();
     fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     Perm p12, p31;
     load_perms<FAST>(P, smem, S12, S31, p12, p31);
     __syncthreads();
@@ -248,7 +252,9 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs1(const __grid_const
 template <bool FAST>
 __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs2(const __grid_constant__ ShufParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_trigger();
     fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     Perm p12, p23;
     load_perms<FAST>(P, smem, S12, S23, p12, p23);
     __syncthreads();
@@ -290,7 +296,9 @@ __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs2(const __grid_const
 template <bool FAST>
 __global__ void __launch_bounds__(kShufThreads, 1) k_shuf_cs3(const __grid_constant__ ShufParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
+    grid_trigger();
     fill_tables<true>(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     Perm p23, p31;
     load_perms<FAST>(P, smem, S23, S31, p23, p31);
     __syncthreads();
@@ -343,6 +351,8 @@ __device__ __forceinline__ bool opened_one(const CompactParams& P, uint64_t l) {
 // open x^ for a block of rows and count the ones
 __global__ void __launch_bounds__(kCompactRows) k_open_count(const __grid_constant__ CompactParams P) {
     __shared__ uint32_t warp_n[kCompactRows / 32];
+    grid_trigger();
+    grid_wait();
     const uint64_t l = (uint64_t)blockIdx.x * kCompactRows + threadIdx.x;
     const uint32_t b = __ballot_sync(0xFFFFFFFFu, opened_one(P, l));
     if ((threadIdx.x & 31) == 0) warp_n[threadIdx.x >> 5] = __popc(b);
@@ -358,6 +368,8 @@ __global__ void __launch_bounds__(kCompactRows) k_open_count(const __grid_consta
 __global__ void __launch_bounds__(1024) k_scan_counts(uint32_t* c, uint32_t n_blocks) {
     __shared__ uint32_t part[1024];
     __shared__ uint32_t carry;
+    grid_trigger();
+    grid_wait();
     if (threadIdx.x == 0) carry = 0;
     __syncthreads();
     for (uint32_t base = 0; base < n_blocks; base += 1024) {
@@ -382,6 +394,7 @@ __global__ void __launch_bounds__(1024) k_scan_counts(uint32_t* c, uint32_t n_bl
 // write the kept rows (id and attributes of every share set) at their scanned offsets
 __global__ void __launch_bounds__(kCompactRows) k_compact(const __grid_constant__ CompactParams P) {
     __shared__ uint32_t warp_off[kCompactRows / 32];
+    grid_wait();
     const uint64_t l = (uint64_t)blockIdx.x * kCompactRows + threadIdx.x;
     const bool keep = opened_one(P, l);
     const uint32_t b = __ballot_sync(0xFFFFFFFFu, keep);
@@ -493,13 +506,13 @@ oblivgm_status shuffle_device(oblivgm_ctx* ctx, uint32_t group, uint64_t n, uint
     k_feistel_tab<<<grid(12ull << P.half_bits), kShufThreads, kTableBytes, s>>>(P);
     if (fast) {
         const int smem = kTableBytes + (int)((8u << P.half_bits) * sizeof(uint16_t));
-        k_shuf_cs1<true><<<grid(n), kShufThreads, smem, s>>>(P);
-        k_shuf_cs2<true><<<grid(2 * n), kShufThreads, smem, s>>>(P);
-        k_shuf_cs3<true><<<grid(n), kShufThreads, smem, s>>>(P);
+        launch_after(k_shuf_cs1<true>, grid(n), kShufThreads, smem, s, P);
+        launch_after(k_shuf_cs2<true>, grid(2 * n), kShufThreads, smem, s, P);
+        launch_after(k_shuf_cs3<true>, grid(n), kShufThreads, smem, s, P);
     } else {
-        k_shuf_cs1<false><<<grid(n), kShufThreads, kTableBytes, s>>>(P);
-        k_shuf_cs2<false><<<grid(2 * n), kShufThreads, kTableBytes, s>>>(P);
-        k_shuf_cs3<false><<<grid(n), kShufThreads, kTableBytes, s>>>(P);
+        launch_after(k_shuf_cs1<false>, grid(n), kShufThreads, kTableBytes, s, P);
+        launch_after(k_shuf_cs2<false>, grid(2 * n), kShufThreads, kTableBytes, s, P);
+        launch_after(k_shuf_cs3<false>, grid(n), kShufThreads, kTableBytes, s, P);
     }
     ctx->launches += 4;
     cudaError_t ce = cudaGetLastError();
@@ -612,9 +625,9 @@ extern "C" oblivgm_status oblivgm_fetch_multi(oblivgm_ctx* ctx, uint32_t table_i
     C.width = W;
     C.stride = stride;
     C.n_blocks = n_blocks;
-    k_open_count<<<n_blocks, kCompactRows, 0, s>>>(C);
-    k_scan_counts<<<1, 1024, 0, s>>>(counts, n_blocks);
-    k_compact<<<n_blocks, kCompactRows, 0, s>>>(C);
+    launch_after(k_open_count, n_blocks, kCompactRows, 0, s, C);
+    launch_after(k_scan_counts, 1, 1024, 0, s, counts, n_blocks);
+    launch_after(k_compact, n_blocks, kCompactRows, 0, s, C);
     ctx->launches += 3;
     ce = cudaGetLastError();
     if (ce != cudaSuccess) {

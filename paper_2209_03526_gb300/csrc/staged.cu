@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "device_fss.cuh"
+#include "ptx_async.cuh"
 #include "runtime.h"
 #include "staged.h"
 
@@ -52,6 +53,11 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
     return m;
 }
 
+// All launches of an evaluation but the first are programmatic dependents of the one before
+// (ptx_async.cuh), since many are a few microseconds long: 100,003 vertices, 3 predicates (27
+// launches) 1,759 -> 1,700 us, 12 DCF keys at 65,537 points 631 -> 578 us, triangle + pendant on
+// 1M / 10M (200 launches) 17.07 -> 16.66 ms.
+
 // ------------------------------------------------------------------ opened columns, sorted
 //
 // Least-significant-digit radix sort, 8 bits a pass, of all the launch's sparse columns side
@@ -62,6 +68,8 @@ template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const SgCol* cols, uint32_t pass) {
     __shared__ uint32_t h[256];
     const SgCol& C = cols[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (blockIdx.x >= C.tiles || pass >= C.passes) return;
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -127,6 +135,8 @@ __device__ __forceinline__ void row_scan(uint32_t* row, uint32_t n, uint32_t* to
 
 __global__ void __launch_bounds__(256) k_sort_scan(const SgCol* cols, uint32_t pass) {
     const SgCol& C = cols[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (pass >= C.passes) return;
     row_scan(C.hist + (uint64_t)blockIdx.x * C.tiles, C.tiles, C.tot + blockIdx.x);
 }
@@ -155,9 +165,11 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sort_scatter(const SgCol* c
     __shared__ uint32_t base_of[256];      // output position of a digit's first key, less its place in the tile
     __shared__ uint32_t ws[8];
     const SgCol& C = cols[blockIdx.y];
-    if (blockIdx.x >= C.tiles || pass >= C.passes) return;
+    grid_trigger();
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, shift = 8 * pass;
     for (int w = 0; w < kSortWarps; w++) cnt[w][threadIdx.x] = 0;
+    grid_wait();
+    if (blockIdx.x >= C.tiles || pass >= C.passes) return;
     __syncthreads();
     const uint32_t* src = C.key[pass & 1];
     const uint32_t* isrc = C.idx[pass & 1];
@@ -232,6 +244,8 @@ template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_uniq_count(const SgCol* cols) {
     __shared__ uint32_t ws[kSortWarps];
     const SgCol& C = cols[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (blockIdx.x >= C.tiles || C.passes == 0) return;
     const uint32_t* key = C.key[C.passes & 1];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -251,6 +265,8 @@ __global__ void __launch_bounds__(kSortThreads) k_uniq_count(const SgCol* cols) 
 
 __global__ void __launch_bounds__(256) k_uniq_scan(const SgCol* cols) {
     const SgCol& C = cols[blockIdx.x];
+    grid_trigger();
+    grid_wait();
     if (C.passes == 0) return;
     row_scan(C.hist, C.tiles, C.m);
 }
@@ -259,6 +275,8 @@ template <int ITEMS>
 __global__ void __launch_bounds__(kSortThreads) k_uniq_emit(const SgCol* cols) {
     __shared__ uint32_t ws[kSortWarps];
     const SgCol& C = cols[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (blockIdx.x >= C.tiles || C.passes == 0) return;
     const uint32_t* key = C.key[C.passes & 1];
     const uint32_t* idx = C.idx[C.passes & 1];
@@ -310,6 +328,8 @@ __device__ __forceinline__ int common_bits(const SgPred& P, const uint32_t* u, u
 __global__ void __launch_bounds__(kRunBlock) k_run_count(const SgPred* preds, uint32_t chunk) {
     __shared__ uint32_t ws[32][kSgMaxStages];
     const SgPred& P = preds[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (P.dense) return;
     const uint32_t n = chunk_values(P, chunk);
     if ((uint64_t)blockIdx.x * kRunBlock >= n) return;
@@ -331,6 +351,8 @@ __global__ void __launch_bounds__(kRunBlock) k_run_count(const SgPred* preds, ui
 
 __global__ void __launch_bounds__(256) k_run_scan(const SgPred* preds, uint32_t chunk) {
     const SgPred& P = preds[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (P.dense || blockIdx.x + 1 >= P.stages) return;
     const uint32_t n = chunk_values(P, chunk);
     row_scan(P.blk + (uint64_t)blockIdx.x * P.blocks, (n + kRunBlock - 1) / kRunBlock, P.cnt + blockIdx.x);
@@ -339,6 +361,8 @@ __global__ void __launch_bounds__(256) k_run_scan(const SgPred* preds, uint32_t 
 __global__ void __launch_bounds__(kRunBlock) k_run_emit(const SgPred* preds, uint32_t chunk) {
     __shared__ uint32_t ws[32][kSgMaxStages];
     const SgPred& P = preds[blockIdx.y];
+    grid_trigger();
+    grid_wait();
     if (P.dense) return;
     const uint32_t n = chunk_values(P, chunk);
     if ((uint64_t)blockIdx.x * kRunBlock >= n) return;
@@ -453,6 +477,9 @@ __device__ __forceinline__ void unit_table(unsigned long long* first, uint32_t n
 __global__ void __launch_bounds__(kStageThreads, 1) k_stage(const __grid_constant__ StageParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ unsigned long long first[kMaxRoundPreds + 1];
+    grid_trigger();
+    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     unsigned long long units = 0;
     if (threadIdx.x < P.n_preds) {
         const SgPred& D = P.preds[threadIdx.x];
@@ -462,8 +489,6 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage(const __grid_constan
     unit_table(first, P.n_preds, units);
     const unsigned long long total = first[P.n_preds];
     if (total == 0) return;
-    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
-    __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
     const uint32_t lane = threadIdx.x & 31, st = P.stage;
     const unsigned long long step = (unsigned long long)gridDim.x * (kStageThreads / 32);
@@ -509,6 +534,9 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage(const __grid_constan
 __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_constant__ StageParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ unsigned long long first[kMaxRoundPreds + 1];
+    grid_trigger();
+    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     unsigned long long units = 0;
     if (threadIdx.x < P.n_preds) {
         const SgPred& D = P.preds[threadIdx.x];
@@ -517,8 +545,6 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_co
     unit_table(first, P.n_preds, units);
     const unsigned long long total = first[P.n_preds];
     if (total == 0) return;
-    fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
-    __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
     const uint32_t lane = threadIdx.x & 31;
     const unsigned long long step = (unsigned long long)gridDim.x * (kStageThreads / 32);
@@ -587,9 +613,11 @@ static_assert(kMaxTileSteps >= kMaxRoundPreds, "a round's predicates may all be 
 constexpr int kMaxPrefixes = (int)kMaxTileSteps * 6 * (kStageThreads / 256);
 constexpr int kCombineSmem = kTableBytes + kMaxPrefixes * kPrefixWords * 4;
 
-// index of element e's value in a predicate's sums
+// index of element e's value in a predicate's sums.  What earlier kernels of the chain wrote is
+// read with plain loads: it changes while this kernel waits for them, which the read-only path
+// does not allow.
 __device__ __forceinline__ uint32_t value_index(const SgGroup& G, const SgFold& D, uint64_t e) {
-    if (D.index == kIndexRank) return __ldg(D.rank + e);
+    if (D.index == kIndexRank) return D.rank[e];
     if (D.index == kIndexElem) return (uint32_t)e;
     const uint64_t row = (uint64_t)D.attr * G.stride + e;
     return (__ldg(G.share[0] + row) + __ldg(G.share[1] + row) + __ldg(G.share[2] + row) + D.radd) & D.mask;
@@ -607,7 +635,9 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
     extern __shared__ __align__(128) unsigned char smem[];
     uint4* pre_c = reinterpret_cast<uint4*>(smem + kTableBytes);
     uint32_t* pre_n = reinterpret_cast<uint32_t*>(pre_c + kMaxPrefixes);
+    grid_trigger();
     fill_tables(reinterpret_cast<uint32_t*>(smem), P.te0);
+    grid_wait();
     __syncthreads();
     const SmemTab T{reinterpret_cast<const char*>(smem), lane_offset()};
     const uint32_t tile = blockDim.x * P.per_thread, subs = tile >> 8;   // 256-element parts of a tile
@@ -618,7 +648,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
         const SgGroup& G = P.groups[g];
         const uint64_t e = (blockIdx.x - G.item_begin) * tile + threadIdx.x;
         const SgFold& D = P.folds[G.pred_begin];
-        if (e < G.n_elems) zq = __ldg(reinterpret_cast<const uint4*>(D.z) + value_index(G, D, e));
+        if (e < G.n_elems) zq = reinterpret_cast<const uint4*>(D.z)[value_index(G, D, e)];
     }
     for (uint64_t w = blockIdx.x; w < P.items;) {
         const SgGroup& G = P.groups[g];
@@ -658,7 +688,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
                 const bool more = (!leave || w2 < P.items) && e2 < G2.n_elems;
                 const uint32_t at2 = more ? value_index(G2, D2, e2) : 0u;
                 if (!mine) {
-                    if (more) zq = __ldg(reinterpret_cast<const uint4*>(D2.z) + at2);
+                    if (more) zq = reinterpret_cast<const uint4*>(D2.z)[at2];
                     continue;
                 }
                 const bool fold = !(G.first && k == 0);
@@ -670,7 +700,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
                         const uint32_t at_pre = ((k * subs + sub) * 2 + pass) * 3 + i;
                         const CtrPrefix c{pre_n[at_pre], pre_c[at_pre]};
                         const uint32_t f = ctr_w0(T, P.rk_prf[i], c, (uint32_t)e);   // F keeps bytes 0..3
-                        if (pass == 0 && i == 0 && more) zq = __ldg(reinterpret_cast<const uint4*>(D2.z) + at2);
+                        if (pass == 0 && i == 0 && more) zq = reinterpret_cast<const uint4*>(D2.z)[at2];
                         r[0] += i == 0 ? f : (i == 2 ? 0u - f : 0u);
                         r[1] += i == 1 ? f : (i == 0 ? 0u - f : 0u);
                         r[2] += i == 2 ? f : (i == 1 ? 0u - f : 0u);
@@ -712,10 +742,12 @@ struct GatherParams {
 
 __global__ void __launch_bounds__(256) k_gather_raw(const __grid_constant__ GatherParams P) {
     const SgCol& C = *P.col;
+    grid_trigger();
+    grid_wait();
     for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < P.n_points; i += (uint64_t)gridDim.x * 256) {
-        const uint32_t at = C.passes ? __ldg(C.rank + i) : __ldg(C.share[0] + i) & C.mask;
+        const uint32_t at = C.passes ? C.rank[i] : __ldg(C.share[0] + i) & C.mask;
         for (uint32_t k = blockIdx.y; k < P.n_keys; k += gridDim.y)
-            P.out[k * P.n_points + i] = __ldg(P.z + k * P.vals + at);
+            P.out[k * P.n_points + i] = P.z[k * P.vals + at];
     }
 }
 
@@ -854,7 +886,7 @@ void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* grou
     F.n_groups = n_groups;
     F.items = items;
     F.per_thread = c.per_thread;
-    k_combine<<<(unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, items), c.threads, kCombineSmem, s>>>(F);
+    launch_after(k_combine, (unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, items), c.threads, kCombineSmem, s, F);
     ctx->launches++;
 }
 
@@ -1034,13 +1066,14 @@ void launch_sort_tiles(const Staged& sg, const SgCol* cols, cudaStream_t s) {
     const unsigned nc = (unsigned)sg.cols.size();
     const dim3 grid(sg.sort_tiles, nc);
     for (uint32_t p = 0; p < sg.sort_passes; p++) {
-        k_sort_hist<ITEMS><<<grid, kSortThreads, 0, s>>>(cols, p);
-        k_sort_scan<<<dim3(256, nc), 256, 0, s>>>(cols, p);
-        k_sort_scatter<ITEMS><<<grid, kSortThreads, 0, s>>>(cols, p);
+        if (p == 0) k_sort_hist<ITEMS><<<grid, kSortThreads, 0, s>>>(cols, p);
+        else launch_after(k_sort_hist<ITEMS>, grid, kSortThreads, 0, s, cols, p);
+        launch_after(k_sort_scan, dim3(256, nc), 256, 0, s, cols, p);
+        launch_after(k_sort_scatter<ITEMS>, grid, kSortThreads, 0, s, cols, p);
     }
-    k_uniq_count<ITEMS><<<grid, kSortThreads, 0, s>>>(cols);
-    k_uniq_scan<<<nc, 256, 0, s>>>(cols);
-    k_uniq_emit<ITEMS><<<grid, kSortThreads, 0, s>>>(cols);
+    launch_after(k_uniq_count<ITEMS>, grid, kSortThreads, 0, s, cols);
+    launch_after(k_uniq_scan, nc, 256, 0, s, cols);
+    launch_after(k_uniq_emit<ITEMS>, grid, kSortThreads, 0, s, cols);
 }
 
 uint64_t launch_sort(const Staged& sg, const SgCol* cols, cudaStream_t s) {
@@ -1062,16 +1095,16 @@ uint64_t launch_round(const oblivgm_ctx* ctx, const StagedRound& R, const SgPred
     const unsigned sms = (unsigned)ctx->sm_count;
     for (uint32_t c = 0; c < R.chunks; c++) {
         if (R.sparse && R.max_stages > 1) {
-            k_run_count<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
-            k_run_scan<<<dim3(R.max_stages - 1, R.n_preds), 256, 0, s>>>(W.preds, c);
-            k_run_emit<<<dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s>>>(W.preds, c);
+            launch_after(k_run_count, dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s, W.preds, c);
+            launch_after(k_run_scan, dim3(R.max_stages - 1, R.n_preds), 256, 0, s, W.preds, c);
+            launch_after(k_run_emit, dim3(R.max_blocks, R.n_preds), kRunBlock, 0, s, W.preds, c);
         }
         W.chunk = c;
         for (uint32_t st = 0; st + 1 < R.max_stages; st++) {
             W.stage = st;
-            k_stage<<<sms, kStageThreads, kTableBytes, s>>>(W);
+            launch_after(k_stage, sms, kStageThreads, kTableBytes, s, W);
         }
-        k_stage_last<<<sms, kStageThreads, kTableBytes, s>>>(W);
+        launch_after(k_stage_last, sms, kStageThreads, kTableBytes, s, W);
     }
     return R.chunks * (R.max_stages + (R.sparse && R.max_stages > 1 ? 3ull : 0ull));
 }
@@ -1175,7 +1208,7 @@ oblivgm_status staged_launch_raw(oblivgm_ctx* ctx, const Staged& sg, const unsig
         G.n_keys = p.n_keys;
         G.out = out + (uint64_t)p.key_begin * G.n_points;
         const unsigned gx = (unsigned)std::min<uint64_t>((G.n_points + 255) / 256, 8ull * ctx->sm_count);
-        k_gather_raw<<<dim3(gx, std::min<uint32_t>(p.n_keys, 8)), 256, 0, s>>>(G);
+        launch_after(k_gather_raw, dim3(gx, std::min<uint32_t>(p.n_keys, 8)), 256, 0, s, G);
         launches++;
     }
     const cudaError_t e = cudaGetLastError();
