@@ -855,12 +855,18 @@ size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
 
 }  // namespace
 
-// Elements per tile of the combine: narrower CTAs where that spreads a small launch over more
-// SMs, several elements per thread, so that a tile's barriers are rare, where every SM still
-// gets a few tiles.
+// Elements per tile of the combine: the CTA width whose waves take the least time (a wave of t
+// threads takes as long as its lookups, or at 384 threads and less as long as an element's chain
+// of PRF words: 100,003 elements in one wave of 768 threads 26 us, in two of 512 46 us), and
+// several elements per thread, so that a tile's barriers are rare, where every SM still gets a
+// few tiles.
 CombineShape combine_shape(uint64_t elems, uint32_t most_preds, int sm_count) {
     CombineShape c;
-    c.threads = elems >= (uint64_t)kStageThreads * sm_count ? kStageThreads : elems >= 512ull * sm_count ? 512 : 256;
+    uint64_t best = ~0ull;
+    for (uint32_t t = 256; t <= (uint32_t)kStageThreads; t += 256) {
+        const uint64_t waves = ((elems + t - 1) / t + sm_count - 1) / sm_count, cost = waves * std::max(t, 384u);
+        if (cost <= best) { best = cost; c.threads = t; }
+    }
     const uint64_t spread = elems / (6ull * kStageThreads * sm_count);
     c.per_thread = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>({8, spread, kMaxTileSteps / most_preds}));
     return c;
