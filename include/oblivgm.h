@@ -602,8 +602,9 @@ oblivgm_status oblivgm_set_schedule(oblivgm_ctx* ctx, uint32_t threads, uint32_t
  * most `max_elems` elements in all is evaluated by the walk-parallel kernel,
  * one thread per key walk (six DPF or twelve DCF walks of an element side by
  * side), instead of one thread per element.  Both kernels give identical
- * output.  Default: 128 x the SM count; 0 turns the walk-parallel kernel off,
- * UINT64_MAX uses it for every batch.  `previous` (may be NULL) receives the
+ * output.  Default: 128 x the SM count, less the batches of several waves whose
+ * elements' shared tree nodes make the staged evaluation faster; 0 turns the
+ * walk-parallel kernel off, UINT64_MAX uses it for every batch.  `previous` (may be NULL) receives the
  * setting it replaces.  Applies to oblivgm_filter_and_combine,
  * oblivgm_filter_batch, the no-alloc entry point, plans created afterwards and
  * the serving loop.  Errors: EINVAL for a NULL context. */

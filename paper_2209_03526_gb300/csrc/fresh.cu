@@ -655,7 +655,7 @@ static oblivgm_status filter_fresh_walks(oblivgm_ctx* ctx, const FreshEvalParams
                        kTableBytes, s>>>(*W);
         ctx->launches++;
         launch_combine(ctx, shape, reinterpret_cast<const SgGroup*>(scratch) + r.group_begin, r.n_groups,
-                       reinterpret_cast<const SgFold*>(scratch + off_folds), r.items, s);
+                       reinterpret_cast<const SgFold*>(scratch + off_folds), /*split=*/false, r.items, s);
     }
     ce = cudaGetLastError();
     if (ce != cudaSuccess) return cuda_fail(ce, "fresh walks launch");

@@ -724,6 +724,7 @@ static oblivgm_status check_ctx(oblivgm_ctx* ctx) {
 struct Plan {
     uint32_t tile = 0, elems_per_thread = 1, threads = 0;
     bool wp = false;   // walk-parallel kernel (k_filter_wp)
+    double wp_seconds = 0;   // its simulated time
     std::vector<GroupDesc> groups;
     std::vector<PredDesc> preds;
     std::vector<DevKey> keys;
@@ -963,19 +964,20 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
     const uint32_t max_tile = !wp ? ctx->threads * ctx->elems_per_thread : ctx->wp_tile ? ctx->wp_tile : (uint32_t)kWpElems;
     std::vector<uint32_t> tiles = tiles_of(max_tile);
     bool wp_wide = wp && max_tile > (uint32_t)kWpElems;
+    std::vector<CtaClass> finish;
+    const auto makespan = [&](const std::vector<uint32_t>& t) {
+        return simulate_makespan(all.size(), n_of, [&](size_t g) { return (uint64_t)t[g]; }, time_of, sm_count, finish);
+    };
     if (wp && step != 0 && items_of(kWpElems, group_tiles ? 2 * kWpElems : kWpElems) > (uint64_t)sm_count) {
         // more than one wave of 32-element tiles: 40-element ones, 6 % slower otherwise, where they
         // take fewer waves (5,000 elements, n = 32, EQ AND RANGE: 134 us against 166)
         std::vector<uint32_t> wide = tiles_of(kWpMaxElems);
-        std::vector<CtaClass> finish;
-        const auto makespan = [&](const std::vector<uint32_t>& t) {
-            return simulate_makespan(all.size(), n_of, [&](size_t g) { return (uint64_t)t[g]; }, time_of, sm_count, finish);
-        };
         if (1.06 * makespan(wide) < makespan(tiles)) {
             tiles = std::move(wide);
             wp_wide = true;
         }
     }
+    if (wp) plan->wp_seconds = 1e-9 * makespan(tiles) + 8e-6;
     plan->threads = !wp ? ctx->threads : (uint32_t)(wp_wide ? WpShape<kWpMaxElems>::kThreads : WpShape<kWpElems>::kThreads);
     plan->groups.clear(); plan->preds.clear(); plan->keys.clear(); plan->item_start.clear();
     plan->tile = *std::max_element(tiles.begin(), tiles.end());
@@ -1004,20 +1006,25 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
     return OBLIVGM_OK;
 }
 
+// no staged evaluation is faster (n = 8, one predicate, dense: 13 to 17 us; sorted ones from 40 us)
+constexpr double kStagedLeastSeconds = 24e-6;
+
 // Plan a batch for the fused kernel in the context's launch shape; a batch whose groups
 // hold at most ctx->wp_max_elems elements in all goes to the walk-parallel kernel instead,
-// in tiles of kWpElems elements, and a larger one to the staged evaluation (staged_ok) where
-// its estimate is below the fused kernel's.
+// in tiles of kWpElems elements, and either to the staged evaluation (staged_ok) where its
+// estimate is below that kernel's.
 oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& tables, uint32_t n_queries,
                            const uint32_t* query_ids, const ParsedQuery* parsed, const uint32_t* n_groups,
                            uint32_t* const* const* outs, bool staged_ok, Plan* plan) {
     plan->staged = false;
     const oblivgm_status s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, ctx, plan);
-    if (s != OBLIVGM_OK || plan->wp) return s;
-    // large launches share tree nodes between elements where that pays; the key-staging expiry
-    // hook is about the fused kernels' waits
-    if (staged_ok && !ctx->test_expire_next)
-        plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap, &plan->sg);
+    if (s != OBLIVGM_OK || (plan->wp && (ctx->wp_fixed || ctx->wp_tile))) return s;
+    // launches share tree nodes between elements where that pays (5 predicates on 12,000 elements,
+    // n = 16: 337 us walk-parallel, 160 staged), but for one wave of walk-parallel tiles, which the
+    // staged launches alone outlast; the key-staging expiry hook is about the fused kernels' waits
+    if (staged_ok && !ctx->test_expire_next && (!plan->wp || plan->wp_seconds > kStagedLeastSeconds))
+        plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap,
+                                   plan->wp ? plan->wp_seconds : 0.0, &plan->sg);
     return OBLIVGM_OK;
 }
 
@@ -1101,6 +1108,14 @@ void apply_test_expiry(oblivgm_ctx* ctx, FilterParams* P) {
 // needs next to none, runs then.
 oblivgm_status launch_staged(oblivgm_ctx* ctx, Plan& plan, cudaStream_t st, bool* ran) {
     *ran = false;
+    if (plan.wp) {
+        // a small launch that is being captured stays one kernel without scratch
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            return OBLIVGM_OK;
+        }
+    }
     unsigned char *image = nullptr, *scratch = nullptr;
     const oblivgm_status as =
         ws_alloc(ctx, reinterpret_cast<void**>(&image), plan.sg.image_bytes, st, "workspace allocation");
@@ -1593,6 +1608,7 @@ oblivgm_status oblivgm_set_walk_parallel(oblivgm_ctx* ctx, uint64_t max_elems, u
     if (st) return st;
     if (previous) *previous = ctx->wp_max_elems;
     ctx->wp_max_elems = max_elems;
+    ctx->wp_fixed = max_elems != (uint64_t)ctx->sm_count * kWpDefaultElemsPerSm;
     return OBLIVGM_OK;
 }
 
@@ -1750,7 +1766,7 @@ extern "C" oblivgm_status oblivgm_plan_create(oblivgm_ctx* ctx, uint32_t n_queri
     p->n_items = plan.item_start.back();
     p->threads = plan.threads;
     p->E = plan.elems_per_thread;
-    p->wp = plan.wp;
+    p->wp = plan.wp && !plan.staged;
     *out_plan = p;
     return OBLIVGM_OK;
 }

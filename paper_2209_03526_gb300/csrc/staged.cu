@@ -530,7 +530,9 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage(const __grid_constan
 }
 
 // The last stage: a warp takes 32 distinct values of one output slot (a server's two key
-// halves, or one key of a raw evaluation) and walks the slot's keys one after another.
+// halves, or one key of a raw evaluation) and walks the slot's keys one after another, or, in a
+// launch of few such units, one of its keys (SgPred::parts): a slot of a range predicate is a
+// chain of four walks that leaves most warps without work.
 __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_constant__ StageParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ unsigned long long first[kMaxRoundPreds + 1];
@@ -540,7 +542,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_co
     unsigned long long units = 0;
     if (threadIdx.x < P.n_preds) {
         const SgPred& D = P.preds[threadIdx.x];
-        units = (unsigned long long)D.slots * ((chunk_values(D, P.chunk) + 31) / 32);
+        units = (unsigned long long)D.slots * D.parts * ((chunk_values(D, P.chunk) + 31) / 32);
     }
     unit_table(first, P.n_preds, units);
     const unsigned long long total = first[P.n_preds];
@@ -553,11 +555,12 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_co
         while (first[p + 1] <= w) p++;
         const SgPred& D = P.preds[p];
         const uint32_t vals = chunk_values(D, P.chunk), per_slot = (vals + 31) / 32;
-        const uint32_t local = (uint32_t)(w - first[p]), slot = local / per_slot;
-        const uint32_t i = (local - slot * per_slot) * 32 + lane;
+        const uint32_t local = (uint32_t)(w - first[p]), sp = local / per_slot;
+        const uint32_t slot = sp / D.parts, part = sp - slot * D.parts;
+        const uint32_t i = (local - sp * per_slot) * 32 + lane;
         if (i >= vals) continue;
         const bool dcf = D.kind == OBLIVGM_PRED_RANGE;
-        const uint32_t S = D.stages, nk = D.n_keys / D.slots;
+        const uint32_t S = D.stages, nk = D.n_keys / D.slots, nk_part = nk / D.parts;
         const int n = (int)D.n, a = S > 1 ? D.lev[S - 2] : 0;
         const uint64_t gi = (uint64_t)P.chunk * D.chunk + i;
         uint32_t x, par = 0;
@@ -570,7 +573,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_co
         }
         uint32_t z = 0;
 #pragma unroll 1
-        for (uint32_t kk = 0; kk < nk; kk++) {
+        for (uint32_t kk = part * nk_part; kk < (part + 1) * nk_part; kk++) {
             const uint32_t key = slot * nk + kk;
             const DevKey* K = P.keys + D.key_begin + key;
             const uint32_t party = __ldg(&K->party);
@@ -589,7 +592,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_stage_last(const __grid_co
             // RANGE: the public constant c * beta' joins party 0's half once (sub 0 of the half)
             if (dcf && (kk & 1u) == 0 && party == 0) z += D.cbeta;
         }
-        D.z[gi * D.z_elem + slot * D.z_slot] = z;
+        D.z[gi * D.z_elem + slot * D.z_slot + 4 * part] = z;
     }
 }
 
@@ -623,6 +626,20 @@ __device__ __forceinline__ uint32_t value_index(const SgGroup& G, const SgFold& 
     return (__ldg(G.share[0] + row) + __ldg(G.share[1] + row) + __ldg(G.share[2] + row) + D.radd) & D.mask;
 }
 
+// the three servers' sums of value `at`, over their parts
+template <bool SPLIT>
+__device__ __forceinline__ uint4 load_sums(const SgFold& D, uint32_t at) {
+    if (!SPLIT) return reinterpret_cast<const uint4*>(D.z)[at];
+    const uint4* z = reinterpret_cast<const uint4*>(D.z) + (uint64_t)at * (D.more + 1);
+    uint4 s = z[0];
+#pragma unroll 1
+    for (uint32_t w = 1; w <= D.more; w++) {
+        const uint4 a = z[w];
+        s.x += a.x; s.y += a.y; s.z += a.z;
+    }
+    return s;
+}
+
 // One thread per element of a tile: for each of the round's predicates the three servers' sums
 // at the element's value (z_i), r_i = z_i + F(k_i) - F(k_{i-1}) (Sec. III-B), and the fold into the
 // group's result with its re-share (Sec. V-D).  The PRF words bound it: 3 per predicate and 3
@@ -631,6 +648,7 @@ __device__ __forceinline__ uint32_t value_index(const SgGroup& G, const SgFold& 
 //     those share (ctr_prefix) and an element's word takes 121 lookups instead of 148;
 //   * the two dependent reads of the sums (rank, then a random 16 bytes) are issued one step
 //     ahead, the step after a tile's last predicate being the next tile's first.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_constant__ CombineParams P) {
     extern __shared__ __align__(128) unsigned char smem[];
     uint4* pre_c = reinterpret_cast<uint4*>(smem + kTableBytes);
@@ -648,7 +666,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
         const SgGroup& G = P.groups[g];
         const uint64_t e = (blockIdx.x - G.item_begin) * tile + threadIdx.x;
         const SgFold& D = P.folds[G.pred_begin];
-        if (e < G.n_elems) zq = reinterpret_cast<const uint4*>(D.z)[value_index(G, D, e)];
+        if (e < G.n_elems) zq = load_sums<SPLIT>(D, value_index(G, D, e));
     }
     for (uint64_t w = blockIdx.x; w < P.items;) {
         const SgGroup& G = P.groups[g];
@@ -688,7 +706,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
                 const bool more = (!leave || w2 < P.items) && e2 < G2.n_elems;
                 const uint32_t at2 = more ? value_index(G2, D2, e2) : 0u;
                 if (!mine) {
-                    if (more) zq = reinterpret_cast<const uint4*>(D2.z)[at2];
+                    if (more) zq = load_sums<SPLIT>(D2, at2);
                     continue;
                 }
                 const bool fold = !(G.first && k == 0);
@@ -700,7 +718,7 @@ __global__ void __launch_bounds__(kStageThreads, 1) k_combine(const __grid_const
                         const uint32_t at_pre = ((k * subs + sub) * 2 + pass) * 3 + i;
                         const CtrPrefix c{pre_n[at_pre], pre_c[at_pre]};
                         const uint32_t f = ctr_w0(T, P.rk_prf[i], c, (uint32_t)e);   // F keeps bytes 0..3
-                        if (pass == 0 && i == 0 && more) zq = reinterpret_cast<const uint4*>(D2.z)[at2];
+                        if (pass == 0 && i == 0 && more) zq = load_sums<SPLIT>(D2, at2);
                         r[0] += i == 0 ? f : (i == 2 ? 0u - f : 0u);
                         r[1] += i == 1 ? f : (i == 0 ? 0u - f : 0u);
                         r[2] += i == 2 ? f : (i == 1 ? 0u - f : 0u);
@@ -756,10 +774,16 @@ __global__ void __launch_bounds__(256) k_gather_raw(const __grid_constant__ Gath
 // GB300 figures the plan weighs: a DPF / DCF level step of one key at the T-table lookup rate,
 // a PRF word, a launch (with its table fill) and a key of a sort pass.
 constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, kLaunch = 4.0e-6;
+// a level step of a thread on its own, and what a small staged evaluation takes on top
+constexpr double kDpfLatency = 0.57e-6, kDcfLatency = 0.92e-6, kStagedFixed = 12e-6;
 constexpr double kSortKeyPass = 12e-12;
 constexpr uint64_t kMaxElems = 1ull << 28;
 constexpr uint32_t kMaxChunk = 1u << 22;      // distinct values evaluated together
 constexpr int kMaxDenseBits = 24;
+// A launch whose last stages have fewer units (32 values of one slot) than this, one and a half
+// for each of the chip's 152 x 24 warps, runs a unit per key there: a range of 5,000 values, n = 32,
+// 167 -> 135 us, of 2^8 (n = 8) 40 -> 17 us; 2^16 values in 1.7 units a warp lose 3 %.
+constexpr uint64_t kSplitUnits = 3 * 152 * 24 / 2;
 
 // distinct l-bit prefixes of n_vals uniform values, the most that a column can be expected to have
 double expected_nodes(double n_vals, int l) {
@@ -791,15 +815,15 @@ double choose_stages(double n_vals, bool dense, int n, double step_s, std::vecto
 size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
 // distinct values a predicate's column can have, and those of one chunk
-uint64_t max_values(const SgPred& p, const SgCol& c) {
-    const uint64_t domain = (uint64_t)p.mask + 1;
-    return p.dense ? domain : std::min<uint64_t>(c.n, domain);
+uint64_t max_values(const SgCol& c) {
+    const uint64_t domain = (uint64_t)c.mask + 1;
+    return c.passes == 0 ? domain : std::min<uint64_t>(c.n, domain);
 }
 
 // Runs a chunk can have after stage s.  A sparse chunk's values ascend in u, so in x^ = u + delta
 // they wrap once past 2^n: the prefix that holds the first value can come up again at the end.
 uint64_t max_runs(const SgPred& p, const SgCol& c, uint32_t s) {
-    return std::min<uint64_t>(std::min<uint64_t>(p.chunk, max_values(p, c)), (1ull << p.lev[s]) + (p.dense ? 0 : 1));
+    return std::min<uint64_t>(std::min<uint64_t>(p.chunk, max_values(c)), (1ull << p.lev[s]) + (p.dense ? 0 : 1));
 }
 
 // Sort tiles: large ones once the sparse columns fill the SMs' tiles several times over.
@@ -831,8 +855,8 @@ size_t layout_col(SgCol* c, unsigned char* base, size_t at) {
 
 size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
     const auto take = [&](size_t b) { unsigned char* q = base + at; at += up256(b); return reinterpret_cast<uint32_t*>(q); };
-    const uint64_t vals = max_values(*p, c);
-    p->z = take(p->z_elem == 4 ? vals * 16 : vals * 4 * p->n_keys);
+    const uint64_t vals = max_values(c);
+    p->z = take(vals * 4 * (p->z_elem > 1 ? p->z_elem : p->n_keys));
     for (int b = 0; b < 2; b++) {
         p->st[b] = reinterpret_cast<uint4*>(take((size_t)p->n_keys * p->cap[b] * 16));
         p->v[b] = p->kind == OBLIVGM_PRED_RANGE ? take((size_t)p->n_keys * p->cap[b] * 4) : nullptr;
@@ -857,7 +881,7 @@ size_t layout_pred(SgPred* p, const SgCol& c, unsigned char* base, size_t at) {
 
 // Elements per tile of the combine: the CTA width whose waves take the least time (a wave of t
 // threads takes as long as its lookups, or at 384 threads and less as long as an element's chain
-// of PRF words: 100,003 elements in one wave of 768 threads 26 us, in two of 512 46 us), and
+// of PRF words: 100,003 elements in one wave of 768 threads 35 us, in two of 512 46 us), and
 // several elements per thread, so that a tile's barriers are rare, where every SM still gets a
 // few tiles.
 CombineShape combine_shape(uint64_t elems, uint32_t most_preds, int sm_count) {
@@ -883,7 +907,7 @@ uint64_t combine_tiles(const CombineShape& c, SgGroup* groups, uint32_t n_groups
 }
 
 void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* groups, uint32_t n_groups,
-                    const SgFold* folds, uint64_t items, cudaStream_t s) {
+                    const SgFold* folds, bool split, uint64_t items, cudaStream_t s) {
     CombineParams F{};
     std::memcpy(F.rk_prf, ctx->rk_prf, sizeof F.rk_prf);
     F.te0 = ctx->d_te0;
@@ -892,22 +916,23 @@ void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* grou
     F.n_groups = n_groups;
     F.items = items;
     F.per_thread = c.per_thread;
-    launch_after(k_combine, (unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, items), c.threads, kCombineSmem, s, F);
+    launch_after(split ? k_combine<true> : k_combine<false>, (unsigned)std::min<uint64_t>((uint64_t)ctx->sm_count, items), c.threads, kCombineSmem, s, F);
     ctx->launches++;
 }
 
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
-                 size_t scratch_cap, Staged* sg) {
+                 size_t scratch_cap, double wp_seconds, Staged* sg) {
     *sg = Staged{};
     sg->n_keys = (uint32_t)n_keys;
     // columns: a share row of the first set
     std::map<const uint32_t*, uint32_t> col_of;
     std::vector<double> col_steps;                      // seconds per node of one level, over its predicates' keys
     std::vector<uint32_t> pred_col(preds.size());
-    double fused = 0, combine = 0;
+    double fused = 0, combine = 0, chain = 0;
     for (const GroupDesc& G : groups) {
         if (G.n_elems == 0) continue;
         if (G.n_elems > kMaxElems) return false;
+        double group_chain = 0;
         for (uint32_t k = 0; k < G.n_preds; k++) {
             const PredDesc& D = preds[G.pred_begin + k];
             const uint64_t row = (uint64_t)D.attr * G.stride;
@@ -927,7 +952,9 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
             col_steps[ins.first->second] += step;
             fused += step * D.n_bits * (double)G.n_elems;
             combine += (k ? 6 : 3) * kPrfWord * (double)G.n_elems;
+            group_chain += D.n_bits * (D.kind == OBLIVGM_PRED_EQ ? 6 * kDpfLatency : 12 * kDcfLatency);
         }
+        chain = std::max(chain, group_chain);
     }
     if (sg->cols.empty()) return false;
     // per column: dense when the whole domain costs no more than its sorted values
@@ -952,11 +979,18 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         sg->sort_passes = std::max(sg->sort_passes, C.passes);
     }
     staged += kLaunch * (double)(most_stages + 1 + (sg->sort_passes ? 6 + 3 * sg->sort_passes : 0));
-    if (staged + combine > 0.85 * (fused + combine)) { *sg = Staged{}; return false; }
+    // against k_filter, whose threads walk an element's keys one after another (at least its chain),
+    // or the walk-parallel kernel's schedule
+    const double other = wp_seconds > 0 ? wp_seconds : std::max(fused + combine, chain);
+    if (kStagedFixed + 1.05 * staged + 1.5 * combine > 0.95 * other) { *sg = Staged{}; return false; }
 
     choose_tiles(sg);
     size_t col_end = 0;
     for (SgCol& C : sg->cols) col_end = layout_col(&C, nullptr, col_end);
+    uint64_t last_units = 0;
+    for (size_t q = 0; q < preds.size(); q++)
+        last_units += 3 * ((max_values(sg->cols[pred_col[q]]) + 31) / 32);
+    sg->split = last_units < kSplitUnits;
     // predicates in group order, cut into rounds whose states fit kRoundBytes
     size_t at = col_end, most = col_end;
     StagedRound R{};
@@ -981,11 +1015,12 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
             p.dense = C.passes == 0;
             p.col = pred_col[G.pred_begin + k];
             p.slots = 3;
-            p.z_elem = 4;
+            p.parts = sg->split ? D.n_keys / 3 : 1;
+            p.z_elem = 4 * p.parts;
             p.z_slot = 1;
             p.stages = (uint32_t)lev[p.col].size();
             std::copy(lev[p.col].begin(), lev[p.col].end(), p.lev);
-            const uint64_t vals = max_values(p, C);
+            const uint64_t vals = max_values(C);
             p.chunk = kRunBlock;
             while (p.chunk < vals && p.chunk < kMaxChunk) p.chunk <<= 1;
             p.blocks = p.chunk / kRunBlock;
@@ -1013,6 +1048,7 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
             f.radd = D.r[0] + D.r[1] + D.r[2];
             f.mask = p.mask;
             f.index = p.dense ? kIndexDense : kIndexRank;
+            f.more = p.parts - 1;
             sg->preds.push_back(p);
             sg->folds.push_back(f);
             R.n_preds++;
@@ -1123,7 +1159,7 @@ oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned 
         launches += launch_round(ctx, R, reinterpret_cast<const SgPred*>(image + sg.off_preds),
                                  reinterpret_cast<const DevKey*>(image + sg.off_keys), s);
         launch_combine(ctx, sg.shape, reinterpret_cast<const SgGroup*>(image + sg.off_groups) + R.group_begin, R.n_groups,
-                       reinterpret_cast<const SgFold*>(image + sg.off_folds), R.items, s);
+                       reinterpret_cast<const SgFold*>(image + sg.off_folds), sg.split, R.items, s);
     }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "staged launch");
@@ -1169,9 +1205,10 @@ bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint
     p.dense = C.passes == 0;
     p.stages = (uint32_t)lev.size();
     std::copy(lev.begin(), lev.end(), p.lev);
-    const uint64_t vals = max_values(p, C);
+    const uint64_t vals = max_values(C);
     p.z_elem = 1;
     p.z_slot = vals;
+    p.parts = 1;
     p.chunk = kRunBlock;
     while (p.chunk < vals && p.chunk < kMaxChunk) p.chunk <<= 1;
     p.blocks = p.chunk / kRunBlock;
@@ -1226,7 +1263,8 @@ oblivgm_status staged_launch_raw(oblivgm_ctx* ctx, const Staged& sg, const unsig
 oblivgm_status set_staged_attrs() {
     cudaError_t e = cudaFuncSetAttribute(k_stage, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_stage_last, cudaFuncAttributeMaxDynamicSharedMemorySize, kTableBytes);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_combine, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_combine<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_combine<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCombineSmem);
     return e == cudaSuccess ? OBLIVGM_OK : cuda_fail(e, "staged kernel attributes");
 }
 

@@ -65,7 +65,8 @@ struct SgPred {
     uint32_t stages;            // levels lev[s-1] .. lev[s] - 1 belong to stage s; lev[stages - 1] = n
     uint32_t slots;             // outputs per value: 3 servers, or one per key (raw evaluation)
     uint32_t col;
-    uint64_t z_elem, z_slot;    // output word of (value i, slot q): z[i * z_elem + q * z_slot]
+    uint64_t z_elem, z_slot;    // output word of (value i, slot q): z[i * z_elem + q * z_slot], part w of
+                                // it 4 w further
     const uint32_t* u;          // distinct values (sorted), *m of them
     const uint32_t* m;
     uint32_t* z;
@@ -78,7 +79,7 @@ struct SgPred {
     uint32_t* blk;              // [stages - 1][blocks] run counts per block, then exclusive sums
     uint32_t* cnt;              // [stages - 1] runs of each stage
     uint32_t blocks;            // blocks of kRunBlock values in a chunk
-    uint32_t pad;
+    uint32_t parts;             // last stage: work units an output is split into (1, or its keys)
     uint64_t pre_off[kSgMaxStages];
     uint8_t lev[kSgMaxStages + 3];
 };
@@ -99,9 +100,9 @@ struct SgFold {                 // per predicate, next to SgPred
     uint32_t step, lin, prod, attr;
     uint32_t radd, mask;
     uint32_t index;             // kIndexRank, kIndexDense or kIndexElem: which sums are element e's
-    uint32_t pad;
+    uint32_t more;              // further parts of the sums
     const uint32_t* rank;
-    const uint32_t* z;          // four words per value: the three servers' sums
+    const uint32_t* z;          // per value and part four words: the three servers' sums
 };
 constexpr uint32_t kIndexRank = 0;    // those of value rank[e]
 constexpr uint32_t kIndexDense = 1;   // those of value x^, opened from the shares
@@ -115,7 +116,7 @@ struct CombineShape {
 CombineShape combine_shape(uint64_t elems, uint32_t most_preds, int sm_count);
 uint64_t combine_tiles(const CombineShape& c, SgGroup* groups, uint32_t n_groups);
 void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* groups, uint32_t n_groups,
-                    const SgFold* folds, uint64_t items, cudaStream_t s);
+                    const SgFold* folds, bool split, uint64_t items, cudaStream_t s);
 
 struct StagedRound {
     uint32_t pred_begin = 0, n_preds = 0;
@@ -133,6 +134,7 @@ struct Staged {
     std::vector<StagedRound> rounds;
     uint32_t n_keys = 0, sort_tiles = 0, sort_passes = 0;
     CombineShape shape;
+    bool split = false;         // last stages of a unit per key
     bool sort_large = false;    // sort tiles of 4,096 keys instead of 1,024
     bool raw = false;           // a raw evaluation: no combine, its keys are elsewhere on the device
     size_t off_preds = 0, off_folds = 0, off_groups = 0, off_keys = 0, image_bytes = 0;
@@ -140,9 +142,10 @@ struct Staged {
 };
 
 // Plans the staged evaluation of a launch; false when it does not pay (or does not apply) and
-// the fused kernels should run.
+// the fused kernels should run.  wp_seconds: the walk-parallel kernel's time where that is the
+// fused kernel of the launch, else 0.
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
-                 size_t scratch_cap, Staged* out);
+                 size_t scratch_cap, double wp_seconds, Staged* out);
 
 // Sets the pointers for scratch at a device address and builds the descriptor image's bytes.
 void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::vector<unsigned char>* bytes);

@@ -115,3 +115,65 @@ def test_fetch_multi_record_widths(ctx, n, attrs):
     assert m == wm == int(flags.sum())
     for j in range(3):
         assert np.array_equal(from_dev(outs[j][:m]), want[j])
+
+
+@pytest.mark.parametrize("bits,n", [(8, 257), (8, 9000), (13, 4097), (16, 12001), (24, 6000), (32, 5003)])
+def test_small_launches_by_every_route(ctx, bits, n):
+    """Launches of several walk-parallel waves may take the staged evaluation, with a unit per key in
+    its last stage: the same shares as the walk-parallel and the per-element kernel, and as the
+    oracle on a sample."""
+    g = W.rng(bits + n)
+    vals = W.uniform_attrs(g, 2, n, bits)
+    vals[1, ::3] = vals[1, 0]                 # a value that many elements share
+    tab = W.table(vals, bits, g)
+    ctx.load_shares(0, [to_dev(s) for s in tab["shares"]], bits)
+    top = (1 << bits) - 1
+    preds = [W.eq_pred(0, 0, 0, int(vals[0, 1])), W.range_pred(0, 1, 0, top // 5, top // 2, W.COMBINE_OR),
+             W.range_pred(0, 0, 1, 0, top - 1), W.eq_pred(0, 1, 2, int(vals[1, 0])),
+             W.range_pred(0, 1, 2, int(vals[1, 0]), top, W.COMBINE_XOR)]
+    toks = P.keygen(preds, bits, bytes(range(7, 23)))
+    got = []
+    default = ctx.set_walk_parallel((1 << 64) - 1)
+    try:
+        for route in (default, (1 << 64) - 1, 0):
+            ctx.set_walk_parallel(route)
+            outs = [[torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(3)] for _ in range(3)]
+            ctx.filter_and_combine(5, toks, outs)
+            ctx.sync()
+            got.append([np.stack([from_dev(t) for t in grp]) for grp in outs])
+    finally:
+        ctx.set_walk_parallel(default)
+    idx = np.unique(np.concatenate([np.arange(0, n, max(1, n // 200)), [n - 1]]))
+    for grp in range(3):
+        assert np.array_equal(got[0][grp], got[1][grp]) and np.array_equal(got[0][grp], got[2][grp]), grp
+        want = oracle.filter_group(toks, 5, PRF, [(tab["shares"], bits)], grp, idx, threads=4)
+        assert np.array_equal(got[0][grp][:, idx], want), grp
+
+
+def test_small_staged_plan_under_capture(ctx):
+    """A prepared plan of a small staged launch, captured into a CUDA graph (its kernels are
+    programmatic dependents), replays to the shares of the direct call."""
+    g = W.rng(77)
+    n, bits = 9000, 16
+    vals = W.uniform_attrs(g, 2, n, bits)
+    tab = W.table(vals, bits, g)
+    ctx.load_shares(0, [to_dev(s) for s in tab["shares"]], bits)
+    preds = [W.eq_pred(0, 0, 0, int(vals[0, 1])), W.range_pred(0, 1, 0, 100, 9000)]
+    toks = P.keygen(preds, bits, bytes(16))
+    outs = [[torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(3)]]
+    ctx.filter_and_combine(5, toks, outs)
+    ctx.sync()
+    want = [t.clone() for t in outs[0]]
+    plan = ctx.plan_create([5], [toks], [outs])
+    for t in outs[0]:
+        t.zero_()
+    torch.cuda.synchronize()
+    graph, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=s):
+        ctx.plan_launch(plan, stream=s.cuda_stream)
+    for _ in range(2):
+        graph.replay()
+    torch.cuda.synchronize()
+    ctx.plan_destroy(plan)
+    for a, b in zip(outs[0], want):
+        assert torch.equal(a, b)
