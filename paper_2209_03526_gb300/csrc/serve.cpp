@@ -273,11 +273,18 @@ oblivgm_status oblivgm_release(oblivgm_ctx* ctx, uint64_t ticket) {
     // Work that the caller queued on the default stream before this call (a copy of the result) may
     // not have run yet, while the next batch on the serve stream could already reuse the memory:
     // the release waits for it on the device.
+    // A capture under way, which forbids the default stream, is left alone.
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     cudaEvent_t read = nullptr;
-    if (cudaEventCreateWithFlags(&read, cudaEventDisableTiming) == cudaSuccess) {
+    if (cudaStreamIsCapturing(cudaStreamLegacy, &capture) == cudaSuccess &&
+        cudaEventCreateWithFlags(&read, cudaEventDisableTiming) == cudaSuccess) {
         if (cudaEventRecord(read, cudaStreamLegacy) == cudaSuccess) cudaStreamWaitEvent(S.streams[q->stream], read, 0);
         cudaEventDestroy(read);
     }
+    cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
     for (uint32_t* p : q->outs)
         if (p) cudaFreeAsync(p, S.streams[q->stream]);
     S.cv_work.notify_all();
