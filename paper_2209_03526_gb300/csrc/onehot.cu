@@ -16,8 +16,8 @@
 //  * the dot pass, one streaming pass over an attribute column's three share rows for
 //    up to 4 predicates on that column: k_onehot_dots_pipe (D >= 2^12, persistent,
 //    rows staged by per-lane cp.async, warps splitting the rows, each lane holding its
-//    slice of the half vectors in registers) or k_onehot_dots (smaller D); parities
-//    are XOR-reduced over the warp and each server's bit written packed;
+//    slice of the half vectors in registers; parities are XOR-reduced over the warp and
+//    each server's bit written packed) or k_onehot_dots (smaller D, a thread per element);
 //  * k_onehot_fold: every group in one launch, each element's bits re-shared in
 //    binary RSS and folded in token order on whole 32-element words (one PRF AES
 //    block from the shared-memory T-tables serves 128 elements); results are packed
@@ -169,114 +169,76 @@ struct DotParams {
     uint32_t pow2[32];            // pow2[i] = 2^i (read at run time by the staged pass)
 };
 
-// The unstaged pass, launched for domains below 2^12 and general in W.  One CTA per 32
-// elements (one packed output word).  The CTA's warps split each share row: with
-// W >= 128 words warp q covers words [128 q, 128 q + 128) of every row in steps of
-// W' = 128 * warps (one uint4 per lane when W' = W); with W < 128 one warp reads the row
-// word by word.  A lane keeps its slice of the predicates' half vectors in registers for
-// all 32 elements and streams 8 elements' rows at a time; its parity bits of the 32
-// elements are XORed over the warp by shuffles and over the warps through shared memory.
-constexpr int kDotBatch = 8;
+// The pass for rows of W <= 64 words (D < 2^12).  A thread takes one element: its rows are a few
+// sectors, the predicates' half vectors come from shared memory (the same word for all lanes),
+// every (predicate, server) has one accumulator over the whole row, and a ballot of the parities
+// is the packed output word.  A warp per row left most lanes without a word: the query of four
+// predicates on 500,000 elements took 311 us at n = 6 and 327 at n = 10, now 42 and 107; 200,000
+// at n = 11 152 -> 98 us.  Short rows leave the launches and EvalAll (30 us), longer ones the row
+// loads, each lane its own lines.
+constexpr int kDotBatch = 8;                  // elements of a step of the staged pass
+constexpr int kDotThreads = 256;
+constexpr uint32_t kDotMaxWords = 64;
 
-__device__ __forceinline__ void slice4(const uint32_t* row, uint32_t W, bool vec, uint32_t w0, uint32_t lane,
-                                       uint32_t out[4]) {
-    if (vec) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(row + w0));
-        out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
+template <int VEC>
+__device__ __forceinline__ void load_words(const uint32_t* p, uint32_t v[VEC]) {
+    if constexpr (VEC == 4) {
+        const uint4 q = *reinterpret_cast<const uint4*>(p);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
     } else {
-#pragma unroll
-        for (int r = 0; r < 4; r++) out[r] = lane + 32u * r < W ? __ldg(row + lane + 32u * r) : 0u;
+        v[0] = *p;
     }
 }
 
-__global__ void __launch_bounds__(512) k_onehot_dots(const __grid_constant__ DotParams P) {
-    __shared__ uint32_t zs[16][kDotPreds][3][2];      // per warp: element masks per (pred, share, half)
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+template <int VEC>     // words per load: 4 where rows are whole 16-byte groups, else 1
+__global__ void __launch_bounds__(kDotThreads) k_onehot_dots(const __grid_constant__ DotParams P) {
+    __shared__ __align__(16) uint32_t hs[kDotPreds * 6 * kDotMaxWords];    // [predicate][server][half][word]
     const uint32_t W = P.words, np = P.n_preds;
-    const bool vec = W >= 128;
-    const uint64_t nwords = (P.n_elems + 31) / 32;
-    const uint64_t wd = blockIdx.x;
-    const uint64_t base = wd * 32;
-    // lane 0 of each warp owns the warp's slots: cleared here, XORed into below
-    if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < kDotPreds; k++)
-#pragma unroll
-            for (int j = 0; j < 3; j++) zs[warp][k][j][0] = zs[warp][k][j][1] = 0;
+    for (uint32_t t = threadIdx.x; t < np * 6 * W; t += kDotThreads) {
+        const uint32_t k = t / (6 * W), r = t - k * 6 * W;
+        hs[t] = P.hv[(uint64_t)P.half_base[k] * W + r];
     }
-    // a lane's words: w0 .. w0 + 3 (vector path) or lane + 32 r (scalar path); the vector
-    // path loops over the row in steps of 128 * warps words
-    for (uint32_t w0 = vec ? warp * 128 + lane * 4 : 0; w0 < (vec ? W : 1u); w0 += vec ? warps * 128 : 1u) {
+    __syncthreads();
+    const uint64_t nwords = (P.n_elems + 31) / 32;
+    for (uint64_t first = (uint64_t)blockIdx.x * kDotThreads; first < P.n_elems; first += (uint64_t)gridDim.x * kDotThreads) {
+        const uint64_t e = first + threadIdx.x, wd = e / 32;
+        uint32_t acc[kDotPreds][3];
 #pragma unroll
-        for (int j = 0; j < 3; j++) {
-            uint32_t h[kDotPreds][2][4];
+        for (int k = 0; k < kDotPreds; k++) acc[k][0] = acc[k][1] = acc[k][2] = 0;
+        if (e < P.n_elems) {
 #pragma unroll
-            for (int k = 0; k < kDotPreds; k++) {
-                if ((uint32_t)k < np) {
-                    slice4(P.hv + (uint64_t)(P.half_base[k] + j * 2) * W, W, vec, w0, lane, h[k][0]);
-                    slice4(P.hv + (uint64_t)(P.half_base[k] + ((j + 2) % 3) * 2 + 1) * W, W, vec, w0, lane, h[k][1]);
-                } else {
+            for (int j = 0; j < 3; j++) {
+                const uint32_t* row = P.share[j] + e * W;
+                // share j meets server j's first half and server j - 1's second
+                const uint32_t i0 = (uint32_t)j, i1 = (uint32_t)(j + 2) % 3;
+#pragma unroll 2
+                for (uint32_t w = 0; w < W; w += VEC) {
+                    uint32_t v[VEC];
+                    load_words<VEC>(row + w, v);
 #pragma unroll
-                    for (int r = 0; r < 4; r++) h[k][0][r] = h[k][1][r] = 0;
-                }
-            }
-            // Lane-local parity bits of the 32 elements, XOR-reduced over the warp below.
-            // Element c = 4 q + f sits at bit 8 f + q: a batch's popcounts (at most 32 each)
-            // are added into the bytes of two words by shift-adds, and their low bits are
-            // moved into place with one mask and one shift per four elements.
-            uint32_t pl[kDotPreds][2];
+                    for (int k = 0; k < kDotPreds; k++) {
+                        if ((uint32_t)k >= np) break;
+                        uint32_t ha[VEC], hb[VEC];
+                        load_words<VEC>(hs + (k * 6 + 2 * i0) * W + w, ha);
+                        load_words<VEC>(hs + (k * 6 + 2 * i1 + 1) * W + w, hb);
 #pragma unroll
-            for (int k = 0; k < kDotPreds; k++) pl[k][0] = pl[k][1] = 0;
-            for (uint32_t c0 = 0; c0 < 32; c0 += kDotBatch) {
-                uint32_t v[kDotBatch][4];
-#pragma unroll
-                for (int b = 0; b < kDotBatch; b++) {
-                    const uint64_t e = base + c0 + b;
-                    if (e < P.n_elems) slice4(P.share[j] + e * W, W, vec, w0, lane, v[b]);
-                    else v[b][0] = v[b][1] = v[b][2] = v[b][3] = 0;
-                }
-#pragma unroll
-                for (int k = 0; k < kDotPreds; k++) {
-                    if ((uint32_t)k >= np) break;
-#pragma unroll
-                    for (int hh = 0; hh < 2; hh++) {
-                        uint32_t cnt[kDotBatch / 4] = {};
-#pragma unroll
-                        for (int b = 0; b < kDotBatch; b++) {
-                            const uint32_t a = (v[b][0] & h[k][hh][0]) ^ (v[b][1] & h[k][hh][1]) ^
-                                               (v[b][2] & h[k][hh][2]) ^ (v[b][3] & h[k][hh][3]);
-                            cnt[b / 4] += (uint32_t)__popc(a) << (8 * (b % 4));
+                        for (int r = 0; r < VEC; r++) {
+                            acc[k][i0] ^= v[r] & ha[r];
+                            acc[k][i1] ^= v[r] & hb[r];
                         }
-#pragma unroll
-                        for (int q = 0; q < kDotBatch / 4; q++)
-                            pl[k][hh] ^= (cnt[q] & 0x01010101u) << (c0 / 4 + q);
                     }
                 }
             }
+        }
 #pragma unroll
-            for (int k = 0; k < kDotPreds; k++) {
-                if ((uint32_t)k >= np) break;
+        for (int k = 0; k < kDotPreds; k++) {
+            if ((uint32_t)k >= np) break;
 #pragma unroll
-                for (int hh = 0; hh < 2; hh++) {
-                    uint32_t m = pl[k][hh];
-#pragma unroll
-                    for (int off = 16; off > 0; off >>= 1) m ^= __shfl_xor_sync(0xFFFFFFFFu, m, off);
-                    if (lane == 0) zs[warp][k][j][hh] ^= m;
-                }
+            for (int i = 0; i < 3; i++) {
+                const uint32_t z = __ballot_sync(0xFFFFFFFFu, __popc(acc[k][i]) & 1);
+                if ((threadIdx.x & 31) == 0 && wd < nwords) P.zbits[k][(uint64_t)i * nwords + wd] = z;
             }
         }
-    }
-    __syncthreads();
-    // server i: first half with share i, second half with share i + 1; element c leaves
-    // bit 8 (c % 4) + c / 4 for bit c of the packed output word
-    if (threadIdx.x < np * 3) {
-        const uint32_t k = threadIdx.x / 3, i = threadIdx.x % 3;
-        uint32_t zp = 0;
-        for (uint32_t q = 0; q < warps; q++) zp ^= zs[q][k][i][0] ^ zs[q][k][(i + 1) % 3][1];
-        uint32_t z = 0;
-#pragma unroll
-        for (uint32_t c = 0; c < 32; c++) z |= ((zp >> (8 * (c % 4) + c / 4)) & 1u) << c;
-        P.zbits[k][(uint64_t)i * nwords + wd] = z;
     }
 }
 
@@ -497,7 +459,11 @@ void launch_dots(const DotParams& D, uint64_t nwords, int sm_count, cudaStream_t
         case 4: return launch_dots_pipe<4>(D, nwords, sm_count, s);
         case 8: return launch_dots_pipe<8>(D, nwords, sm_count, s);
         case 16: return launch_dots_pipe<16>(D, nwords, sm_count, s);
-        default: k_onehot_dots<<<(unsigned)nwords, 32, 0, s>>>(D);      // D < 2^12: one warp's words at most
+        default: {                                     // D < 2^12
+            const unsigned grid = (unsigned)std::min<uint64_t>((D.n_elems + kDotThreads - 1) / kDotThreads, 8ull * sm_count);
+            if (D.words % 4 == 0) k_onehot_dots<4><<<grid, kDotThreads, 0, s>>>(D);
+            else k_onehot_dots<1><<<grid, kDotThreads, 0, s>>>(D);
+        }
     }
 }
 
