@@ -1103,19 +1103,23 @@ void apply_test_expiry(oblivgm_ctx* ctx, FilterParams* P) {
     ctx->test_expire_next = false;
 }
 
+// Whether work on the stream is being recorded into a graph (also the legacy stream while another
+// one captures).  The staged evaluation's descriptors go up from a host buffer that lives only for
+// the call, so a replay would copy freed memory into them: a call under capture takes a fused
+// kernel, and oblivgm_plan_* the staged evaluation.
+bool under_capture(cudaStream_t st) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) == cudaSuccess) return capture != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
 // The staged evaluation of a plan: a small descriptor image and a scratch block, both stream
 // ordered.  *ran is false when the device has no room for the scratch: the fused kernel, which
 // needs next to none, runs then.
 oblivgm_status launch_staged(oblivgm_ctx* ctx, Plan& plan, cudaStream_t st, bool* ran) {
     *ran = false;
-    if (plan.wp) {
-        // a small launch that is being captured stays one kernel without scratch
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            return OBLIVGM_OK;
-        }
-    }
+    if (under_capture(st)) return OBLIVGM_OK;
     unsigned char *image = nullptr, *scratch = nullptr;
     const oblivgm_status as =
         ws_alloc(ctx, reinterpret_cast<void**>(&image), plan.sg.image_bytes, st, "workspace allocation");
@@ -1403,7 +1407,7 @@ static oblivgm_status eval_batch(oblivgm_ctx* ctx, uint32_t kind, const uint8_t*
     // all keys at all points: the walks share tree nodes (staged.cu) where that pays and there
     // is room for it
     Staged sg;
-    if (all && staged_plan_raw(kind, (uint32_t)n, n_keys, points, n_points, ctx->scratch_cap, &sg)) {
+    if (all && staged_plan_raw(kind, (uint32_t)n, n_keys, points, n_points, ctx->scratch_cap, &sg) && !under_capture(s)) {
         unsigned char* scratch = nullptr;
         const size_t img = (sg.image_bytes + 255) / 256 * 256;
         const cudaError_t ae =
