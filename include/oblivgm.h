@@ -594,7 +594,9 @@ oblivgm_status oblivgm_serve_stats(oblivgm_ctx* ctx, uint64_t* admitted, uint64_
 /* Autotuned launch shape of the fused evaluation kernel: threads per CTA and
  * elements per thread ("paths per thread").  oblivgm_autotune times the
  * candidates on a synthetic table and keeps the fastest; the choice is
- * reported (and may be forced with oblivgm_set_schedule, 0 = keep). */
+ * reported (and may be forced with oblivgm_set_schedule, 0 = keep).  It is the
+ * shape of the per-element kernel; the walk-parallel kernel and the staged
+ * evaluation (oblivgm_set_walk_parallel) have shapes of their own. */
 oblivgm_status oblivgm_autotune(oblivgm_ctx* ctx, uint32_t* threads, uint32_t* elems_per_thread);
 oblivgm_status oblivgm_set_schedule(oblivgm_ctx* ctx, uint32_t threads, uint32_t elems_per_thread);
 
@@ -602,10 +604,13 @@ oblivgm_status oblivgm_set_schedule(oblivgm_ctx* ctx, uint32_t threads, uint32_t
  * most `max_elems` elements in all is evaluated by the walk-parallel kernel,
  * one thread per key walk (six DPF or twelve DCF walks of an element side by
  * side), instead of one thread per element.  Both kernels give identical
- * output.  Default: 128 x the SM count, less the batches of several waves whose
- * elements' shared tree nodes make the staged evaluation faster; 0 turns the
- * walk-parallel kernel off, UINT64_MAX uses it for every batch.  `previous` (may be NULL) receives the
- * setting it replaces.  Applies to oblivgm_filter_and_combine,
+ * output.  Default: 128 x the SM count, and a batch of any size whose elements
+ * share enough tree nodes goes to the staged evaluation, with the same output,
+ * where that is estimated faster.  A value of the caller's own is followed as
+ * it is: batches up to it are walk-parallel (UINT64_MAX: every batch), larger
+ * ones stay the library's choice, and 0 evaluates every batch with one thread
+ * per element.  `previous` (may be NULL) receives the setting it replaces;
+ * setting the default again gives the choice back.  Applies to oblivgm_filter_and_combine,
  * oblivgm_filter_batch, the no-alloc entry point, plans created afterwards and
  * the serving loop.  Errors: EINVAL for a NULL context. */
 oblivgm_status oblivgm_set_walk_parallel(oblivgm_ctx* ctx, uint64_t max_elems, uint64_t* previous);

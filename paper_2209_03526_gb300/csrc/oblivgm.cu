@@ -1018,7 +1018,9 @@ oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& ta
                            uint32_t* const* const* outs, bool staged_ok, Plan* plan) {
     plan->staged = false;
     const oblivgm_status s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, ctx, plan);
-    if (s != OBLIVGM_OK || (plan->wp && (ctx->wp_fixed || ctx->wp_tile))) return s;
+    // what the caller asked for is what runs: the walk-parallel kernel up to a switch-over or in a
+    // tile of its own, the per-element kernel with a switch-over of 0
+    if (s != OBLIVGM_OK || (plan->wp ? ctx->wp_fixed || ctx->wp_tile : ctx->wp_max_elems == 0)) return s;
     // launches share tree nodes between elements where that pays (5 predicates on 12,000 elements,
     // n = 16: 337 us walk-parallel, 160 staged), but for one wave of walk-parallel tiles, which the
     // staged launches alone outlast; the key-staging expiry hook is about the fused kernels' waits

@@ -120,7 +120,7 @@ struct oblivgm_ctx {
     uint32_t threads = 768;          // the autotuner's pick on GB300 (256 x 4 spills)
     uint32_t elems_per_thread = 1;
     uint64_t wp_max_elems = 0;       // batches with at most this many elements in all run walk-parallel
-    bool wp_fixed = false;           // that number was set by the caller: no staged evaluation below it
+    bool wp_fixed = false;           // that number was set by the caller: no staged evaluation up to it (0: none at all)
     size_t scratch_cap = 0;          // most scratch a staged evaluation may take
     cudaMemPool_t scratch_pool = nullptr;   // its stream-ordered scratch; keeps kScratchKeep bytes between calls
     uint32_t wp_tile = 0;            // walk-parallel elements per tile; 0 = chosen per launch

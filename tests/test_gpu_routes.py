@@ -1,0 +1,70 @@
+"""Which kernels a filter launch takes: what a caller asks for is what runs."""
+import numpy as np
+import pytest
+
+import oracle
+import workload as W
+from tests._helpers import PRF, alloc_outs, from_dev, load_tables, oracle_group
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+P = pytest.importorskip("paper_2209_03526_gb300")
+
+ALWAYS = (1 << 64) - 1
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c = P.Context(0, prf_keys=PRF)
+    yield c
+    c.close()
+
+
+def _workload(n, bits=32, seed=5):
+    g = W.rng(seed)
+    wl = {"tables": [W.table(W.uniform_attrs(g, 2, n, bits), bits, g)]}
+    v = wl["tables"][0]["values"]
+    wl["preds"] = [W.eq_pred(0, 0, 0, int(v[0, n // 2])), W.range_pred(0, 1, 0, 5, (1 << bits) // 2, combine=P.COMBINE_OR),
+                   W.range_pred(0, 0, 1, 9, (1 << bits) - 1)]
+    return wl
+
+
+def _shares(outs):
+    return [np.stack([from_dev(t) for t in grp]) for grp in outs]
+
+
+@pytest.mark.parametrize("setting", [0, ALWAYS])
+@pytest.mark.parametrize("n", [1, 3333, 25000])
+def test_a_caller_s_switch_over_is_followed(ctx, n, setting):
+    """0: one thread per element for every batch, UINT64_MAX: walk-parallel; one launch either way,
+    as a call and as a plan, and the shares of the library's own choice."""
+    wl = _workload(n)
+    load_tables(ctx, wl)
+    toks = P.keygen(wl["preds"], 32, bytes(range(16)))
+    own = alloc_outs(wl)
+    ctx.filter_and_combine(7, toks, own)
+    ctx.sync()
+    prev = ctx.set_walk_parallel(setting)
+    try:
+        outs = alloc_outs(wl)
+        before = ctx.launch_count()
+        ctx.filter_and_combine(7, toks, outs)
+        ctx.sync()
+        assert ctx.launch_count() - before == 1
+        planned = alloc_outs(wl)
+        plan = ctx.plan_create([7], [toks], [planned])
+        assert ctx.plan_describe(plan)["kernel"] == ("k_filter_wp" if setting else "k_filter")
+        before = ctx.launch_count()
+        ctx.plan_launch(plan)
+        ctx.sync()
+        assert ctx.launch_count() - before == 1
+        ctx.plan_destroy(plan)
+    finally:
+        ctx.set_walk_parallel(prev)
+    idx = np.unique([0, n // 2, n - 1])
+    for grp, (a, b, c) in enumerate(zip(_shares(own), _shares(outs), _shares(planned))):
+        assert np.array_equal(a, b) and np.array_equal(a, c), grp
+        assert np.array_equal(a[:, idx], oracle_group(oracle, wl, toks, 7, grp, idx)), grp
