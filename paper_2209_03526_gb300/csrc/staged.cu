@@ -777,6 +777,8 @@ constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, 
 // a level step of a thread on its own, and what a small staged evaluation takes on top
 constexpr double kDpfLatency = 0.57e-6, kDcfLatency = 0.92e-6, kStagedFixed = 12e-6;
 constexpr double kSortKeyPass = 12e-12;
+// what a staged raw evaluation takes beside its launches: scratch, descriptors and their copy
+constexpr double kRawFixed = 3.0e-6;
 constexpr uint64_t kMaxElems = 1ull << 28;
 constexpr uint32_t kMaxChunk = 1u << 22;      // distinct values evaluated together
 constexpr int kMaxDenseBits = 24;
@@ -1179,10 +1181,16 @@ bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint
     const bool dcf = kind == OBLIVGM_KEY_DCF;
     // at most 64 keys a round; a round's launches are its own, the sort is shared
     const double rounds = (n_keys + 63) / 64, step = n_keys / rounds * (dcf ? kDcfStep : kDpfStep);
+    // the per-item kernel's time, less a margin, is what a staged evaluation may take (2 DCF keys at
+    // 15,000 points, n = 8: per item 17.5 us, staged 20.3; at 30,000 points 32.9 and 19.2); most
+    // small calls are decided by the launches alone
+    const double other = 0.95 * rounds * step * n_bits * (double)n_points + kLaunch;
+    const bool may_be_dense = (int)n_bits <= kMaxDenseBits;
+    const double sort = (double)C.n * kSortKeyPass * C.passes + kLaunch * (3 + 3 * rounds + 3 * C.passes);
+    if (kRawFixed + 2 * rounds * kLaunch + (may_be_dense ? 0 : sort) > other) return false;
     std::vector<uint8_t> lev, ld;
-    double cs = rounds * choose_stages((double)C.n, false, (int)n_bits, step, &lev) +
-                (double)C.n * kSortKeyPass * C.passes + kLaunch * (3 + 3 * rounds + 3 * C.passes);
-    if ((int)n_bits <= kMaxDenseBits) {
+    double cs = rounds * choose_stages((double)C.n, false, (int)n_bits, step, &lev) + sort;
+    if (may_be_dense) {
         const double cd = rounds * choose_stages(0, true, (int)n_bits, step, &ld);
         if (cd <= cs) {
             cs = cd;
@@ -1190,7 +1198,7 @@ bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint
             lev = ld;
         }
     }
-    if (cs + rounds * kLaunch > 0.85 * (rounds * step * n_bits * (double)n_points + kLaunch)) return false;
+    if (kRawFixed + cs + rounds * kLaunch > other) return false;
     sg->raw = true;
     sg->sort_passes = C.passes;
     sg->cols.push_back(C);

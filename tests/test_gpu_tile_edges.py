@@ -177,3 +177,29 @@ def test_small_staged_plan_under_capture(ctx):
     ctx.plan_destroy(plan)
     for a, b in zip(outs[0], want):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dcf", [False, True])
+@pytest.mark.parametrize("points", [1, 64, 65, 152 * 64 + 1, 152 * 768, 152 * 768 + 1, 2 * 152 * 768 + 33])
+def test_per_item_evaluation_in_even_waves(ctx, dcf, points):
+    """Points with a key each, around one item per warp and per thread of every SM and two full
+    waves: a sample against the oracle, and on every point the pair's two keys add up to beta where
+    x = alpha or x < alpha."""
+    g, bits = np.random.default_rng(points), 9
+    kind, L = (P.KEY_DCF, 28 + 24 * bits) if dcf else (P.KEY_DPF, 28 + 20 * bits)
+    x = g.integers(0, 1 << bits, points, dtype=np.uint64).astype(np.uint32)
+    alpha, beta = int(x[points // 2]), 0x9E3779B1
+    keys = torch.zeros(2 * L, dtype=torch.uint8, device="cuda")
+    ctx.keygen_device(kind, bits, to_dev(np.uint32([alpha])), to_dev(np.uint32([beta])), SEED, keys)
+    raw, got = keys.cpu().numpy().tobytes(), []
+    idx = np.unique([0, points - 1, points // 2, *g.integers(0, points, 16)])
+    for k in range(2):
+        out = torch.full((points,), -1, dtype=torch.int32, device="cuda")
+        of = torch.full((points,), k, dtype=torch.int32, device="cuda")
+        ctx.eval_device_keys(kind, bits, keys, 2, to_dev(x), out, key_of_point=of)
+        ctx.sync()
+        got.append(from_dev(out))
+        want = oracle.eval_many(raw[k * L:(k + 1) * L], x[idx], oracle.KIND_DCF if dcf else oracle.KIND_DPF)
+        assert np.array_equal(got[k][idx], want)
+    hit = x < alpha if dcf else x == alpha
+    assert np.array_equal(got[0] + got[1], np.where(hit, np.uint32(beta), np.uint32(0)))
