@@ -774,8 +774,10 @@ __global__ void __launch_bounds__(256) k_gather_raw(const __grid_constant__ Gath
 // GB300 figures the plan weighs: a DPF / DCF level step of one key at the T-table lookup rate,
 // a PRF word, a launch (with its table fill) and a key of a sort pass.
 constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, kLaunch = 4.0e-6;
-// a level step of a thread on its own, and what a small staged evaluation takes on top
-constexpr double kDpfLatency = 0.57e-6, kDcfLatency = 0.92e-6, kStagedFixed = 12e-6;
+// a level step of a thread on its own, and what a staged evaluation and k_filter take on top (of 564
+// plans of 1,000 to 100,000 elements, one to five predicates and n = 8 to 32, timed both ways,
+// the estimates with these pick the slower one, by 5 % and more, in 35, each by staying fused)
+constexpr double kDpfLatency = 0.57e-6, kDcfLatency = 0.92e-6, kStagedFixed = 8e-6, kFusedFixed = 20e-6;
 constexpr double kSortKeyPass = 12e-12;
 // what a staged raw evaluation takes beside its launches: scratch, descriptors and their copy
 constexpr double kRawFixed = 3.0e-6;
@@ -971,19 +973,20 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         if (n <= kMaxDenseBits) cd = choose_stages(0, true, n, col_steps[c], &ld);
         const double sort = (double)C.n * kSortKeyPass * C.passes;
         const double cs = choose_stages((double)C.n, false, n, col_steps[c], &lev[c]) + sort;
-        if (cd <= cs + 6 * kLaunch) {
+        const bool dense = cd <= cs + 6 * kLaunch;
+        if (dense) {
             C.passes = 0;
             lev[c] = ld;
         }
         // the columns' launches are shared, so they are counted once below
-        staged += std::min(cd, cs) - kLaunch * (double)lev[c].size();
+        staged += (dense ? cd : cs) - kLaunch * (double)lev[c].size();
         most_stages = std::max(most_stages, lev[c].size());
         sg->sort_passes = std::max(sg->sort_passes, C.passes);
     }
     staged += kLaunch * (double)(most_stages + 1 + (sg->sort_passes ? 6 + 3 * sg->sort_passes : 0));
     // against k_filter, whose threads walk an element's keys one after another (at least its chain),
     // or the walk-parallel kernel's schedule
-    const double other = wp_seconds > 0 ? wp_seconds : std::max(fused + combine, chain);
+    const double other = wp_seconds > 0 ? wp_seconds : kFusedFixed + std::max(fused + combine, chain);
     if (kStagedFixed + 1.05 * staged + 1.5 * combine > 0.95 * other) { *sg = Staged{}; return false; }
 
     choose_tiles(sg);

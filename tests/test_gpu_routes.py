@@ -68,3 +68,21 @@ def test_a_caller_s_switch_over_is_followed(ctx, n, setting):
     for grp, (a, b, c) in enumerate(zip(_shares(own), _shares(outs), _shares(planned))):
         assert np.array_equal(a, b) and np.array_equal(a, c), grp
         assert np.array_equal(a[:, idx], oracle_group(oracle, wl, toks, 7, grp, idx)), grp
+
+
+def test_a_dense_column_is_weighed_by_what_it_costs(ctx):
+    """Two equality predicates on 5,000 16-bit values: all 2^16 nodes of the last levels cost twice
+    the walk-parallel kernel, though the sorted values alone, without their sort, would not."""
+    n = 5000
+    wl = {"tables": [W.table(W.uniform_attrs(W.rng(8), 2, n, 16), 16, W.rng(9))]}
+    v = wl["tables"][0]["values"]
+    wl["preds"] = [W.eq_pred(0, 0, 0, int(v[0, 1])), W.eq_pred(0, 1, 1, int(v[1, n - 1]))]
+    load_tables(ctx, wl)
+    toks = P.keygen(wl["preds"], 16, bytes(range(2, 18)))
+    outs = alloc_outs(wl)
+    before = ctx.launch_count()
+    ctx.filter_and_combine(8, toks, outs)
+    ctx.sync()
+    assert ctx.launch_count() - before == 1
+    for grp, got in enumerate(_shares(outs)):
+        assert np.array_equal(got, oracle_group(oracle, wl, toks, 8, grp, np.arange(n))), grp
