@@ -86,3 +86,25 @@ def test_a_dense_column_is_weighed_by_what_it_costs(ctx):
     assert ctx.launch_count() - before == 1
     for grp, got in enumerate(_shares(outs)):
         assert np.array_equal(got, oracle_group(oracle, wl, toks, 8, grp, np.arange(n))), grp
+
+
+@pytest.mark.parametrize("sizes", [(2500, 2500), (2700, 2700), (3040, 1), (5200,), (9728,)])
+def test_equality_groups_of_one_wave(ctx, sizes):
+    """Groups of equality predicates alone, of more elements than 32 a CTA and at most 64: one wave of
+    tiles, and the oracle's shares."""
+    g = W.rng(sum(sizes))
+    wl = {"tables": [W.table(W.uniform_attrs(g, 1, n, 24), 24, g) for n in sizes]}
+    wl["preds"] = [W.eq_pred(t, 0, t, int(wl["tables"][t]["values"][0, -1])) for t in range(len(sizes))]
+    load_tables(ctx, wl)
+    toks = P.keygen(wl["preds"], 24, bytes(range(4, 20)))
+    outs = alloc_outs(wl)
+    plan = ctx.plan_create([9], [toks], [outs])
+    shape = ctx.plan_describe(plan)
+    before = ctx.launch_count()
+    ctx.plan_launch(plan)
+    ctx.sync()
+    launches = ctx.launch_count() - before
+    ctx.plan_destroy(plan)
+    assert launches == 1 and shape["kernel"] == "k_filter_wp" and shape["items"] == shape["grid"]
+    for grp, got in enumerate(_shares(outs)):
+        assert np.array_equal(got, oracle_group(oracle, wl, toks, 9, grp, np.arange(sizes[grp]))), grp
