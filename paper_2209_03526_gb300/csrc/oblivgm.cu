@@ -1023,16 +1023,23 @@ oblivgm_status plan_queries(const std::map<uint32_t, Table>& tables, uint32_t n_
     return OBLIVGM_OK;
 }
 
-// no staged evaluation is faster (n = 8, one predicate, dense: 13 to 17 us; sorted ones from 40 us)
-constexpr double kStagedLeastSeconds = 24e-6;
+// Whether a launch may be staged, and as what: a call allocates and uploads on the way, which a
+// prepared plan has behind it.  No staged evaluation is faster than the least one (n = 8, one
+// predicate, dense: a plan 12 to 17 us, a call 25 to 28; sorted ones from 40 us), so that no
+// walk-parallel launch below that is weighed against it.
+struct StagedUse {
+    bool ok = false;
+    double fixed = 0, least = 0;      // seconds beside its kernels, and of the least one
+};
+constexpr StagedUse kNotStaged{}, kStagedCall{true, 12e-6, 24e-6}, kStagedPlan{true, 8e-6, 16e-6};
 
 // Plan a batch for the fused kernel in the context's launch shape; a batch whose groups
 // hold at most ctx->wp_max_elems elements in all goes to the walk-parallel kernel instead,
-// in tiles of kWpElems elements, and either to the staged evaluation (staged_ok) where its
+// in tiles of kWpElems elements, and either to the staged evaluation where its
 // estimate is below that kernel's.
 oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& tables, uint32_t n_queries,
                            const uint32_t* query_ids, const ParsedQuery* parsed, const uint32_t* n_groups,
-                           uint32_t* const* const* outs, bool staged_ok, Plan* plan) {
+                           uint32_t* const* const* outs, const StagedUse& use, Plan* plan) {
     plan->staged = false;
     const oblivgm_status s = plan_queries(tables, n_queries, query_ids, parsed, n_groups, outs, ctx, plan);
     // what the caller asked for is what runs: the walk-parallel kernel up to a switch-over or in a
@@ -1041,9 +1048,9 @@ oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& ta
     // launches share tree nodes between elements where that pays (5 predicates on 12,000 elements,
     // n = 16: 337 us walk-parallel, 160 staged), but for one wave of walk-parallel tiles, which the
     // staged launches alone outlast; the key-staging expiry hook is about the fused kernels' waits
-    if (staged_ok && !ctx->test_expire_next && (!plan->wp || plan->wp_seconds > kStagedLeastSeconds))
+    if (use.ok && !ctx->test_expire_next && (!plan->wp || plan->wp_seconds > use.least))
         plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap,
-                                   plan->wp ? plan->wp_seconds : 0.0, &plan->sg);
+                                   use.fixed, plan->wp ? plan->wp_seconds : 0.0, &plan->sg);
     return OBLIVGM_OK;
 }
 
@@ -1193,7 +1200,7 @@ oblivgm_status launch_parsed(oblivgm_ctx* ctx, uint32_t n_queries, const uint32_
                              const ParsedQuery* parsed, const uint32_t* n_groups, uint32_t* const* const* outs,
                              const std::map<uint32_t, Table>& tables, cudaStream_t st, bool staged_ok) {
     Plan plan;
-    oblivgm_status s = plan_filter(ctx, tables, n_queries, query_ids, parsed, n_groups, outs, staged_ok, &plan);
+    oblivgm_status s = plan_filter(ctx, tables, n_queries, query_ids, parsed, n_groups, outs, staged_ok ? kStagedCall : kNotStaged, &plan);
     if (s != OBLIVGM_OK) return s;
     return launch_plan(ctx, plan, st, ctx->d_error);
 }
@@ -1700,7 +1707,7 @@ extern "C" oblivgm_status oblivgm_filter_and_combine_noalloc(oblivgm_ctx* ctx, u
     if (st != OBLIVGM_OK) return fail(st, err);
     uint32_t* const* outs[1] = {out};
     Plan plan;
-    st = plan_filter(ctx, ctx->tables, 1, &query_id, &parsed, &n_groups, outs, /*staged_ok=*/false, &plan);
+    st = plan_filter(ctx, ctx->tables, 1, &query_id, &parsed, &n_groups, outs, kNotStaged, &plan);
     if (st != OBLIVGM_OK) return st;
     if (plan.item_start.back() == 0) return OBLIVGM_OK;
     const WsImage im = build_ws_image(plan);
@@ -1757,7 +1764,7 @@ extern "C" oblivgm_status oblivgm_plan_create(oblivgm_ctx* ctx, uint32_t n_queri
         if (st != OBLIVGM_OK) return fail(st, err);
     }
     Plan plan;
-    st = plan_filter(ctx, ctx->tables, n_queries, query_ids, parsed.data(), n_groups, outs, /*staged_ok=*/true, &plan);
+    st = plan_filter(ctx, ctx->tables, n_queries, query_ids, parsed.data(), n_groups, outs, kStagedPlan, &plan);
     if (st != OBLIVGM_OK) return st;
     auto* p = new (std::nothrow) oblivgm_plan();
     if (!p) return fail(OBLIVGM_ENOMEM, "host allocation");

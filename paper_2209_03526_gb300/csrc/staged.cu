@@ -774,10 +774,10 @@ __global__ void __launch_bounds__(256) k_gather_raw(const __grid_constant__ Gath
 // GB300 figures the plan weighs: a DPF / DCF level step of one key at the T-table lookup rate,
 // a PRF word, a launch (with its table fill) and a key of a sort pass.
 constexpr double kDpfStep = 16.7e-12, kDcfStep = 32.2e-12, kPrfWord = 15.5e-12, kLaunch = 4.0e-6;
-// a level step of a thread on its own, and what a staged evaluation and k_filter take on top (of 564
-// plans of 1,000 to 100,000 elements, one to five predicates and n = 8 to 32, timed both ways,
-// the estimates with these pick the slower one, by 5 % and more, in 35, each by staying fused)
-constexpr double kDpfLatency = 0.57e-6, kDcfLatency = 0.92e-6, kStagedFixed = 8e-6, kFusedFixed = 20e-6;
+// a level step of a thread on its own, and what k_filter takes on top (of 564 plans of 1,000 to
+// 100,000 elements, one to five predicates and n = 8 to 32, timed both ways, the estimates
+// pick the slower one, by 5 % and more, in 25, each by staying fused)
+constexpr double kDpfLatency = 0.57e-6, kDcfLatency = 0.92e-6, kFusedFixed = 20e-6;
 constexpr double kSortKeyPass = 12e-12;
 // what a staged raw evaluation takes beside its launches: scratch, descriptors and their copy
 constexpr double kRawFixed = 3.0e-6;
@@ -925,7 +925,7 @@ void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* grou
 }
 
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
-                 size_t scratch_cap, double wp_seconds, Staged* sg) {
+                 size_t scratch_cap, double fixed, double wp_seconds, Staged* sg) {
     *sg = Staged{};
     sg->n_keys = (uint32_t)n_keys;
     // columns: a share row of the first set
@@ -987,7 +987,7 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
     // against k_filter, whose threads walk an element's keys one after another (at least its chain),
     // or the walk-parallel kernel's schedule
     const double other = wp_seconds > 0 ? wp_seconds : kFusedFixed + std::max(fused + combine, chain);
-    if (kStagedFixed + 1.05 * staged + 1.5 * combine > 0.95 * other) { *sg = Staged{}; return false; }
+    if (fixed + 1.05 * staged + 1.5 * combine > 0.95 * other) { *sg = Staged{}; return false; }
 
     choose_tiles(sg);
     size_t col_end = 0;

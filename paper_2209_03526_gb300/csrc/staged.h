@@ -142,10 +142,10 @@ struct Staged {
 };
 
 // Plans the staged evaluation of a launch; false when it does not pay (or does not apply) and
-// the fused kernels should run.  wp_seconds: the walk-parallel kernel's time where that is the
-// fused kernel of the launch, else 0.
+// the fused kernels should run.  fixed: what it takes beside its kernels; wp_seconds: the
+// walk-parallel kernel's time where that is the fused kernel of the launch, else 0.
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
-                 size_t scratch_cap, double wp_seconds, Staged* out);
+                 size_t scratch_cap, double fixed, double wp_seconds, Staged* out);
 
 // Sets the pointers for scratch at a device address and builds the descriptor image's bytes.
 void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::vector<unsigned char>* bytes);
