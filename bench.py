@@ -48,6 +48,7 @@ import workload as W  # noqa: E402
 
 METRIC = "FSS predicate evals/s (element-predicate evaluations per second, 3 simulated servers)"
 UNIT = "element-predicates/s"
+STAGED_KERNELS = "k_stage, k_stage_last, k_combine (staged evaluation)"
 N_VERTICES = 1 << 20
 PRF = bytes(range(48))
 KEY_SEED = bytes(range(16))
@@ -379,7 +380,7 @@ def run_ours(args):
     lookups_step = node_lookups(preds, wl["tables"][0]["values"], 32)
     peak_lu = sm_count * LDS_LANES_PER_CLK * max_mhz * 1e6 / 1e9
     roofline = lookup_roofline(lookups_step, ms_per_step / 1e3, peak_lu, aes_step)
-    roofline.update({"kernel": "k_stage, k_stage_last, k_combine (staged evaluation)",
+    roofline.update({"kernel": STAGED_KERNELS,
                      "peak_basis": f"{sm_count} SMs x {LDS_LANES_PER_CLK} lookups/clk x "
                                    f"{max_mhz:.0f} MHz (sm_max_mhz of MEASURED_PEAKS.json)",
                      "counted": "each distinct tree node once per key, and the re-share PRF words; "
@@ -798,13 +799,16 @@ def filter_workload_record(P, torch, name: str, graph, queries, sched, steps: in
     step_s = float(np.mean(ms)) / 1e3
     k_check = min(8, len(queries))
     rec = {"metric": METRIC, "value": units / step_s, "unit": UNIT, "ms_per_step": step_s * 1e3,
-           "steps": steps, "warmup": warmup, "gpu_launches": steps,
+           "steps": steps, "warmup": warmup, "gpu_launches": steps * shape["launches"],
            "config": {"workload": name, "queries": len(queries), "element_predicates_per_step": units,
                       "aes_blocks_per_step": aes, "tables": {str(k): v for k, v in table_n.items()},
                       "n_bits": n_bits, "l2": "flushed between timed steps",
-                      "launch": f"one persistent {shape['kernel']} launch ({shape['grid']} CTAs x "
-                                f"{shape['threads']} threads, {shape['items']} tiles of up to {shape['tile']} "
-                                "elements) replayed from a CUDA graph",
+                      "launch": (f"one staged evaluation ({shape['launches']} launches, {shape['rounds']} rounds, "
+                                 f"{shape['scratch']} bytes of scratch) replayed from a CUDA graph"
+                                 if shape["staged"] else
+                                 f"one persistent {shape['kernel']} launch ({shape['grid']} CTAs x "
+                                 f"{shape['threads']} threads, {shape['items']} tiles of up to {shape['tile']} "
+                                 "elements) replayed from a CUDA graph"),
                       "warmup_launches": f"{warmup} of this plan" + (
                           f", after 3 of the first {plain['queries']} queries' plan (same kernel)" if plain else ""),
                       "reconstructs_to_plaintext_sampled": sampled_parity(torch, graph, queries[:k_check],
@@ -812,7 +816,7 @@ def filter_workload_record(P, torch, name: str, graph, queries, sched, steps: in
                       "parity_queries_checked": k_check},
            "roofline": lookup_roofline(lookups, step_s, peak_lu, aes),
            "clocks": clocks}
-    rec["roofline"]["kernel"] = shape["kernel"]
+    rec["roofline"]["kernel"] = STAGED_KERNELS if shape["staged"] else shape["kernel"]
     if plain:
         rec["plain_path"] = plain
     ctx.close()

@@ -272,8 +272,13 @@ oblivgm_status oblivgm_filter_and_combine(oblivgm_ctx* ctx, uint32_t query_id, c
                                           const size_t tok_len[3], uint32_t n_groups, uint32_t* const* out,
                                           void* stream);
 
-/* The same for n_queries queries in ONE persistent launch (work items of all
- * queries' groups and element tiles in a shared queue, ordered by cost).
+/* The same for n_queries queries at once: ONE persistent launch (work
+ * items of all queries' groups and element tiles in a shared queue, ordered by
+ * cost), or, where elements share enough tree nodes, the launches of one
+ * staged evaluation, with its scratch from a pool of the device's contexts:
+ * at most an eighth of the device's memory while it runs, of which 4 GiB are
+ * kept between calls until the device's last context is destroyed.  Where the
+ * scratch cannot be had, the fused launch runs.
  * query_ids[q]; toks[3 q + i], tok_lens[3 q + i]; n_groups[q];
  * outs[q] is the query's array of 3 * n_groups[q] device pointers.
  * Each query's output equals what oblivgm_filter_and_combine gives for it
@@ -285,8 +290,11 @@ oblivgm_status oblivgm_filter_batch(oblivgm_ctx* ctx, uint32_t n_queries, const 
 /* Prepared batches for CUDA-graph capture.  oblivgm_plan_create parses the
  * queries (arguments as oblivgm_filter_batch), fixes the launch shape and
  * uploads descriptors and device keys into a plan-owned device buffer
- * (synchronous; allocates).  oblivgm_plan_launch then only resets the plan's
- * work counter and launches the fused kernel on `stream`: no host-side work,
+ * (synchronous; allocates).  A plan of a staged evaluation also owns its
+ * scratch, up to an eighth of the device's memory, until it is destroyed
+ * (oblivgm_plan_route).  oblivgm_plan_launch then only resets the plan's
+ * work counter and launches the fused kernel, or launches the staged
+ * kernels, on `stream`: no host-side work,
  * no allocation and no pageable copies, so it may be captured into a CUDA
  * graph and replayed; every launch recomputes the same shares into the
  * outputs given at creation (which must stay valid).  Launches of one plan
@@ -299,7 +307,8 @@ oblivgm_status oblivgm_plan_create(oblivgm_ctx* ctx, uint32_t n_queries, const u
 oblivgm_status oblivgm_plan_launch(oblivgm_plan* plan, void* stream);
 oblivgm_status oblivgm_plan_destroy(oblivgm_plan* plan);
 
-/* The launch a plan fixed: walk_parallel = 1 for the walk-parallel kernel
+/* The fused launch that a plan fixed, which a staged plan's scratch saves it
+ * (oblivgm_plan_route): walk_parallel = 1 for the walk-parallel kernel
  * (one thread per key walk), 0 for the per-element kernel; threads per CTA;
  * elements per work item (tile: for the walk-parallel kernel, which may give
  * each of a few groups its own width, the widest); work items; CTAs launched
@@ -307,6 +316,15 @@ oblivgm_status oblivgm_plan_destroy(oblivgm_plan* plan);
  * NULL plan. */
 oblivgm_status oblivgm_plan_describe(const oblivgm_plan* plan, uint32_t* walk_parallel, uint32_t* threads,
                                      uint32_t* tile, uint64_t* n_items, uint32_t* grid);
+
+/* What oblivgm_plan_launch runs: staged = 1 for the staged evaluation, 0 for
+ * the fused launch of oblivgm_plan_describe; kernel launches of one
+ * oblivgm_plan_launch; and of a staged plan (0 otherwise) the rounds that its
+ * predicates are cut into, the chunks of distinct values in the round with the
+ * most, and the bytes of scratch it owns.  Any output pointer may be NULL.
+ * Errors: EINVAL for a NULL plan. */
+oblivgm_status oblivgm_plan_route(const oblivgm_plan* plan, uint32_t* staged, uint64_t* launches, uint32_t* rounds,
+                                  uint32_t* chunks, uint64_t* scratch_bytes);
 
 /* The plain per-query GPU path: the same computation and results as
  * oblivgm_filter_and_combine (Alg. 3 + Eq. predEval + re-share + AND), but

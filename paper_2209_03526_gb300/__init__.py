@@ -336,13 +336,20 @@ class Context:
         N.check(self._lib.oblivgm_plan_launch(plan, _stream_handle(stream)), "oblivgm_plan_launch")
 
     def plan_describe(self, plan) -> dict:
-        """The launch a plan fixed (oblivgm_plan_describe)."""
+        """The fused launch a plan fixed (oblivgm_plan_describe), and what a plan launch runs: "staged",
+        its kernel "launches", and a staged plan's "rounds", "chunks" and "scratch" bytes
+        (oblivgm_plan_route)."""
         wp, th, tile, grid = (ctypes.c_uint32() for _ in range(4))
         items = ctypes.c_uint64()
         N.check(self._lib.oblivgm_plan_describe(plan, ctypes.byref(wp), ctypes.byref(th), ctypes.byref(tile),
                                                 ctypes.byref(items), ctypes.byref(grid)), "oblivgm_plan_describe")
+        staged, rounds, chunks = (ctypes.c_uint32() for _ in range(3))
+        launches, scratch = ctypes.c_uint64(), ctypes.c_uint64()
+        N.check(self._lib.oblivgm_plan_route(plan, ctypes.byref(staged), ctypes.byref(launches), ctypes.byref(rounds),
+                                             ctypes.byref(chunks), ctypes.byref(scratch)), "oblivgm_plan_route")
         return {"kernel": "k_filter_wp" if wp.value else "k_filter", "threads": th.value, "tile": tile.value,
-                "items": items.value, "grid": grid.value}
+                "items": items.value, "grid": grid.value, "staged": bool(staged.value), "launches": launches.value,
+                "rounds": rounds.value, "chunks": chunks.value, "scratch": scratch.value}
 
     def plan_destroy(self, plan):
         N.check(self._lib.oblivgm_plan_destroy(plan), "oblivgm_plan_destroy")

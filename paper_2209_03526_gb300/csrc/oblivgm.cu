@@ -1826,6 +1826,19 @@ extern "C" oblivgm_status oblivgm_plan_describe(const oblivgm_plan* p, uint32_t*
     return OBLIVGM_OK;
 }
 
+extern "C" oblivgm_status oblivgm_plan_route(const oblivgm_plan* p, uint32_t* staged, uint64_t* launches,
+                                             uint32_t* rounds, uint32_t* chunks, uint64_t* scratch_bytes) {
+    if (!p) return fail(OBLIVGM_EINVAL, "NULL plan");
+    uint32_t most = 0;
+    for (const StagedRound& R : p->sg.rounds) most = std::max(most, R.chunks);
+    if (staged) *staged = p->staged ? 1u : 0u;
+    if (launches) *launches = p->staged ? staged_launches(p->sg) : p->n_items ? 1 : 0;
+    if (rounds) *rounds = (uint32_t)p->sg.rounds.size();
+    if (chunks) *chunks = most;
+    if (scratch_bytes) *scratch_bytes = p->staged ? p->sg.scratch_bytes : 0;
+    return OBLIVGM_OK;
+}
+
 extern "C" oblivgm_status oblivgm_plan_destroy(oblivgm_plan* p) {
     if (!p) return OBLIVGM_OK;
     cudaSetDevice(p->ctx->device);

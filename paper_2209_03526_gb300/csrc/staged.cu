@@ -1123,11 +1123,17 @@ void launch_sort_tiles(const Staged& sg, const SgCol* cols, cudaStream_t s) {
     launch_after(k_uniq_emit<ITEMS>, grid, kSortThreads, 0, s, cols);
 }
 
+uint64_t sort_launches(const Staged& sg) { return sg.sort_passes ? 3ull * sg.sort_passes + 3 : 0; }
+
+uint64_t round_launches(const StagedRound& R) {
+    return R.chunks * (R.max_stages + (R.sparse && R.max_stages > 1 ? 3ull : 0ull));
+}
+
 uint64_t launch_sort(const Staged& sg, const SgCol* cols, cudaStream_t s) {
     if (!sg.sort_passes) return 0;
     if (sg.sort_large) launch_sort_tiles<kSortItemsLarge>(sg, cols, s);
     else launch_sort_tiles<kSortItemsSmall>(sg, cols, s);
-    return 3 * sg.sort_passes + 3;
+    return sort_launches(sg);
 }
 
 // the sums of a round's predicates at every distinct value
@@ -1153,10 +1159,16 @@ uint64_t launch_round(const oblivgm_ctx* ctx, const StagedRound& R, const SgPred
         }
         launch_after(k_stage_last, sms, kStageThreads, kTableBytes, s, W);
     }
-    return R.chunks * (R.max_stages + (R.sparse && R.max_stages > 1 ? 3ull : 0ull));
+    return round_launches(R);
 }
 
 }  // namespace
+
+uint64_t staged_launches(const Staged& sg) {
+    uint64_t launches = sort_launches(sg);
+    for (const StagedRound& R : sg.rounds) launches += round_launches(R) + 1;
+    return launches;
+}
 
 oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s) {
     uint64_t launches = launch_sort(sg, reinterpret_cast<const SgCol*>(image), s);

@@ -153,6 +153,7 @@ void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::v
 // Launches it on an image in device memory: no host work beyond the launches, no allocation,
 // capturable.
 oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, cudaStream_t s);
+uint64_t staged_launches(const Staged& sg);     // kernels of one launch
 
 // Raw evaluation of n_keys keys of one kind at the same n_points points (OBLIVGM_ALL_PAIRS):
 // plan (false: does not pay) and launch; out[k * n_points + i] = Eval(key k, points[i]).

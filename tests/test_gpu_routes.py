@@ -108,3 +108,21 @@ def test_equality_groups_of_one_wave(ctx, sizes):
     assert launches == 1 and shape["kernel"] == "k_filter_wp" and shape["items"] == shape["grid"]
     for grp, got in enumerate(_shares(outs)):
         assert np.array_equal(got, oracle_group(oracle, wl, toks, 9, grp, np.arange(sizes[grp]))), grp
+
+
+def test_a_staged_plan_says_so(ctx):
+    """What plan_describe reports of a staged plan and of a fused one is what a launch does."""
+    for n, staged in ((60000, True), (1000, False)):
+        wl = _workload(n)
+        load_tables(ctx, wl)
+        toks = P.keygen(wl["preds"], 32, bytes(16))
+        plan = ctx.plan_create([3], [toks], [alloc_outs(wl)])
+        d = ctx.plan_describe(plan)
+        before = ctx.launch_count()
+        ctx.plan_launch(plan)
+        ctx.sync()
+        assert ctx.launch_count() - before == d["launches"]
+        ctx.plan_destroy(plan)
+        assert d["staged"] == staged and (d["launches"] > 10) == staged and (d["rounds"] == 1) == staged
+        # at least the columns' sorted keys, element numbers and ranks, twice and once, for two columns
+        assert d["scratch"] >= 2 * 20 * n if staged else d["scratch"] == 0
