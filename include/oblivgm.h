@@ -660,6 +660,16 @@ oblivgm_status oblivgm_test_expire_next_wait(oblivgm_ctx* ctx, uint32_t limit_us
  * counterpart. */
 oblivgm_status oblivgm_test_fail_next_alloc(oblivgm_ctx* ctx);
 
+/* Test hook for the staged evaluation's limits: its scratch requests above
+ * scratch_bytes find no memory (0: all of them; UINT64_MAX: none but the
+ * device's own refusals), so that the calls and plans that make them take the
+ * kernels that need none; the predicates evaluated together take round_bytes
+ * of scratch and the distinct values chunk_values (a power of two of 1,024 or
+ * more; 0 is the default for both).  Outputs do not change.  Errors: EINVAL
+ * (NULL context, chunk_values). */
+oblivgm_status oblivgm_test_staged_limits(oblivgm_ctx* ctx, uint64_t scratch_bytes, uint64_t round_bytes,
+                                          uint32_t chunk_values);
+
 /* Count of this library's kernel launches so far on the context (for the
  * bench's launch accounting). */
 uint64_t oblivgm_launch_count(oblivgm_ctx* ctx);

@@ -436,6 +436,11 @@ class Context:
         """Failure-path test hook: the next device workspace allocation reports ENOMEM."""
         N.check(self._lib.oblivgm_test_fail_next_alloc(self._h), "oblivgm_test_fail_next_alloc")
 
+    def test_staged_limits(self, scratch_bytes: int = (1 << 64) - 1, round_bytes: int = 0, chunk_values: int = 0):
+        """Test hook: the staged evaluation's scratch, rounds and chunks; without arguments the defaults."""
+        N.check(self._lib.oblivgm_test_staged_limits(self._h, scratch_bytes, round_bytes, chunk_values),
+                "oblivgm_test_staged_limits")
+
     def test_expire_next_wait(self, limit_us: int):
         """Failure-path test hook: the next fused launch's key-staging waits run out after limit_us."""
         N.check(self._lib.oblivgm_test_expire_next_wait(self._h, limit_us), "oblivgm_test_expire_next_wait")

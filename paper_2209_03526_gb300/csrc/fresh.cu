@@ -556,7 +556,7 @@ extern "C" oblivgm_status oblivgm_keygen_fresh(oblivgm_ctx* ctx, const oblivgm_p
     return OBLIVGM_OK;
 }
 
-// Walks and combine over a scratch block of the predicates' sums, in rounds that fit kRoundBytes.
+// Walks and combine over a scratch block of the predicates' sums, in rounds that fit limits.round_bytes.
 // *ran stays false where the scratch cannot be had.
 static oblivgm_status filter_fresh_walks(oblivgm_ctx* ctx, const FreshEvalParams& E, uint64_t total, cudaStream_t s,
                                          bool* ran) {
@@ -575,7 +575,7 @@ static oblivgm_status filter_fresh_walks(oblivgm_ctx* ctx, const FreshEvalParams
         if (N >> 32) return OBLIVGM_OK;
         bool open = false;
         for (uint32_t k = 0; k < G.n_preds; k++) {
-            if (rounds.empty() || (at && at + up(16 * N) > kRoundBytes)) {
+            if (rounds.empty() || (at && at + up(16 * N) > ctx->limits.round_bytes)) {
                 rounds.push_back(Round{(uint32_t)folds.size(), 0, (uint32_t)groups.size(), 0, 0});
                 at = 0;
                 open = false;
@@ -609,12 +609,9 @@ static oblivgm_status filter_fresh_walks(oblivgm_ctx* ctx, const FreshEvalParams
     for (Round& r : rounds) r.items = combine_tiles(shape, groups.data() + r.group_begin, r.n_groups);
     const uint64_t off_folds = up(groups.size() * sizeof(SgGroup)), off_z = off_folds + up(folds.size() * sizeof(SgFold));
     unsigned char* scratch = nullptr;
-    const cudaError_t ae =
-        cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), off_z + most, ctx->scratch_pool, s);
-    if (ae == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return OBLIVGM_OK;
-    }
+    if (off_z + most > ctx->limits.cap) return OBLIVGM_OK;
+    const cudaError_t ae = scratch_alloc(ctx, &scratch, off_z + most, s);
+    if (ae == cudaErrorMemoryAllocation) return OBLIVGM_OK;
     if (ae != cudaSuccess) return cuda_fail(ae, "fresh scratch allocation");
     ScratchGuard guard(scratch, s);
     for (size_t p = 0; p < folds.size(); p++) folds[p].z = reinterpret_cast<const uint32_t*>(scratch + off_z + z_at[p]);

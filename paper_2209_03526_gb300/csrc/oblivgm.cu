@@ -49,6 +49,14 @@ oblivgm_status ws_alloc(oblivgm_ctx* ctx, void** p, size_t bytes, cudaStream_t s
     return e == cudaSuccess ? OBLIVGM_OK : cuda_fail(e, what);
 }
 
+cudaError_t scratch_alloc(oblivgm_ctx* ctx, unsigned char** p, size_t bytes, cudaStream_t s) {
+    *p = nullptr;
+    if (bytes > ctx->limits.have) return cudaErrorMemoryAllocation;
+    const cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, ctx->scratch_pool, s);
+    if (e == cudaErrorMemoryAllocation) cudaGetLastError();
+    return e;
+}
+
 #define OGM_CUDA(call, what)                      \
     do {                                          \
         cudaError_t _e = (call);                  \
@@ -1049,7 +1057,7 @@ oblivgm_status plan_filter(oblivgm_ctx* ctx, const std::map<uint32_t, Table>& ta
     // n = 16: 337 us walk-parallel, 160 staged), but for one wave of walk-parallel tiles, which the
     // staged launches alone outlast; the key-staging expiry hook is about the fused kernels' waits
     if (use.ok && !ctx->test_expire_next && (!plan->wp || plan->wp_seconds > use.least))
-        plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->scratch_cap,
+        plan->staged = staged_plan(plan->groups, plan->preds, plan->keys.size(), ctx->sm_count, ctx->limits,
                                    use.fixed, plan->wp ? plan->wp_seconds : 0.0, &plan->sg);
     return OBLIVGM_OK;
 }
@@ -1151,12 +1159,8 @@ oblivgm_status launch_staged(oblivgm_ctx* ctx, Plan& plan, cudaStream_t st, bool
         ws_alloc(ctx, reinterpret_cast<void**>(&image), plan.sg.image_bytes, st, "workspace allocation");
     if (as != OBLIVGM_OK) return as;
     ScratchGuard guard(image, st);
-    const cudaError_t ae =
-        cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), plan.sg.scratch_bytes, ctx->scratch_pool, st);
-    if (ae == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        return OBLIVGM_OK;
-    }
+    const cudaError_t ae = scratch_alloc(ctx, &scratch, plan.sg.scratch_bytes, st);
+    if (ae == cudaErrorMemoryAllocation) return OBLIVGM_OK;
     if (ae != cudaSuccess) return cuda_fail(ae, "scratch allocation");
     ScratchGuard scratch_guard(scratch, st);
     std::vector<unsigned char> bytes;
@@ -1247,7 +1251,7 @@ oblivgm_status oblivgm_create(oblivgm_ctx** out, int32_t device, const oblivgm_c
     if (!ctx) return fail(OBLIVGM_ENOMEM, "host allocation");
     ctx->device = device;
     ctx->sm_count = prop.multiProcessorCount;
-    ctx->scratch_cap = prop.totalGlobalMem / 8;
+    ctx->limits.cap = prop.totalGlobalMem / 8;
     ctx->wp_max_elems = (uint64_t)ctx->sm_count * kWpDefaultElemsPerSm;
     build_aes_params(&ctx->aes);
     for (int i = 0; i < 3; i++) {
@@ -1322,6 +1326,19 @@ oblivgm_status oblivgm_sync(oblivgm_ctx* ctx, void* stream) {
         return fail(OBLIVGM_EFAULT_DEVICE, (flag & 1u) ? "a bounded device wait expired (key staging)"
                                                        : "a device-resident key had a malformed header");
     }
+    return OBLIVGM_OK;
+}
+
+oblivgm_status oblivgm_test_staged_limits(oblivgm_ctx* ctx, uint64_t scratch_bytes, uint64_t round_bytes,
+                                          uint32_t chunk_values) {
+    oblivgm_status st = check_ctx(ctx);
+    if (st) return st;
+    if (chunk_values && (chunk_values < 1024 || (chunk_values & (chunk_values - 1))))
+        return fail(OBLIVGM_EINVAL, "a chunk is a power of two of 1,024 or more values");
+    const StagedLimits d;
+    ctx->limits.have = scratch_bytes;
+    ctx->limits.round_bytes = round_bytes ? round_bytes : d.round_bytes;
+    ctx->limits.chunk = chunk_values ? chunk_values : d.chunk;
     return OBLIVGM_OK;
 }
 
@@ -1433,11 +1450,10 @@ static oblivgm_status eval_batch(oblivgm_ctx* ctx, uint32_t kind, const uint8_t*
     // all keys at all points: the walks share tree nodes (staged.cu) where that pays and there
     // is room for it
     Staged sg;
-    if (all && staged_plan_raw(kind, (uint32_t)n, n_keys, points, n_points, ctx->scratch_cap, &sg) && !under_capture(s)) {
+    if (all && staged_plan_raw(kind, (uint32_t)n, n_keys, points, n_points, ctx->limits, &sg) && !under_capture(s)) {
         unsigned char* scratch = nullptr;
         const size_t img = (sg.image_bytes + 255) / 256 * 256;
-        const cudaError_t ae =
-            cudaMallocFromPoolAsync(reinterpret_cast<void**>(&scratch), img + sg.scratch_bytes, ctx->scratch_pool, s);
+        const cudaError_t ae = scratch_alloc(ctx, &scratch, img + sg.scratch_bytes, s);
         if (ae == cudaSuccess) {
             ScratchGuard scratch_guard(scratch, s);
             std::vector<unsigned char> bytes;
@@ -1452,7 +1468,6 @@ static oblivgm_status eval_batch(oblivgm_ctx* ctx, uint32_t kind, const uint8_t*
             return OBLIVGM_OK;
         }
         if (ae != cudaErrorMemoryAllocation) return cuda_fail(ae, "scratch allocation");
-        cudaGetLastError();
     }
     RawParams P{};
     P.aes = ctx->aes;
@@ -1768,7 +1783,8 @@ extern "C" oblivgm_status oblivgm_plan_create(oblivgm_ctx* ctx, uint32_t n_queri
     if (st != OBLIVGM_OK) return st;
     auto* p = new (std::nothrow) oblivgm_plan();
     if (!p) return fail(OBLIVGM_ENOMEM, "host allocation");
-    if (plan.staged && cudaMalloc(&p->scratch, plan.sg.scratch_bytes) != cudaSuccess) {
+    if (plan.staged && (plan.sg.scratch_bytes > ctx->limits.have ||
+                        cudaMalloc(&p->scratch, plan.sg.scratch_bytes) != cudaSuccess)) {
         cudaGetLastError();            // no room for the scratch: the fused kernel's plan instead
         plan.staged = false;
     }

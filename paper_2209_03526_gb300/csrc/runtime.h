@@ -45,7 +45,14 @@ struct ScratchGuard {
     ScratchGuard& operator=(const ScratchGuard&) = delete;
 };
 
-constexpr uint64_t kScratchKeep = 4ull << 30;
+// Limits of the staged evaluation and its scratch.
+constexpr uint64_t kScratchKeep = 4ull << 30;     // bytes that the pool keeps between calls
+struct StagedLimits {
+    uint64_t cap = 0;                      // most scratch that a plan may ask for (an eighth of the device)
+    uint64_t round_bytes = 5ull << 29;     // scratch of the predicates evaluated together (2.5 GiB)
+    uint32_t chunk = 1u << 22;             // distinct values evaluated together, a power of two
+    uint64_t have = UINT64_MAX;            // larger requests find no memory (test hook)
+};
 
 struct Table {
     uint32_t* dev = nullptr;   // [share set j][attr][stride] uint32
@@ -121,7 +128,7 @@ struct oblivgm_ctx {
     uint32_t elems_per_thread = 1;
     uint64_t wp_max_elems = 0;       // batches with at most this many elements in all run walk-parallel
     bool wp_fixed = false;           // that number was set by the caller: no staged evaluation up to it (0: none at all)
-    size_t scratch_cap = 0;          // most scratch a staged evaluation may take
+    ogm::StagedLimits limits;
     cudaMemPool_t scratch_pool = nullptr;   // its stream-ordered scratch; keeps kScratchKeep bytes between calls
     uint32_t wp_tile = 0;            // walk-parallel elements per tile; 0 = chosen per launch
     std::atomic<uint64_t> launches{0};
@@ -183,6 +190,9 @@ oblivgm_status set_onehot_attrs();
 oblivgm_status set_keygen_attrs();
 // stream-ordered device workspace; ENOMEM when the allocator refuses (or the test hook says so)
 oblivgm_status ws_alloc(oblivgm_ctx* ctx, void** p, size_t bytes, cudaStream_t s, const char* what);
+// stream-ordered scratch of the staged evaluation and the fresh-key walks; cudaErrorMemoryAllocation, with
+// the error cleared, where there is no room: their callers then run a kernel that needs none
+cudaError_t scratch_alloc(oblivgm_ctx* ctx, unsigned char** p, size_t bytes, cudaStream_t s);
 oblivgm_status set_fresh_attrs();
 oblivgm_status set_shuffle_attrs();
 oblivgm_status set_prg_attrs();

@@ -782,7 +782,6 @@ constexpr double kSortKeyPass = 12e-12;
 // what a staged raw evaluation takes beside its launches: scratch, descriptors and their copy
 constexpr double kRawFixed = 3.0e-6;
 constexpr uint64_t kMaxElems = 1ull << 28;
-constexpr uint32_t kMaxChunk = 1u << 22;      // distinct values evaluated together
 constexpr int kMaxDenseBits = 24;
 // A launch whose last stages have fewer units (32 values of one slot) than this, one and a half
 // for each of the chip's 152 x 24 warps, runs a unit per key there: a range of 5,000 values, n = 32,
@@ -925,7 +924,7 @@ void launch_combine(oblivgm_ctx* ctx, const CombineShape& c, const SgGroup* grou
 }
 
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
-                 size_t scratch_cap, double fixed, double wp_seconds, Staged* sg) {
+                 const StagedLimits& limits, double fixed, double wp_seconds, Staged* sg) {
     *sg = Staged{};
     sg->n_keys = (uint32_t)n_keys;
     // columns: a share row of the first set
@@ -996,7 +995,7 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
     for (size_t q = 0; q < preds.size(); q++)
         last_units += 3 * ((max_values(sg->cols[pred_col[q]]) + 31) / 32);
     sg->split = last_units < kSplitUnits;
-    // predicates in group order, cut into rounds whose states fit kRoundBytes
+    // predicates in group order, cut into rounds whose states fit limits.round_bytes
     size_t at = col_end, most = col_end;
     StagedRound R{};
     const auto close = [&]() {
@@ -1027,10 +1026,10 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
             std::copy(lev[p.col].begin(), lev[p.col].end(), p.lev);
             const uint64_t vals = max_values(C);
             p.chunk = kRunBlock;
-            while (p.chunk < vals && p.chunk < kMaxChunk) p.chunk <<= 1;
+            while (p.chunk < vals && p.chunk < limits.chunk) p.chunk <<= 1;
             p.blocks = p.chunk / kRunBlock;
             for (uint32_t s = 0; s + 1 < p.stages; s++) p.cap[s & 1] = std::max(p.cap[s & 1], (uint32_t)max_runs(p, C, s));
-            if (R.n_preds && (R.n_preds >= kMaxRoundPreds || layout_pred(&p, C, nullptr, at) - col_end > kRoundBytes)) {
+            if (R.n_preds && (R.n_preds >= kMaxRoundPreds || layout_pred(&p, C, nullptr, at) - col_end > limits.round_bytes)) {
                 close();
                 open = false;
             }
@@ -1075,7 +1074,7 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
     sg->shape = combine_shape(elems, most_preds, sm_count);
     for (StagedRound& r : sg->rounds) r.items = combine_tiles(sg->shape, sg->groups.data() + r.group_begin, r.n_groups);
     sg->scratch_bytes = most;
-    if (sg->scratch_bytes > scratch_cap) { *sg = Staged{}; return false; }
+    if (sg->scratch_bytes > limits.cap) { *sg = Staged{}; return false; }
     sg->off_preds = up256(sg->cols.size() * sizeof(SgCol));
     sg->off_folds = sg->off_preds + up256(sg->preds.size() * sizeof(SgPred));
     sg->off_groups = sg->off_folds + up256(sg->folds.size() * sizeof(SgFold));
@@ -1185,7 +1184,7 @@ oblivgm_status staged_launch(oblivgm_ctx* ctx, const Staged& sg, const unsigned 
 }
 
 bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint32_t* points, uint64_t n_points,
-                     size_t scratch_cap, Staged* sg) {
+                     const StagedLimits& limits, Staged* sg) {
     *sg = Staged{};
     if (n_points > kMaxElems) return false;
     SgCol C{};
@@ -1233,13 +1232,13 @@ bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint
     p.z_slot = vals;
     p.parts = 1;
     p.chunk = kRunBlock;
-    while (p.chunk < vals && p.chunk < kMaxChunk) p.chunk <<= 1;
+    while (p.chunk < vals && p.chunk < limits.chunk) p.chunk <<= 1;
     p.blocks = p.chunk / kRunBlock;
     for (uint32_t s = 0; s + 1 < p.stages; s++) p.cap[s & 1] = std::max(p.cap[s & 1], (uint32_t)max_runs(p, C, s));
     p.n_keys = std::min<uint32_t>(n_keys, 64);
-    while (p.n_keys > 1 && layout_pred(&p, C, nullptr, col_end) - col_end > kRoundBytes) p.n_keys = (p.n_keys + 1) / 2;
+    while (p.n_keys > 1 && layout_pred(&p, C, nullptr, col_end) - col_end > limits.round_bytes) p.n_keys = (p.n_keys + 1) / 2;
     sg->scratch_bytes = layout_pred(&p, C, nullptr, col_end);
-    if (sg->scratch_bytes > scratch_cap) { *sg = Staged{}; return false; }
+    if (sg->scratch_bytes > limits.cap) { *sg = Staged{}; return false; }
     const uint32_t per = p.n_keys;
     for (uint32_t k = 0; k < n_keys; k += per) {
         p.key_begin = k;

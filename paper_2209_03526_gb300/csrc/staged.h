@@ -13,6 +13,8 @@ struct oblivgm_ctx;
 
 namespace ogm {
 
+struct StagedLimits;
+
 // One AND-group of a launch.
 struct GroupDesc {
     const uint32_t* share[3];   // share set j of the group's table: [attr][stride]
@@ -37,7 +39,6 @@ struct PredDesc {
 };
 
 constexpr int kSgMaxStages = 33;
-constexpr size_t kRoundBytes = 5ull << 29;    // scratch of the predicates evaluated together (2.5 GiB)
 
 // One opened column of the launch (an attribute of a table, all its elements).
 struct SgCol {
@@ -145,7 +146,7 @@ struct Staged {
 // the fused kernels should run.  fixed: what it takes beside its kernels; wp_seconds: the
 // walk-parallel kernel's time where that is the fused kernel of the launch, else 0.
 bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDesc>& preds, size_t n_keys, int sm_count,
-                 size_t scratch_cap, double fixed, double wp_seconds, Staged* out);
+                 const StagedLimits& limits, double fixed, double wp_seconds, Staged* out);
 
 // Sets the pointers for scratch at a device address and builds the descriptor image's bytes.
 void staged_image(Staged* sg, const DevKey* keys, unsigned char* scratch, std::vector<unsigned char>* bytes);
@@ -158,7 +159,7 @@ uint64_t staged_launches(const Staged& sg);     // kernels of one launch
 // Raw evaluation of n_keys keys of one kind at the same n_points points (OBLIVGM_ALL_PAIRS):
 // plan (false: does not pay) and launch; out[k * n_points + i] = Eval(key k, points[i]).
 bool staged_plan_raw(uint32_t kind, uint32_t n_bits, uint32_t n_keys, const uint32_t* points, uint64_t n_points,
-                     size_t scratch_cap, Staged* out);
+                     const StagedLimits& limits, Staged* out);
 oblivgm_status staged_launch_raw(oblivgm_ctx* ctx, const Staged& sg, const unsigned char* image, const DevKey* keys,
                                  uint32_t* out, cudaStream_t s);
 
