@@ -599,7 +599,14 @@ oblivgm_status oblivgm_poll(oblivgm_ctx* ctx, uint64_t ticket, int32_t timeout_m
  * (NULL context, max_ms 0). */
 oblivgm_status oblivgm_set_poll_limit(oblivgm_ctx* ctx, uint32_t max_ms, uint32_t* previous);
 
-/* Return a served result's memory to the arena (re-admits waiting work). */
+/* Return a served result's memory to the arena (re-admits waiting work).
+ * Reads of the result that were queued before on the default stream, or on a
+ * stream that synchronises with it, are waited for on the device, together
+ * with whatever else those streams hold at that point; reads on any other
+ * stream have to be complete, or ordered before the default stream, first.
+ * While a stream capture forbids the default stream, or if the wait cannot be
+ * queued, the memory stays reserved until a later release, or a submit that
+ * needs it, frees it. */
 oblivgm_status oblivgm_release(oblivgm_ctx* ctx, uint64_t ticket);
 
 /* Serving statistics: queries admitted, completed, rejected (EAGAIN), and the

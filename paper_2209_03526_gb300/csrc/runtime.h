@@ -89,6 +89,14 @@ struct ServeQuery {
     std::string error;
 };
 
+// A released result whose memory could not be freed yet in order after the caller's reads; its
+// bytes stay reserved.
+struct ServeDeferred {
+    std::vector<uint32_t*> outs;
+    int stream = 0;
+    size_t bytes = 0;
+};
+
 struct ServeBatch;
 
 struct ServeState {
@@ -97,6 +105,7 @@ struct ServeState {
     std::deque<uint64_t> queued;
     std::map<uint64_t, std::unique_ptr<ServeQuery>> queries;
     std::map<uint32_t, int> table_refs;
+    std::vector<ServeDeferred> deferred;
     uint64_t next_ticket = 1;
     uint64_t arena = 0, reserved = 0;
     uint32_t max_inflight = 64, inflight = 0;

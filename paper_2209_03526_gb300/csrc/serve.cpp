@@ -123,6 +123,57 @@ void worker_main(oblivgm_ctx* ctx) {
     }
 }
 
+// Makes the serve stream wait for the work that the caller has queued on the default stream, such
+// as a copy of the result: the next batch there could otherwise reuse the memory first.  A capture
+// under way that forbids the default stream is left alone; false then, or when a step fails.
+bool order_after_default_stream(cudaStream_t serve) {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaEvent_t read = nullptr;
+    bool ordered = false;
+    if (cudaStreamIsCapturing(cudaStreamLegacy, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone &&
+        cudaEventCreateWithFlags(&read, cudaEventDisableTiming) == cudaSuccess) {
+        ordered = cudaEventRecord(read, cudaStreamLegacy) == cudaSuccess &&
+                  cudaStreamWaitEvent(serve, read, 0) == cudaSuccess;
+        cudaEventDestroy(read);
+    }
+    cudaGetLastError();
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return ordered;
+}
+
+// Frees released results' memory (`add`, and what waits from before) in order after the caller's
+// reads; what cannot be ordered waits, still reserved, for the next release or the next submit
+// that needs it.
+void free_released(oblivgm_ctx* ctx, ServeDeferred* add) {
+    ServeState& S = ctx->serve;
+    std::vector<ServeDeferred> todo;
+    {
+        std::lock_guard<std::mutex> lk(S.mu);
+        todo.swap(S.deferred);
+    }
+    if (add) todo.push_back(std::move(*add));
+    cudaSetDevice(ctx->device);
+    bool ordered[ServeState::kStreams];
+    for (int i = 0; i < ServeState::kStreams; i++) {
+        bool used = false;
+        for (const ServeDeferred& d : todo) used |= d.stream == i && !d.outs.empty();
+        ordered[i] = !used || order_after_default_stream(S.streams[i]);
+    }
+    for (const ServeDeferred& d : todo)
+        if (ordered[d.stream])
+            for (uint32_t* p : d.outs) cudaFreeAsync(p, S.streams[d.stream]);
+    std::lock_guard<std::mutex> lk(S.mu);
+    for (ServeDeferred& d : todo) {
+        if (ordered[d.stream]) S.reserved -= d.bytes;
+        else S.deferred.push_back(std::move(d));
+    }
+}
+
 }  // namespace
 
 oblivgm_status serve_init(oblivgm_ctx* ctx) {
@@ -155,6 +206,9 @@ void serve_shutdown(oblivgm_ctx* ctx) {
     for (auto& kv : S.queries)
         for (uint32_t* p : kv.second->outs)
             if (p) cudaFree(p);
+    for (const ServeDeferred& d : S.deferred)
+        for (uint32_t* p : d.outs) cudaFree(p);
+    S.deferred.clear();
     S.queries.clear();
     for (int i = 0; i < ServeState::kStreams; i++)
         if (S.streams[i]) cudaStreamDestroy(S.streams[i]);
@@ -205,6 +259,12 @@ oblivgm_status oblivgm_submit(oblivgm_ctx* ctx, const uint8_t* const tok[3], con
     q->bytes = 0;
     for (uint32_t g = 0; g < ng; g++) q->bytes += 3 * std::max<uint64_t>(q->n_elems[g], 4) * sizeof(uint32_t);
     ServeState& S = ctx->serve;
+    {
+        std::unique_lock<std::mutex> lk(S.mu);
+        const bool retry = !S.deferred.empty() && S.reserved + q->bytes > S.arena;
+        lk.unlock();
+        if (retry) free_released(ctx, nullptr);
+    }
     std::lock_guard<std::mutex> lk(S.mu);
     if (S.inflight >= S.max_inflight || S.reserved + q->bytes > S.arena) {
         S.rejected++;
@@ -266,27 +326,14 @@ oblivgm_status oblivgm_release(oblivgm_ctx* ctx, uint64_t ticket) {
         q = std::move(it->second);
         S.queries.erase(it);
         S.inflight--;
-        S.reserved -= q->bytes;
         for (auto& kv : q->tables) S.table_refs[kv.first]--;
     }
-    cudaSetDevice(ctx->device);
-    // Work that the caller queued on the default stream before this call (a copy of the result) may
-    // not have run yet, while the next batch on the serve stream could already reuse the memory:
-    // the release waits for it on the device.
-    // A capture under way, which forbids the default stream, is left alone.
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    cudaEvent_t read = nullptr;
-    if (cudaStreamIsCapturing(cudaStreamLegacy, &capture) == cudaSuccess &&
-        cudaEventCreateWithFlags(&read, cudaEventDisableTiming) == cudaSuccess) {
-        if (cudaEventRecord(read, cudaStreamLegacy) == cudaSuccess) cudaStreamWaitEvent(S.streams[q->stream], read, 0);
-        cudaEventDestroy(read);
-    }
-    cudaGetLastError();
-    cudaThreadExchangeStreamCaptureMode(&mode);
+    ServeDeferred d;
     for (uint32_t* p : q->outs)
-        if (p) cudaFreeAsync(p, S.streams[q->stream]);
+        if (p) d.outs.push_back(p);
+    d.stream = q->stream;
+    d.bytes = q->bytes;
+    free_released(ctx, &d);
     S.cv_work.notify_all();
     return OBLIVGM_OK;
 }
