@@ -959,7 +959,8 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         }
         chain = std::max(chain, group_chain);
     }
-    if (sg->cols.empty()) return false;
+    // a column is a row of the sort kernels' grids
+    if (sg->cols.empty() || sg->cols.size() > 65535) { *sg = Staged{}; return false; }
     // per column: dense when the whole domain costs no more than its sorted values
     std::vector<std::vector<uint8_t>> lev(sg->cols.size());
     double staged = 0;
@@ -983,6 +984,10 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
         sg->sort_passes = std::max(sg->sort_passes, C.passes);
     }
     staged += kLaunch * (double)(most_stages + 1 + (sg->sort_passes ? 6 + 3 * sg->sort_passes : 0));
+    // further rounds (of predicates; of bytes only where the walks take far longer) launch anew, each
+    // launch while the one before runs
+    const double more_rounds = (double)((preds.size() - 1) / kMaxRoundPreds);
+    staged += 0.5 * kLaunch * more_rounds * (double)(most_stages + 1 + (sg->sort_passes ? 3 : 0));
     // against k_filter, whose threads walk an element's keys one after another (at least its chain),
     // or the walk-parallel kernel's schedule
     const double other = wp_seconds > 0 ? wp_seconds : kFusedFixed + std::max(fused + combine, chain);
