@@ -783,10 +783,10 @@ constexpr double kSortKeyPass = 12e-12;
 constexpr double kRawFixed = 3.0e-6;
 constexpr uint64_t kMaxElems = 1ull << 28;
 constexpr int kMaxDenseBits = 24;
-// A launch whose last stages have fewer units (32 values of one slot) than this, one and a half
-// for each of the chip's 152 x 24 warps, runs a unit per key there: a range of 5,000 values, n = 32,
+// A launch whose last stages have fewer units (32 values of one slot) than this for each SM, one and
+// a half for each of its 24 warps, runs a unit per key there: a range of 5,000 values, n = 32,
 // 167 -> 135 us, of 2^8 (n = 8) 40 -> 17 us; 2^16 values in 1.7 units a warp lose 3 %.
-constexpr uint64_t kSplitUnits = 3 * 152 * 24 / 2;
+constexpr uint64_t kSplitUnitsPerSm = 3 * (kStageThreads / 32) / 2;
 
 // distinct l-bit prefixes of n_vals uniform values, the most that a column can be expected to have
 double expected_nodes(double n_vals, int l) {
@@ -999,7 +999,7 @@ bool staged_plan(const std::vector<GroupDesc>& groups, const std::vector<PredDes
     uint64_t last_units = 0;
     for (size_t q = 0; q < preds.size(); q++)
         last_units += 3 * ((max_values(sg->cols[pred_col[q]]) + 31) / 32);
-    sg->split = last_units < kSplitUnits;
+    sg->split = last_units < kSplitUnitsPerSm * (uint64_t)sm_count;
     // predicates in group order, cut into rounds whose states fit limits.round_bytes
     size_t at = col_end, most = col_end;
     StagedRound R{};
