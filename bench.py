@@ -262,33 +262,47 @@ def gpu_index_of(local: int) -> int:
 LDS_PIPE = "shared-memory (LDS/MIO) AES T-table lookups, one 4-byte word per lane per clock per SM"
 
 
-def lookup_roofline(lookups: float, seconds: float, peak_lu: float, aes: float | None = None) -> dict:
+ELEMENT_WALKS = "every element's walks from the root, and the re-share PRF words"
+NODE_WALKS = ("each distinct tree node once per key, and the re-share PRF words; aes_blocks_per_s counts every "
+              "element's walks from the root")
+
+
+def lookup_roofline(lookups: float, seconds: float, peak_lu: float, aes: float | None = None,
+                    counted: str = ELEMENT_WALKS) -> dict:
     """Roofline record of a filter run against the shared-memory T-table lookup ceiling."""
     ach = lookups / seconds / 1e9
     out = {"bound": "lds", "achieved": ach, "peak": peak_lu, "unit": "Glookup/s", "frac": ach / peak_lu,
-           "traffic": None, "pipe": LDS_PIPE,
-           "counted": "every element's walks from the root; a staged evaluation visits the nodes that elements "
-                      "share once and reads above the peak"}
+           "traffic": None, "pipe": LDS_PIPE, "counted": counted}
     if aes is not None:
         out["aes_blocks_per_s"] = aes / seconds
     return out
 
 
-def node_lookups(preds, values, n_bits: int) -> float:
-    """T-table lookups of a filter that visits each distinct tree node once: per node and key 160
-    (DPF) or 160 + 148 (DCF), and the re-share PRF words of every element.  The mask shifts a
-    column's values, which hardly changes how many prefixes they have; it is taken as 0."""
-    total, nodes = 0.0, {}
+def column_nodes(column, n_bits: int) -> int:
+    """Distinct non-root nodes of the tree that a column's values walk: their distinct prefixes of 1 to
+    n_bits bits.  The mask shifts the values, which hardly changes how many prefixes they have;
+    it is taken as 0."""
+    x, c = np.unique(column), 0
+    for _ in range(n_bits):
+        c += len(x)
+        x = x >> 1
+        x = x[np.concatenate([[True], x[1:] != x[:-1]])]
+    return c
+
+
+def node_lookups(preds, tables, n_bits: int, nodes: dict | None = None) -> float:
+    """T-table lookups of a query that visits each distinct tree node once: per node and key 160
+    (DPF) or 160 + 148 (DCF), and the re-share PRF words of every group's elements.  tables: values
+    per table id; nodes keeps the columns' counts from one query to the next."""
+    nodes = {} if nodes is None else nodes
+    total, groups = 0.0, {}
     for p in preds:
-        if p["attr"] not in nodes:
-            x, c = np.unique(values[p["attr"]]), 0
-            for _ in range(n_bits):
-                c += len(x)
-                x = x >> 1
-                x = x[np.concatenate([[True], x[1:] != x[:-1]])]
-            nodes[p["attr"]] = c
-        total += nodes[p["attr"]] * (6 * 160 if p["kind"] == W.PRED_EQ else 12 * 308)
-    return total + values.shape[1] * 148.0 * 3 * (2 * len(preds) - 1)
+        at = (p["table"], p["attr"])
+        if at not in nodes:
+            nodes[at] = column_nodes(tables[at[0]][at[1]], n_bits)
+        total += nodes[at] * (6 * 160 if p["kind"] == W.PRED_EQ else 12 * 308)
+        groups.setdefault(p["group"], []).append(p)
+    return total + sum(tables[g[0]["table"]].shape[1] * 148.0 * 3 * (2 * len(g) - 1) for g in groups.values())
 
 
 def run_ours(args):
@@ -377,27 +391,13 @@ def run_ours(args):
     sm_count = torch.cuda.get_device_properties(dev).multi_processor_count
     max_mhz = float(peaks.get("sm_max_mhz", 2070.0))
     lookups_all = lookups_per_element(preds) * N_VERTICES
-    lookups_step = node_lookups(preds, wl["tables"][0]["values"], 32)
+    lookups_step = node_lookups(preds, {0: wl["tables"][0]["values"]}, 32)
     peak_lu = sm_count * LDS_LANES_PER_CLK * max_mhz * 1e6 / 1e9
-    roofline = lookup_roofline(lookups_step, ms_per_step / 1e3, peak_lu, aes_step)
+    roofline = lookup_roofline(lookups_step, ms_per_step / 1e3, peak_lu, aes_step, NODE_WALKS)
     roofline.update({"kernel": STAGED_KERNELS,
                      "peak_basis": f"{sm_count} SMs x {LDS_LANES_PER_CLK} lookups/clk x "
                                    f"{max_mhz:.0f} MHz (sm_max_mhz of MEASURED_PEAKS.json)",
-                     "counted": "each distinct tree node once per key, and the re-share PRF words; "
-                                "aes_blocks_per_s counts every element's walks from the root",
                      "lookups_per_step": lookups_step, "lookups_per_step_element_walks": lookups_all})
-    rec_traffic = kernel_record("k_filter_traffic.json")
-    if rec_traffic:
-        roofline["traffic"] = rec_traffic.get("bytes_per_launch")
-    rec_issue = kernel_record("k_filter_issue.json")
-    if rec_issue:
-        # every instruction the kernel issues, per AES block (ncu), against the SMs' issue slots
-        # for 32-bit integer work: 128 lanes per clock per SM
-        ipb = float(rec_issue["thread_inst_per_aes_block"])
-        roofline["int32_issue_frac"] = roofline["aes_blocks_per_s"] * ipb / (sm_count * 128 * max_mhz * 1e6)
-        roofline["int32_issue_basis"] = (f"AES blocks/s x {ipb:.1f} thread-instructions per block (ncu, "
-                                         f"{rec_issue['source']}) / ({sm_count} SMs x 128 lanes x {max_mhz:.0f} MHz)")
-
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "u32", "data": "synthetic",
@@ -525,34 +525,6 @@ def run_profile_case(args):
         ctx.sync()
     print(json.dumps({"profile_case": True, "elements": n, "aes_blocks_per_launch": aes_per_element(preds) * n}))
     return 0
-
-
-def kernel_hash() -> str:
-    """Hash of the k_filter source: the device AES/FSS and async-copy headers and the kernel's
-    part of oblivgm.cu (from the PTX helpers to the raw-batch section), so host-code edits
-    elsewhere do not invalidate a capture."""
-    import hashlib
-    h = hashlib.sha256()
-    for hdr in ("device_fss.cuh", "ptx_async.cuh"):
-        with open(os.path.join(ROOT, "paper_2209_03526_gb300", "csrc", hdr), "rb") as fh:
-            h.update(fh.read())
-    with open(os.path.join(ROOT, "paper_2209_03526_gb300", "csrc", "oblivgm.cu"), "rb") as fh:
-        src = fh.read()
-    a = src.index(b"// ------------------------------------------------------------------ PTX helpers")
-    b = src.index(b"// ------------------------------------------------------------------ raw batches")
-    h.update(src[a:b])
-    return h.hexdigest()[:16]
-
-
-def kernel_record(name: str):
-    """An ncu record under profiles/ taken on the current k_filter source, else None."""
-    path = os.path.join(ROOT, "profiles", name)
-    try:
-        with open(path) as f:
-            rec = json.load(f)
-    except (OSError, ValueError):
-        return None
-    return rec if rec.get("kernel_source_hash") == kernel_hash() else None
 
 
 def query_aes(preds, table_n, n_bits=32):
@@ -816,6 +788,10 @@ def filter_workload_record(P, torch, name: str, graph, queries, sched, steps: in
                       "parity_queries_checked": k_check},
            "roofline": lookup_roofline(lookups, step_s, peak_lu, aes),
            "clocks": clocks}
+    if shape["staged"]:
+        vals, nodes = {t: tab["values"] for t, tab in enumerate(graph["tables"])}, {}
+        rec["roofline"] = lookup_roofline(sum(node_lookups(q["preds"], vals, n_bits, nodes) for q in queries), step_s,
+                                          peak_lu, aes, NODE_WALKS)
     rec["roofline"]["kernel"] = STAGED_KERNELS if shape["staged"] else shape["kernel"]
     if plain:
         rec["plain_path"] = plain
@@ -923,7 +899,8 @@ def record_serve(P, torch, args, sched) -> dict:
                                "(50, 200, 1000 q/s)",
                       "launches": "the serving loop's fused batches on two streams (continuous batching); "
                                   "plain path FIFO on the same arrival prefix"},
-           "roofline": lookup_roofline(sat_lookups, sat_s, peak_lu, sat_aes),
+           "roofline": lookup_roofline(sat_lookups, sat_s, peak_lu, sat_aes, ELEMENT_WALKS + "; batches that are "
+                                       "staged visit the nodes that elements share once and read above the peak"),
            "serving": runs, "clocks": clocks}
     if not args.no_cpu_baseline:
         import oracle
@@ -1230,7 +1207,7 @@ def workload_line(args) -> dict:
         line.update({"metric": "secShuffle records/s", "unit": "records/s", "value": n_v / shuf_s,
                      "ms_per_step": shuf_s * 1e3, "steps": args.steps, "warmup": args.warmup,
                      "config": {"l2": "flushed between timed steps", "workload": "shuffle_1048576x6_add", "records": n_v, "words_per_record": width,
-                                "launch": "k_feistel_tab + k_perms + one kernel per server (k_shuf_cs1..3)"},
+                                "launch": "k_feistel_tab + one kernel per server (k_shuf_cs1..3)"},
                      "roofline": {"bound": "lds", "pipe": LDS_PIPE, "achieved": lookups / shuf_s / 1e9, "peak": peak_lu,
                                   "unit": "Glookup/s", "frac": lookups / shuf_s / 1e9 / peak_lu},
                      "fetch_case_ii": {"candidates": n_v, "matches": int(m), "ms_host_clock": float(np.mean(fms)) * 1e3,
