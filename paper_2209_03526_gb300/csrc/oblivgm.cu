@@ -508,7 +508,9 @@ __global__ void __launch_bounds__(WpShape<ELEMS>::kThreads, 1) k_filter_wp(const
                 for (int j = 0; j < 3; j++) xh += __ldg(G.share[j] + row + e);
                 xh &= mask;
             }
-            const DevKey& K = pkeys[slot];
+            // an equality predicate has six keys; the other six slots of a group that also has ranges
+            // must not read past them, which may be the end of the shared memory
+            const DevKey& K = pkeys[slot < 6 * nsub ? slot : 0u];
             uint32_t y = 0;
             // one loop for both kinds: the seed thread walks the seed / control-bit chain (a
             // DPF walk whole); for a DCF the value thread takes each level's value block on

@@ -203,3 +203,33 @@ def test_per_item_evaluation_in_even_waves(ctx, dcf, points):
         assert np.array_equal(got[k][idx], want)
     hit = x < alpha if dcf else x == alpha
     assert np.array_equal(got[0] + got[1], np.where(hit, np.uint32(beta), np.uint32(0)))
+
+
+@pytest.mark.parametrize("bits", [4, 29])
+@pytest.mark.parametrize("groups", [((0, 0, 0, 1, 1, 1, 1, 1),), ((0, 1, 0), (1, 0, 1, 1, 1)), ((0, 0, 0, 0, 1), (1, 1))])
+def test_walk_parallel_keys_up_to_the_end_of_shared_memory(ctx, bits, groups):
+    """66 keys, the most that a launch keeps in shared memory, in groups of both kinds whose last
+    predicate is an equality: its walks' idle slots have no key of their own there."""
+    g, n = W.rng(bits + len(groups)), 207
+    vals = W.uniform_attrs(g, 2, n, bits)
+    tab = W.table(vals, bits, g)
+    ctx.load_shares(0, [to_dev(s) for s in tab["shares"]], bits)
+    top, preds = (1 << bits) - 1, []
+    for grp, kinds in enumerate(groups):
+        for k, eq in enumerate(kinds):
+            op = (W.COMBINE_AND, W.COMBINE_OR, W.COMBINE_XOR)[k % 3] if k else W.COMBINE_AND
+            preds.append(W.eq_pred(0, k % 2, grp, int(vals[k % 2, k]), op) if eq else
+                         W.range_pred(0, k % 2, grp, k, top // 2 + k, op))
+    assert sum(6 if p["kind"] == W.PRED_EQ else 12 for p in preds) == 66
+    toks = P.keygen(preds, bits, bytes(range(5, 21)))
+    prev = ctx.set_walk_parallel((1 << 64) - 1)
+    try:
+        outs = [[torch.zeros(n, dtype=torch.int32, device="cuda") for _ in range(3)] for _ in groups]
+        ctx.filter_and_combine(9, toks, outs)
+        ctx.sync()
+    finally:
+        ctx.set_walk_parallel(prev)
+    for grp in range(len(groups)):
+        got = np.stack([from_dev(t) for t in outs[grp]])
+        want = oracle.filter_group(toks, 9, PRF, [(tab["shares"], bits)], grp, np.arange(n), threads=4)
+        assert np.array_equal(got, want), grp
