@@ -84,8 +84,8 @@ typedef struct {
      * server i holds k_i and k_{i-1}.  F(k, ctr) = bytes 0..3 of AES_k(ctr). */
     uint8_t  prf_keys[3][16];
     /* serving loop: device bytes it may reserve for in-flight queries' outputs
-     * (0 = 25 % of free memory at create time) and in-flight query slots
-     * (0 = 64). */
+     * (0 = 25 % of free memory at create time; a staged batch's scratch, as in
+     * oblivgm_filter_batch, comes on top) and in-flight query slots (0 = 64). */
     uint64_t serve_arena_bytes;
     uint32_t serve_max_inflight;
     uint32_t flags;   /* reserved, must be 0 */

@@ -392,7 +392,7 @@ __host__ __device__ inline int wp_shared_levels(uint32_t elems, int n) {
     return top;
 }
 
-// The seed warp w and the value warp kWalks / 32 + w of a walk pair meet at named barrier
+// The seed warp and the value warp of walks 32 w .. 32 w + 31 meet at named barrier
 // 1 + w (64 threads): the per-level hand-over needs only the two of them, so pairs do not
 // wait for one another and drift apart, which keeps the lookup and logic pipes busy.
 __device__ __forceinline__ void wp_pair_sync(uint32_t walk) {

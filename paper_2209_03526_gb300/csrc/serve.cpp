@@ -3,7 +3,7 @@
 // Queries are admitted by memory (their output share sets must fit in the
 // serve arena) and by slot count.  A worker thread takes admitted queries in
 // arrival order into a batch until the batch holds enough work to fill the GPU
-// (about 3e9 AES blocks) and launches it as one fused kernel on one of two
+// (about 3e9 AES blocks) and launches it, fused or staged, on one of two
 // streams; the next batch goes to the other stream at once and takes over the
 // SMs the running one releases (continuous batching).  A host callback on the
 // batch's stream marks its queries done.
@@ -81,7 +81,7 @@ void worker_main(oblivgm_ctx* ctx) {
         S.running_batches++;
         lk.unlock();
 
-        // allocate outputs in stream order, then one fused launch for the whole batch
+        // allocate outputs in stream order, then one launch, fused or staged, for the whole batch
         std::vector<uint32_t> qids, ngroups;
         std::vector<uint32_t* const*> outs;
         std::vector<ParsedQuery> parsed;

@@ -126,3 +126,21 @@ def test_a_staged_plan_says_so(ctx):
         assert d["staged"] == staged and (d["launches"] > 10) == staged and (d["rounds"] == 1) == staged
         # at least the columns' sorted keys, element numbers and ranks, twice and once, for two columns
         assert d["scratch"] >= 2 * 20 * n if staged else d["scratch"] == 0
+
+
+def test_a_small_call_is_weighed_as_a_call(ctx):
+    """An equality and a range on 3,200 12-bit values each: a staged call would allocate and upload for
+    longer than the walk-parallel kernel runs."""
+    n = 3200
+    wl = {"tables": [W.table(W.uniform_attrs(W.rng(12), 2, n, 12), 12, W.rng(13))]}
+    v = wl["tables"][0]["values"]
+    wl["preds"] = [W.eq_pred(0, 0, 0, int(v[0, 0])), W.range_pred(0, 1, 1, 100, 2000)]
+    load_tables(ctx, wl)
+    toks = P.keygen(wl["preds"], 12, bytes(range(6, 22)))
+    outs = alloc_outs(wl)
+    before = ctx.launch_count()
+    ctx.filter_and_combine(11, toks, outs)
+    ctx.sync()
+    assert ctx.launch_count() - before == 1
+    for grp, got in enumerate(_shares(outs)):
+        assert np.array_equal(got, oracle_group(oracle, wl, toks, 11, grp, np.arange(n))), grp
